@@ -70,7 +70,6 @@ static AngleParams angle_params(double theta, int frame, int nx, int ny, int nb,
     P.f0_k = db / (cc * h);
     P.f0_c = -0.5 * (nb - 1) * db / (cc * h) + 0.5 * (nfast - 1) + 0.5 * (nstep - 1) * (ss / cc);
     P.df = -ss / cc;
-    split12(P.df, P.df_hi, P.df_lo);
     P.wstep_d = h / std::fabs(cc);
     P.wstep = (float)P.wstep_d;
     // t(i, j) = (x_i c + y_j s)/db + (nb-1)/2
@@ -85,11 +84,11 @@ static AngleParams angle_params(double theta, int frame, int nx, int ny, int nb,
     P.rfoot = (float)P.rfoot_d;
     P.wfoot = (float)P.wfoot_d;
     P.inv_rfoot = (float)(1.0 / P.rfoot_d);
-    const double fci = std::floor(P.f0_c);
-    P.f0c_i = (int)std::fmax(std::fmin(fci, 1e9), -1e9);
-    P.f0c_f = (float)(P.f0_c - fci);
-    split12(P.f0_k, P.f0k_hi, P.f0k_lo);
-    P.df_f = (float)P.df;
+    P.wide = !(std::fabs(P.f0_c) < F0_LIMIT && std::fabs(P.f0_c + (nb - 1) * P.f0_k) < F0_LIMIT);
+    P.f0kQ = P.wide ? 0 : std::llround(std::ldexp(P.f0_k, 40));
+    P.f0cQ = P.wide ? 0 : std::llround(std::ldexp(P.f0_c, 40));
+    P.dfQ = std::llround(std::ldexp(P.df, 40));
+    P.wstep_lo = (float)(P.wstep_d - (double)P.wstep);
     return P;
 }
 
@@ -123,10 +122,8 @@ static void fan_ray(double theta, double gamma, double poff, int nx, int ny, dou
     if constexpr (sizeof(real) == 4) {
         (void)jlo;
         (void)jhi;
-        const double fl = std::floor(f0);
-        R.ibr = 2 * (int)std::fmax(std::fmin(fl, 5e8), -5e8) + rows;
-        R.fb = (float)(f0 - fl);
-        split12(df, R.df_hi, R.df_lo);
+        R.f0q = 2 * std::llround(std::ldexp(std::fmin(std::fmax(f0, -F0_LIMIT), F0_LIMIT), 40)) + rows;
+        R.dq = std::llround(std::ldexp(df, 40));
     } else {
         R.rows = rows;
         R.jlo = jlo;

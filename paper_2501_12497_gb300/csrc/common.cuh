@@ -40,11 +40,15 @@ long long launches_so_far();
 #define MOF_LAUNCH_CHECK() MOF_CUDA(cudaGetLastError())
 
 // ------------------------------------------------------- per-angle tables
+// Bound, in pixels, of a march's f0 in fixed point: beyond it (frames hold at most 4096
+// pixels a side and |df| <= 1) a ray cannot reach the frame, so f0 is held there.
+constexpr double F0_LIMIT = 2097152.0;
 // Host-computed (FP64) parameters of one projection angle. The FP32
-// kernels evaluate affine coordinates base + j * step with the step split
-// into a 12-significant-bit head (exact products with |j| < 4096) and a
-// tail, so that the fractional interpolation weight keeps ~1e-7 absolute
-// accuracy at any grid size (see affine_frac below).
+// kernels evaluate affine coordinates base + j * step in fixed point (the
+// march), or with the step split into a
+// 12-significant-bit head (exact products with |j| < 4096) and a tail (the
+// transpose), so that the fractional interpolation weight keeps
+// ~1e-7 absolute accuracy at any grid size.
 struct AngleParams {
     double c, s;        // cos, sin
     // Ray-driven (Joseph) march, in the frame of the stepping axis:
@@ -52,7 +56,6 @@ struct AngleParams {
     double f0_k;        // d f0 / d bin
     double f0_c;        // constant part
     double df;          // step of f per step index
-    float df_hi, df_lo; // split of df
     float wstep;        // h / max(|c|, |s|): path length per step
     int rows;           // 1: step over rows y (|c| >= |s|), fast axis x; 0: transposed
     // Pixel-driven footprint: bin coordinate t(i, j) = t0 + i * tA + j * tB
@@ -63,12 +66,12 @@ struct AngleParams {
     int frame;          // frame this angle belongs to
     int pad_;
     double wstep_d, rfoot_d, wfoot_d;  // the same three in FP64 (FP64 kernels)
-    // FP32 ray set-up without FP64: f0(k) = f0c_i + f0c_f + k (f0k_hi + f0k_lo),
-    // f0k_hi with 12 significant bits (k * f0k_hi exact for k < 4096)
-    int f0c_i;
-    float f0c_f, f0k_hi, f0k_lo;
+    // FP32 march in fixed point, units of 2^-40 pixels: f(j) = f0cQ + k f0kQ + j dfQ; wide: some
+    // ray's f0 lies beyond F0_LIMIT pixels (f0_c and f0_k then give it in FP64)
+    long long f0kQ, f0cQ, dfQ;
+    int wide;
+    float wstep_lo;     // wstep_d - wstep
     float inv_rfoot;    // 1 / rfoot
-    float df_f;         // df rounded to FP32 (step-range bounds only)
 };
 
 // Fan beam (flat detector): one Joseph march per ray (view a, bin k), stored per
@@ -79,9 +82,8 @@ struct AngleParams {
 // march may skip them and the transpose needs no step range.
 template <typename real> struct FanRay;
 template <> struct __align__(16) FanRay<float> {
-    int ibr;             // 2 floor(f0) + rows
-    float fb;            // f0 - floor(f0)
-    float df_hi, df_lo;  // df split, df_hi with 12 significant bits
+    long long f0q;       // 2 f0 + rows, f0 in units of 2^-40 pixels (within F0_LIMIT)
+    long long dq;        // df in units of 2^-40
 };
 template <> struct FanRay<double> {
     double f0, df, wstep;
@@ -171,19 +173,6 @@ __device__ __forceinline__ float warp_maxf(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
-}
-
-// floor and fraction of base + j * (hi + lo), base = ibase + fbase with
-// fbase in [0, 1): j * hi is exact for |j| < 4096, so the fraction carries
-// only the rounding of a sum of O(1) terms.
-__device__ __forceinline__ void affine_frac(int ibase, float fbase, float hi, float lo, int j,
-                                            int &ifl, float &frac) {
-    const float pj = (float)j * hi;  // exact
-    const float pf = floorf(pj);
-    const float r = fbase + (pj - pf) + (float)j * lo;
-    const float rf = floorf(r);
-    ifl = ibase + (int)pf + (int)rf;
-    frac = r - rf;
 }
 
 // Error-free FP32 accumulation of a dot product ("double-float"): hi + lo carries the

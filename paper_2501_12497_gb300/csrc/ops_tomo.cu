@@ -16,7 +16,51 @@
 // cross the pixel's two Joseph segments and re-evaluates the forward entry.
 #include "common.cuh"
 
+#include <algorithm>
+
 namespace mof {
+
+// ------------------------------------------------------------------ helpers
+constexpr float FLOOR_MAGIC = 12582912.0f;      // 1.5 2^23: x + FLOOR_MAGIC rounded down is floor(x) + FLOOR_MAGIC
+constexpr int FLOOR_BITS = 0x4B400000;          // its bit pattern: an integer n adds n to it
+constexpr float INV32 = 2.3283064365386963e-10f;  // 2^-32
+
+// Two FP32 values in a register pair; one instruction for both (the kernels here are bound by
+// instruction issue).
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pack2(float x, float y) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ F2 both(float x) { return pack2(x, x); }
+__device__ __forceinline__ void unpack2(F2 a, float &x, float &y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a.v)); }
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 add2_rd(F2 a, F2 b) {
+    F2 r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+// floor and fraction of both values: the bits of floor + FLOOR_MAGIC in n0, n1
+__device__ __forceinline__ F2 floor2(F2 f, int &n0, int &n1) {
+    const F2 t = add2_rd(f, both(FLOOR_MAGIC));
+    float t0, t1;
+    unpack2(t, t0, t1);
+    n0 = __float_as_int(t0);
+    n1 = __float_as_int(t1);
+    return sub2(f, sub2(t, both(FLOOR_MAGIC)));
+}
 
 // --------------------------------------------------------------- transpose
 // uT[t][x][y] = u[t][y][x], 32x32 tiles through shared memory.
@@ -37,114 +81,54 @@ __global__ void k_transpose(const real *__restrict__ u, real *__restrict__ uT, i
 }
 
 // -------------------------------------------------------------- K1 project
-// One thread per ray (angle a = blockIdx.y, bin k). Rays of one warp are 32
-// adjacent bins of one angle, so at each step they read adjacent pixels of
-// one image row (of the transposed frame for steep angles): coalesced. In FP32
-// the ray sum is compensated (Kahan, per step of two taps): its rounding stays
-// at a few units of FP32 however long the ray.
-template <typename real>
-__global__ void __launch_bounds__(128) k_project(const real *__restrict__ u, const real *__restrict__ uT,
-                                                 real *__restrict__ b, const AngleParams *__restrict__ ang,
-                                                 int nx, int ny, int nb) {
-    const int a = blockIdx.y;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nb) return;
-    const AngleParams &P = ang[a];
-    const long long ns = (long long)nx * ny;
-    const int rows = P.rows;
-    const real *img = rows ? u + P.frame * ns : uT + P.frame * ns;
-    const int nfast = rows ? nx : ny, nstep = rows ? ny : nx;
-    real acc = 0;
-    if constexpr (sizeof(real) == 4) {
-        // f(k, j) = f0(k) + j df, in FP32 with split steps (the base in FP64 when nb >= 4096):
-        // the base f0(k) = f0c_i + f0c_f + k (f0k_hi + f0k_lo) and each step j df are
-        // evaluated as an integer part plus a fraction accurate to ~1e-7
-        int ib;
-        float fb;
-        if (nb < 4096) {
-            affine_frac(P.f0c_i, P.f0c_f, P.f0k_hi, P.f0k_lo, k, ib, fb);
-        } else {  // k * f0k_hi would not be exact: the base in FP64
-            const double f0d = (double)k * P.f0_k + P.f0_c, fl0 = floor(f0d);
-            ib = (int)fmax(fmin(fl0, 1e9), -1e9);
-            fb = (float)(f0d - fl0);
-        }
-        // steps whose crossing can lie in (-1, nfast), with two steps of margin each side
-        // (the taps are bounds-checked, so extra steps add nothing)
-        int jlo = 0, jhi = nstep - 1;
-        const float f0 = (float)ib + fb;
-        if (P.df_f != 0.0f) {
-            const float ja = (-1.0f - f0) / P.df_f, jb = ((float)nfast - f0) / P.df_f;
-            const float lo = fmaxf(fminf(ja, jb), -1.0f), hi = fminf(fmaxf(ja, jb), (float)nstep);
-            jlo = max(0, (int)floorf(lo) - 2);
-            jhi = min(nstep - 1, (int)ceilf(hi) + 2);
-        } else if (!(f0 > -1.0f && f0 < (float)nfast)) {
-            jhi = -1;
-        }
-        float cmp = 0.f;  // Kahan compensation of the ray sum (a ray adds up to 2 nx taps)
-#pragma unroll 4
-        for (int j = jlo; j <= jhi; ++j) {
-            int i0;
-            float w1;
-            affine_frac(ib, fb, P.df_hi, P.df_lo, j, i0, w1);
-            const real *row = img + (long long)j * nfast;
-            float tap = 0.f;
-            if (i0 >= 0 && i0 < nfast) tap = (1.0f - w1) * ldg(row + i0);
-            if (i0 + 1 >= 0 && i0 + 1 < nfast) tap = fmaf(w1, ldg(row + i0 + 1), tap);
-            const float y = __fsub_rn(tap, cmp), t = __fadd_rn(acc, y);
-            cmp = __fsub_rn(__fsub_rn(t, acc), y);
-            acc = t;
-        }
-        b[(long long)a * nb + k] = acc * P.wstep;
-    } else {
-        const double f0 = (double)k * P.f0_k + P.f0_c;  // fractional fast index at step 0
-        int jlo = 0, jhi = nstep - 1;
-        if (P.df != 0.0) {
-            double ja = (-1.0 - f0) / P.df, jb = ((double)nfast - f0) / P.df;
-            double lo = fmin(ja, jb), hi = fmax(ja, jb);
-            lo = fmax(lo, -1.0);
-            hi = fmin(hi, (double)nstep);
-            jlo = max(0, (int)floor(lo) - 1);
-            jhi = min(nstep - 1, (int)ceil(hi) + 1);
-        } else if (!(f0 > -1.0 && f0 < (double)nfast)) {
-            jhi = -1;
-        }
-        for (int j = jlo; j <= jhi; ++j) {
-            const double f = fma((double)j, P.df, f0);
-            const double fl = floor(f);
-            const int i0 = (int)fl;
-            const double w1 = f - fl;
-            const real *row = img + (long long)j * nfast;
-            if (i0 >= 0 && i0 < nfast) acc = fma(1.0 - w1, ldg(row + i0), acc);
-            if (i0 + 1 >= 0 && i0 + 1 < nfast) acc = fma(w1, ldg(row + i0 + 1), acc);
-        }
-        b[(long long)a * nb + k] = acc * (real)P.wstep_d;
-    }
-}
+// FP32: one lane per ray, the 32 rays of a warp at the same step j, so that every load of
+// the warp falls into one row of the frame (of the transposed frame for steep rays).
+// The crossing f(j) = f0 + j df runs in fixed point (2^-40 pixels, 64-bit integers) from block
+// to block of MARCH steps; within a block it is f = fc + (e - MARCH / 2) df in FP32 about the
+// block's middle, fc in [0, 1), so it is exact to 2^-22 pixels. The floor comes from an
+// addition that rounds down to the integers (1.5 2^23): one FMA and three additions a step, no
+// conversion and no integer arithmetic but the address.
+// A block in which every lane's two taps lie inside the row is taken without bounds checks;
+// only the blocks where a ray of the warp enters or leaves the frame test each tap.
+// The sums of the blocks are compensated (Kahan): a ray's rounding stays at a few units of
+// FP32 however long it is.
+// What bounds it: the two 4-byte loads a step, each of which touches two to three 128-byte
+// lines of L1 (32 adjacent rays cross 32 to 46 pixels of a row; 65 % of the L1 data pipe), and
+// instruction issue (63 %, 13 instructions a step). 1024x1024x64, 90 views: 2.99 ms against 7.21
+// for the march with a conversion pair per coordinate and per-ray step ranges, whose lanes read
+// different rows; 256x256x32, 30 views: 62 against 130 us. Fan beam 256x256x32: 68 against 119 us.
+// Few rays leave the chip idle and the march's load latency exposed, so the warps of a CTA
+// share rays of small problems: each takes a segment of the steps (ProjSplit).
+constexpr int MARCH = 8;  // steps per block
+constexpr int PW = 8;     // warps per CTA
+// The warps of a CTA as (32-bin groups) x (adjacent views) x (segments of the steps), all
+// powers of two with product PW. Adjacent views cross the same rows together, so they share
+// L1 lines.
+struct ProjSplit {
+    int views, segs, bins;  // bins in groups of 32
+};
 
-// ---------------------------------------------------------- K1 fan beam
-// One thread per ray (view a = blockIdx.y, bin k); the march of the parallel
-// kernel with the ray's own start and step from the ray table.
-template <typename real>
-__global__ void __launch_bounds__(128) k_project_fan(const real *__restrict__ u, const real *__restrict__ uT,
-                                                     real *__restrict__ b, const FanRay<real> *__restrict__ rays,
-                                                     const AngleParams *__restrict__ ang, int nx, int ny, int nb, real h) {
-    const int a = blockIdx.y;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nb) return;
-    const long long ns = (long long)nx * ny;
-    const FanRay<real> R = rays[(long long)a * nb + k];
-    const int frame = ang[a].frame;
-    real acc = 0, wstep;
-    if constexpr (sizeof(real) == 4) {
-        const int rows = R.ibr & 1, ib = R.ibr >> 1;
-        const float *img = rows ? u + frame * ns : uT + frame * ns;
-        const int nfast = rows ? nx : ny, nstep = rows ? ny : nx;
-        const float df = R.df_hi + R.df_lo;
-        wstep = h * sqrtf(fmaf(df, df, 1.0f));
-        // steps whose crossing can lie in (-1, nfast), two steps of margin each side
-        int jlo = 0, jhi = nstep - 1;
-        const float f0 = (float)ib + R.fb;
-        if (df != 0.0f) {
+// The sum of one ray's taps, as the compensated pair (sum, correction to subtract). img: the
+// frame in the march's orientation; F, D: f0 and df in 2^-40 pixels, |f0| < 2^22 pixels,
+// |df| <= 1; off lanes (on = false) take part in the warp's votes only; segment seg of nseg of
+// the warp's steps. All lanes call.
+__device__ __forceinline__ float2 ray_march(const float *__restrict__ img, int nfast, int nstep, long long F, long long D,
+                                            bool on, int seg, int nseg) {
+    const unsigned lanes = __ballot_sync(0xffffffffu, on);
+    if (!lanes) return make_float2(0.f, 0.f);
+    const int src = __ffs(lanes) - 1;  // off lanes follow a ray that is marched
+    const long long Fs = __shfl_sync(0xffffffffu, F, src), Ds = __shfl_sync(0xffffffffu, D, src);
+    if (!on) {
+        F = Fs;
+        D = Ds;
+    }
+    // steps whose crossing can lie in (-1, nfast), with two steps of margin each side (the
+    // checked taps beyond add nothing), over the warp's rays
+    int jlo = 0, jhi = nstep - 1;
+    {
+        const float f0 = (float)(int)(F >> 40) + (float)(unsigned)((unsigned long long)F >> 8) * INV32;
+        const float df = (float)D * 9.094947017729282e-13f;
+        if (D != 0) {
             const float ja = (-1.0f - f0) / df, jb = ((float)nfast - f0) / df;
             const float lo = fmaxf(fminf(ja, jb), -1.0f), hi = fminf(fmaxf(ja, jb), (float)nstep);
             jlo = max(0, (int)floorf(lo) - 2);
@@ -152,29 +136,238 @@ __global__ void __launch_bounds__(128) k_project_fan(const real *__restrict__ u,
         } else if (!(f0 > -1.0f && f0 < (float)nfast)) {
             jhi = -1;
         }
-#pragma unroll 4
-        for (int j = jlo; j <= jhi; ++j) {
-            int i0;
-            float w1;
-            affine_frac(ib, R.fb, R.df_hi, R.df_lo, j, i0, w1);
-            const float *row = img + (long long)j * nfast;
-            if (i0 >= 0 && i0 < nfast) acc = fmaf(1.0f - w1, ldg(row + i0), acc);
-            if (i0 + 1 >= 0 && i0 + 1 < nfast) acc = fmaf(w1, ldg(row + i0 + 1), acc);
-        }
-    } else {
-        const double *img = R.rows ? u + frame * ns : uT + frame * ns;
-        const int nfast = R.rows ? nx : ny;
-        wstep = R.wstep;
-        for (int j = R.jlo; j <= R.jhi; ++j) {
-            const double f = fma((double)j, R.df, R.f0), fl = floor(f);
-            const int i0 = (int)fl;
-            const double w1 = f - fl;
-            const double *row = img + (long long)j * nfast;
-            if (i0 >= 0 && i0 < nfast) acc = fma(1.0 - w1, ldg(row + i0), acc);
-            if (i0 + 1 >= 0 && i0 + 1 < nfast) acc = fma(w1, ldg(row + i0 + 1), acc);
-        }
     }
-    b[(long long)a * nb + k] = acc * wstep;
+    jlo = __reduce_min_sync(0xffffffffu, jlo);
+    jhi = __reduce_max_sync(0xffffffffu, jhi);
+    if (nseg > 1) {  // whole blocks
+        const int nblk = (jhi - jlo + MARCH) / MARCH;
+        const int b0 = seg * nblk / nseg, b1 = (seg + 1) * nblk / nseg;
+        jhi = min(jhi, jlo + b1 * MARCH - 1);
+        jlo += b0 * MARCH;
+    }
+    float acc = 0.f, cmp = 0.f;
+    const unsigned last = (unsigned)(nfast - 1);
+    const float df = (float)D * 9.094947017729282e-13f;
+    F += (jlo + MARCH / 2) * D;  // the crossing at the middle of the block
+    const F2 df2 = both(df), one = both(1.0f);
+    for (int j = jlo; j <= jhi; j += MARCH) {
+        const int ic = (int)(F >> 40);
+        const float fc = (float)(unsigned)((unsigned long long)F >> 8) * INV32;
+        const F2 fc2 = both(fc);
+        int n[MARCH];
+        F2 w[MARCH / 2];
+#pragma unroll
+        for (int e = 0; e < MARCH; e += 2)
+            w[e / 2] = floor2(fma2(pack2((float)(e - MARCH / 2), (float)(e + 1 - MARCH / 2)), df2, fc2), n[e], n[e + 1]);
+        const int c0 = ic - FLOOR_BITS;
+        const bool inside = j + MARCH <= nstep && (unsigned)(n[0] + c0) < last && (unsigned)(n[MARCH - 1] + c0) < last;
+        float a[MARCH], c[MARCH];
+        if (__all_sync(0xffffffffu, inside)) {
+            const unsigned long long base = (unsigned long long)(uintptr_t)(img + (j * nfast + ic)) - 4ull * (unsigned)FLOOR_BITS;
+#pragma unroll
+            for (int e = 0; e < MARCH; ++e) {
+                const float *t = reinterpret_cast<const float *>((uintptr_t)(base + 4ull * ((unsigned)n[e] + (unsigned)(e * nfast))));
+                a[e] = ldg(t);
+                c[e] = ldg(t + 1);
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < MARCH; ++e) {
+                const int i0 = n[e] + c0;
+                const float *t = img + ((j + e) * nfast + i0);
+                const bool row = j + e <= jhi;
+                a[e] = (row && (unsigned)i0 <= last) ? ldg(t) : 0.f;
+                c[e] = (row && (unsigned)(i0 + 1) <= last) ? ldg(t + 1) : 0.f;
+            }
+        }
+        F2 s2 = both(0.f);
+#pragma unroll
+        for (int e = 0; e < MARCH; e += 2)
+            s2 = fma2(w[e / 2], pack2(c[e], c[e + 1]), fma2(sub2(one, w[e / 2]), pack2(a[e], a[e + 1]), s2));
+        float s, so;
+        unpack2(s2, s, so);
+        s += so;
+        F += MARCH * D;
+        const float y = __fsub_rn(s, cmp), t = __fadd_rn(acc, y);
+        cmp = __fsub_rn(__fsub_rn(t, acc), y);
+        acc = t;
+    }
+    return make_float2(acc, cmp);
+}
+
+// The segments' sums of the CTA's rays, added in segment order by the first segment's warps
+// (true there; the others are done). All threads call.
+__device__ __forceinline__ bool join_segments(float2 &r, const ProjSplit &sp) {
+    __shared__ float2 part[32 * PW];
+    if (sp.segs == 1) return true;
+    part[threadIdx.x] = r;
+    __syncthreads();
+    const int w = threadIdx.x >> 5, per = PW / sp.segs;
+    if (w >= per) return false;
+    for (int g = 1; g < sp.segs; ++g) {
+        const float2 o = part[threadIdx.x + g * per * 32];
+        const float y = __fsub_rn(o.x, __fadd_rn(r.y, o.y)), t = __fadd_rn(r.x, y);
+        r.y = __fsub_rn(__fsub_rn(t, r.x), y);
+        r.x = t;
+    }
+    return true;
+}
+
+// (sum - correction) * w with w = wh + wl, rounded once
+__device__ __forceinline__ float scale_sum(float2 a, float wh, float wl) {
+    const float p = __fmul_rn(a.x, wh);
+    const float e = fmaf(-a.y, wh, fmaf(a.x, wl, __fmaf_rn(a.x, wh, -p)));
+    return isfinite(p) ? p + e : p;
+}
+
+__global__ void __launch_bounds__(32 * PW) k_project32(const float *__restrict__ u, const float *__restrict__ uT,
+                                                       float *__restrict__ b, const AngleParams *__restrict__ ang, int nang,
+                                                       int nx, int ny, int nb, ProjSplit sp) {
+    const int w = threadIdx.x >> 5, per = PW / sp.segs, seg = w / per, wr = w - seg * per;
+    const int a = blockIdx.y * sp.views + wr % sp.views;
+    const int k = (blockIdx.x * sp.bins + wr / sp.views) * 32 + (threadIdx.x & 31);
+    const AngleParams &P = ang[min(a, nang - 1)];
+    const int kk = min(k, nb - 1);
+    long long F;
+    if (!P.wide) {
+        F = P.f0cQ + kk * P.f0kQ;
+    } else {  // rays so far apart that 2^-40 pixels do not fit: the ray's own f0, held off the frame
+        const double f0 = fmin(fmax((double)kk * P.f0_k + P.f0_c, -F0_LIMIT), F0_LIMIT);
+        F = __double2ll_rn(f0 * 1099511627776.0);
+    }
+    const long long ns = (long long)nx * ny;
+    const int rows = P.rows;
+    const bool on = a < nang && k < nb;
+    float2 r = ray_march((rows ? u : uT) + P.frame * ns, rows ? nx : ny, rows ? ny : nx, F, P.dfQ, on, seg, sp.segs);
+    if (join_segments(r, sp) && on) b[(long long)a * nb + k] = scale_sum(r, P.wstep, P.wstep_lo);
+}
+
+// FP64: one thread per ray (angle a = blockIdx.y, bin k).
+__global__ void __launch_bounds__(128) k_project64(const double *__restrict__ u, const double *__restrict__ uT,
+                                                   double *__restrict__ b, const AngleParams *__restrict__ ang, int nx,
+                                                   int ny, int nb) {
+    const int a = blockIdx.y;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= nb) return;
+    const AngleParams &P = ang[a];
+    const long long ns = (long long)nx * ny;
+    const int rows = P.rows;
+    const double *img = rows ? u + P.frame * ns : uT + P.frame * ns;
+    const int nfast = rows ? nx : ny, nstep = rows ? ny : nx;
+    double acc = 0;
+    const double f0 = (double)k * P.f0_k + P.f0_c;  // fractional fast index at step 0
+    int jlo = 0, jhi = nstep - 1;
+    if (P.df != 0.0) {
+        double ja = (-1.0 - f0) / P.df, jb = ((double)nfast - f0) / P.df;
+        double lo = fmin(ja, jb), hi = fmax(ja, jb);
+        lo = fmax(lo, -1.0);
+        hi = fmin(hi, (double)nstep);
+        jlo = max(0, (int)floor(lo) - 1);
+        jhi = min(nstep - 1, (int)ceil(hi) + 1);
+    } else if (!(f0 > -1.0 && f0 < (double)nfast)) {
+        jhi = -1;
+    }
+    for (int j = jlo; j <= jhi; ++j) {
+        const double f = fma((double)j, P.df, f0);
+        const double fl = floor(f);
+        const int i0 = (int)fl;
+        const double w1 = f - fl;
+        const double *row = img + (long long)j * nfast;
+        if (i0 >= 0 && i0 < nfast) acc = fma(1.0 - w1, ldg(row + i0), acc);
+        if (i0 + 1 >= 0 && i0 + 1 < nfast) acc = fma(w1, ldg(row + i0 + 1), acc);
+    }
+    b[(long long)a * nb + k] = acc * P.wstep_d;
+}
+
+// ---------------------------------------------------------- K1 fan beam
+// FP32: the march of the parallel kernel with each ray's own start and step from the ray
+// table; the rays of a warp that step over rows, then those that step over columns (both
+// only where a fan straddles 45 degrees).
+__global__ void __launch_bounds__(32 * PW) k_project_fan32(const float *__restrict__ u, const float *__restrict__ uT,
+                                                           float *__restrict__ b, const FanRay<float> *__restrict__ rays,
+                                                           const AngleParams *__restrict__ ang, int nang, int nx, int ny,
+                                                           int nb, float h, ProjSplit sp) {
+    const int w = threadIdx.x >> 5, per = PW / sp.segs, seg = w / per, wr = w - seg * per;
+    const int a = blockIdx.y * sp.views + wr % sp.views, ac = min(a, nang - 1);
+    const int k = (blockIdx.x * sp.bins + wr / sp.views) * 32 + (threadIdx.x & 31);
+    const bool on = a < nang && k < nb;
+    const long long ns = (long long)nx * ny;
+    const FanRay<float> R = rays[(long long)ac * nb + min(k, nb - 1)];
+    const int rows = (int)(R.f0q & 1);
+    const long long F = R.f0q >> 1, D = R.dq, fr = ang[ac].frame * ns;
+    float2 r = ray_march(u + fr, nx, ny, F, D, on && rows, seg, sp.segs);
+    const float2 rc = ray_march(uT + fr, ny, nx, F, D, on && !rows, seg, sp.segs);
+    if (!rows) r = rc;
+    if (!join_segments(r, sp) || !on) return;
+    // length per step h sqrt(1 + df^2), its rounding kept: r = sqrt(x) + e, e = (x - s^2) / (2 s)
+    const float df = (float)D * 9.094947017729282e-13f, dl = (float)(D - __float2ll_rn(df * 1099511627776.0f)) * 9.094947017729282e-13f;
+    const float d2 = __fmul_rn(df, df), x = 1.0f + d2;
+    const float xl = fmaf(2.0f * df, dl, fmaf(df, df, -d2)) + (d2 - (x - 1.0f));
+    const float s = sqrtf(x), sl = (fmaf(-s, s, x) + xl) / (2.0f * s);
+    const float wh = h * s, wl = fmaf(h, s, -wh) + h * sl;
+    b[(long long)a * nb + k] = scale_sum(r, wh, wl);
+}
+
+__global__ void __launch_bounds__(128) k_project_fan64(const double *__restrict__ u, const double *__restrict__ uT,
+                                                       double *__restrict__ b, const FanRay<double> *__restrict__ rays,
+                                                       const AngleParams *__restrict__ ang, int nx, int ny, int nb) {
+    const int a = blockIdx.y;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= nb) return;
+    const long long ns = (long long)nx * ny;
+    const FanRay<double> R = rays[(long long)a * nb + k];
+    const int frame = ang[a].frame;
+    double acc = 0;
+    const double *img = R.rows ? u + frame * ns : uT + frame * ns;
+    const int nfast = R.rows ? nx : ny;
+    for (int j = R.jlo; j <= R.jhi; ++j) {
+        const double f = fma((double)j, R.df, R.f0), fl = floor(f);
+        const int i0 = (int)fl;
+        const double w1 = f - fl;
+        const double *row = img + (long long)j * nfast;
+        if (i0 >= 0 && i0 < nfast) acc = fma(1.0 - w1, ldg(row + i0), acc);
+        if (i0 + 1 >= 0 && i0 + 1 < nfast) acc = fma(w1, ldg(row + i0 + 1), acc);
+    }
+    b[(long long)a * nb + k] = acc * R.wstep;
+}
+
+// Segments per ray: doubled while the launch has fewer warps than two rounds of full SMs
+// (152 x 64) and a segment keeps four blocks of steps; the other warps of a CTA take up to four
+// adjacent views. Measured: 256x256x32 (30 views) 97 us with one segment, 87 with this rule, 89
+// with twice the warps; 181x149x9 (23 views) 44 and 26 us; 1024x1024x64 is above the line. One
+// view per CTA: 1024x1024x64 3.94 against 3.79 ms for four and 3.81 for eight (all with the
+// march before its packed form).
+constexpr long long PROJ_WARPS = 2LL * 152 * 64;
+constexpr int PROJ_VIEWS = 4;
+static ProjSplit proj_split(const mof_problem *p, int nang) {
+    const long long warps = (long long)nang * ((p->nb + 31) / 32);
+    const int blocks = std::max(p->nx, p->ny) / MARCH;
+    ProjSplit sp{1, 1, 1};
+    while (sp.segs < PW && warps * sp.segs < PROJ_WARPS && blocks >= 8 * sp.segs) sp.segs *= 2;
+    sp.views = std::min(PW / sp.segs, PROJ_VIEWS);
+    sp.bins = PW / (sp.segs * sp.views);
+    return sp;
+}
+
+// the rays of `nang` views from a0 on; b from the first of them on
+static void project_views(const mof_problem *p, const float *u, const float *uT, float *b, int a0, int nang, cudaStream_t st) {
+    const ProjSplit sp = proj_split(p, nang);
+    const dim3 grid((p->nb + 32 * sp.bins - 1) / (32 * sp.bins), (nang + sp.views - 1) / sp.views);
+    if (p->fan)
+        ::mof::count_launch(), k_project_fan32<<<grid, 32 * PW, 0, st>>>(
+            u, uT, b, static_cast<const FanRay<float> *>(p->d_fanray) + (long long)a0 * p->nb, p->d_ang + a0, nang, p->nx,
+            p->ny, p->nb, (float)p->h, sp);
+    else
+        ::mof::count_launch(), k_project32<<<grid, 32 * PW, 0, st>>>(u, uT, b, p->d_ang + a0, nang, p->nx, p->ny, p->nb, sp);
+}
+static void project_views(const mof_problem *p, const double *u, const double *uT, double *b, int a0, int nang, cudaStream_t st) {
+    const dim3 grid((p->nb + 127) / 128, nang);
+    if (p->fan)
+        ::mof::count_launch(), k_project_fan64<<<grid, 128, 0, st>>>(
+            u, uT, b, static_cast<const FanRay<double> *>(p->d_fanray) + (long long)a0 * p->nb, p->d_ang + a0, p->nx, p->ny,
+            p->nb);
+    else
+        ::mof::count_launch(), k_project64<<<grid, 128, 0, st>>>(u, uT, b, p->d_ang + a0, p->nx, p->ny, p->nb);
 }
 
 template <typename real>
@@ -185,24 +378,13 @@ mof_status launch_project(const mof_problem *p, const real *u, real *uT, real *b
         for (int t = 0; t < p->nt; ++t) {
             dim3 tg1((p->nx + 31) / 32, (p->ny + 31) / 32, 1);
             ::mof::count_launch(), k_transpose<real><<<tg1, tb, 0, st>>>(u + t * ns, uT + t * ns, p->nx, p->ny);
-            const int a0 = p->aoff[t], na = p->aoff[t + 1] - a0;
-            ::mof::count_launch(), k_project<real><<<dim3((p->nb + 127) / 128, na), 128, 0, st>>>(u, uT, b + (long long)a0 * p->nb,
-                                                                                             p->d_ang + a0, p->nx, p->ny, p->nb);
+            project_views(p, u, uT, b + (long long)p->aoff[t] * p->nb, p->aoff[t], p->aoff[t + 1] - p->aoff[t], st);
         }
         MOF_LAUNCH_CHECK();
         return MOF_OK;
     }
     ::mof::count_launch(), k_transpose<real><<<tg, tb, 0, st>>>(u, uT, p->nx, p->ny);
-    MOF_LAUNCH_CHECK();
-    if (p->fan) {
-        dim3 grid((p->nb + 127) / 128, p->A);
-        ::mof::count_launch(), k_project_fan<real><<<grid, 128, 0, st>>>(u, uT, b, static_cast<const FanRay<real> *>(p->d_fanray),
-                                                                        p->d_ang, p->nx, p->ny, p->nb, (real)p->h);
-        MOF_LAUNCH_CHECK();
-        return MOF_OK;
-    }
-    dim3 grid((p->nb + 127) / 128, p->A);
-    ::mof::count_launch(), k_project<real><<<grid, 128, 0, st>>>(u, uT, b, p->d_ang, p->nx, p->ny, p->nb);
+    project_views(p, u, uT, b, 0, p->A, st);
     MOF_LAUNCH_CHECK();
     return MOF_OK;
 }
@@ -423,11 +605,13 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject_fan(const real *__
             int i0, fast;
             real w1, wstep;
             if constexpr (sizeof(real) == 4) {
-                const int rows = R.ibr & 1;
+                const int rows = (int)(R.f0q & 1);
                 const int j = rows ? y : x;
                 fast = rows ? x : y;
-                affine_frac(R.ibr >> 1, R.fb, R.df_hi, R.df_lo, j, i0, w1);
-                const float df = R.df_hi + R.df_lo;
+                const long long f = (R.f0q >> 1) + j * R.dq;
+                i0 = (int)(f >> 40);
+                w1 = (float)(unsigned)((unsigned long long)f >> 8) * 2.3283064365386963e-10f;
+                const float df = (float)R.dq * 9.094947017729282e-13f;
                 wstep = h * sqrtf(fmaf(df, df, 1.0f));
             } else {
                 const int j = R.rows ? y : x;
