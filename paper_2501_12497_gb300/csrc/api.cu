@@ -227,6 +227,23 @@ mof_status mof_problem_create(const mof_geometry *g, int precision, mof_problem 
     for (int t = 0; t < g->nt; ++t)
         for (int a = p->aoff[t]; a < p->aoff[t + 1]; ++a)
             tab[a] = angle_params(g->angles[a], t, g->nx, g->ny, g->nb, g->pixel_size, g->bin_size);
+    // The tiled FP32 transpose needs every footprint within two bins each side (then a 32 x 32
+    // tile's bin coordinates span at most 62 bins per bin of reach, less where they are narrow: the
+    // segments it stages hold 64 words per bin of reach, a few of them margins) and
+    // bin numbers that fit its fixed point.
+    double reach = 0.0, span = 0.0;
+    for (const AngleParams &P : tab) {
+        reach = std::fmax(reach, P.rfoot_d);
+        span = std::fmax(span, 31.0 * (std::fabs(P.tA) + std::fabs(P.tB)));
+    }
+    if (g->nb <= (1 << 20) && reach <= 1.0 && span <= 58.0) p->bp_reach = 1;
+    else if (g->nb <= (1 << 20) && reach <= 2.0 && span <= 120.0) p->bp_reach = 2;
+    if (p->bp_reach)
+        for (AngleParams &P : tab) {
+            P.t0Q = std::llround(std::ldexp(P.t0, 40));
+            P.tAQ = std::llround(std::ldexp(P.tA, 40));
+            P.tBQ = std::llround(std::ldexp(P.tB, 40));
+        }
     cudaError_t e = cudaGetDevice(&p->device);
     if (e == cudaSuccess) e = cudaMalloc(&p->d_ang, sizeof(AngleParams) * A);
     if (e == cudaSuccess) e = cudaMalloc(&p->d_aoff, sizeof(int) * (g->nt + 1));

@@ -45,9 +45,9 @@ long long launches_so_far();
 constexpr double F0_LIMIT = 2097152.0;
 // Host-computed (FP64) parameters of one projection angle. The FP32
 // kernels evaluate affine coordinates base + j * step in fixed point (the
-// march), or with the step split into a
+// march, the tiled transpose), or with the step split into a
 // 12-significant-bit head (exact products with |j| < 4096) and a tail (the
-// transpose), so that the fractional interpolation weight keeps
+// general transpose), so that the fractional interpolation weight keeps
 // ~1e-7 absolute accuracy at any grid size.
 struct AngleParams {
     double c, s;        // cos, sin
@@ -71,6 +71,7 @@ struct AngleParams {
     long long f0kQ, f0cQ, dfQ;
     int wide;
     float wstep_lo;     // wstep_d - wstep
+    long long t0Q, tAQ, tBQ;  // t0, tA, tB in units of 2^-40 bins (set where mof_problem::bp_reach > 0)
     float inv_rfoot;    // 1 / rfoot
 };
 
@@ -114,6 +115,7 @@ struct mof_problem {
     int timing = 0;
     void *timer = nullptr;              // kernel-class timer (solver.cu)
     int warp_mode = 0;                  // M(s): 0 bilinear, 1 rounding and clipping (Sec. 3)
+    int bp_reach = 0;                   // parallel FP32 transpose: footprints within this many bins each side (1, 2), 0: any
     int fan = 0;                        // 1: fan beam with a flat detector
     double rs = 0, rd = 0;              // source and detector distances from the centre
     float fan_scale = 0;                // (rs + rd) / db

@@ -42,6 +42,16 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
     return r;
 }
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
 __device__ __forceinline__ F2 add2_rd(F2 a, F2 b) {
     F2 r;
     asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
@@ -390,22 +400,13 @@ mof_status launch_project(const mof_problem *p, const real *u, real *uT, real *b
 }
 
 // ---------------------------------------------------------- K2 backproject
-// One thread per pixel (tile 32 x 8 per block), looping over the angles of
-// its frame. Per angle the block's base bin coordinate at the tile origin is
-// computed once in FP64 (shared memory); each pixel adds its small in-tile
-// offset with the split-step evaluation, keeping the footprint weight
-// accurate to ~1e-7 at any grid size.
+// FP64: one thread per pixel (tile 32 x 8 per block), looping over the angles of its frame. Per
+// angle the bin coordinate at the tile origin is computed once (shared memory).
 constexpr int BP_TX = 32, BP_TY = 8, BP_CHUNK = 64;
 
-template <typename real>
-__global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject(const real *__restrict__ b, real *__restrict__ u,
-                                                              const AngleParams *__restrict__ ang,
-                                                              const int *__restrict__ aoff, int nx, int ny, int nb, int t0) {
-    // per angle of the chunk: the bin coordinate at the tile origin (integer + fraction,
-    // from FP64) and the constants of the footprint, shared by the block's pixels
-    __shared__ int s_ib[BP_CHUNK];
-    __shared__ float s_fb[BP_CHUNK], s_tAh[BP_CHUNK], s_tAl[BP_CHUNK], s_tBh[BP_CHUNK], s_tBl[BP_CHUNK];
-    __shared__ float s_r[BP_CHUNK], s_ir[BP_CHUNK], s_wf[BP_CHUNK];
+__global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject64(const double *__restrict__ b, double *__restrict__ u,
+                                                                const AngleParams *__restrict__ ang,
+                                                                const int *__restrict__ aoff, int nx, int ny, int nb, int t0) {
     __shared__ double s_tb[BP_CHUNK];
     const int t = t0 + blockIdx.z;
     const int x0 = blockIdx.x * BP_TX, y0 = blockIdx.y * BP_TY;
@@ -413,64 +414,29 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject(const real *__rest
     const int x = x0 + di, y = y0 + dj;
     const int tid = threadIdx.y * BP_TX + threadIdx.x;
     const int a_begin = aoff[t], a_end = aoff[t + 1];
-    real acc = 0;
+    double acc = 0;
     for (int ac = a_begin; ac < a_end; ac += BP_CHUNK) {
         const int cn = min(BP_CHUNK, a_end - ac);
         __syncthreads();
         if (tid < cn) {
             const AngleParams &P = ang[ac + tid];
-            const double tb = P.t0 + (double)x0 * P.tA + (double)y0 * P.tB;
-            const double fl = floor(tb);
-            s_ib[tid] = (int)fmax(fmin(fl, 1e9), -1e9);
-            s_fb[tid] = (float)(tb - fl);
-            s_tb[tid] = tb;
-            s_tAh[tid] = P.tA_hi;
-            s_tAl[tid] = P.tA_lo;
-            s_tBh[tid] = P.tB_hi;
-            s_tBl[tid] = P.tB_lo;
-            s_r[tid] = P.rfoot;
-            s_ir[tid] = P.inv_rfoot;
-            s_wf[tid] = P.wfoot;
+            s_tb[tid] = P.t0 + (double)x0 * P.tA + (double)y0 * P.tB;
         }
         __syncthreads();
         if (x < nx && y < ny) {
             for (int q = 0; q < cn; ++q) {
-                const real *row = b + (long long)(ac + q) * nb;
-                if constexpr (sizeof(real) == 4) {
-                    // bin coordinate t = ib + fr of this pixel (split-step, exact products)
-                    const float pa = (float)di * s_tAh[q], pb = (float)dj * s_tBh[q];
-                    const float pfa = floorf(pa), pfb = floorf(pb);
-                    float fr = s_fb[q] + (pa - pfa) + (pb - pfb) + fmaf((float)di, s_tAl[q], (float)dj * s_tBl[q]);
-                    const float ff = floorf(fr);
-                    const int ib = s_ib[q] + (int)pfa + (int)pfb + (int)ff;
-                    fr -= ff;
-                    const float r = s_r[q], ir = s_ir[q], wf = s_wf[q];
-                    if (r <= 1.0f) {  // at most the two bins around t
-                        const float d1 = 1.0f - fr;
-                        if (fr < r && ib >= 0 && ib < nb) acc = fmaf(wf * (1.0f - fr * ir), ldg(row + ib), acc);
-                        if (d1 < r && ib + 1 >= 0 && ib + 1 < nb) acc = fmaf(wf * (1.0f - d1 * ir), ldg(row + ib + 1), acc);
-                    } else {
-                        // bins k with |k - t| < r: k = ib - m (distance fr + m) and ib + 1 + m (1 - fr + m)
-                        for (int m = 0; (float)m < r; ++m) {
-                            const float d0 = fr + (float)m, d1 = 1.0f - fr + (float)m;
-                            const int k0 = ib - m, k1 = ib + 1 + m;
-                            if (d0 < r && k0 >= 0 && k0 < nb) acc = fmaf(wf * (1.0f - d0 * ir), ldg(row + k0), acc);
-                            if (d1 < r && k1 >= 0 && k1 < nb) acc = fmaf(wf * (1.0f - d1 * ir), ldg(row + k1), acc);
-                        }
-                    }
-                } else {
-                    const AngleParams &P = ang[ac + q];
-                    const double tt = s_tb[q] + (double)di * P.tA + (double)dj * P.tB;
-                    const double ff = floor(tt);
-                    const int ib = (int)ff;
-                    const double fr = tt - ff;
-                    const double rd = P.rfoot_d, wf = P.wfoot_d;
-                    for (int m = 0; (double)m < rd; ++m) {
-                        const double d0 = fr + m, d1 = 1.0 - fr + m;
-                        const int k0 = ib - m, k1 = ib + 1 + m;
-                        if (d0 < rd && k0 >= 0 && k0 < nb) acc = fma(wf * (1.0 - d0 / rd), ldg(row + k0), acc);
-                        if (d1 < rd && k1 >= 0 && k1 < nb) acc = fma(wf * (1.0 - d1 / rd), ldg(row + k1), acc);
-                    }
+                const double *row = b + (long long)(ac + q) * nb;
+                const AngleParams &P = ang[ac + q];
+                const double tt = s_tb[q] + (double)di * P.tA + (double)dj * P.tB;
+                const double ff = floor(tt);
+                const int ib = (int)ff;
+                const double fr = tt - ff;
+                const double rd = P.rfoot_d, wf = P.wfoot_d;
+                for (int m = 0; (double)m < rd; ++m) {
+                    const double d0 = fr + m, d1 = 1.0 - fr + m;
+                    const int k0 = ib - m, k1 = ib + 1 + m;
+                    if (d0 < rd && k0 >= 0 && k0 < nb) acc = fma(wf * (1.0 - d0 / rd), ldg(row + k0), acc);
+                    if (d1 < rd && k1 >= 0 && k1 < nb) acc = fma(wf * (1.0 - d1 / rd), ldg(row + k1), acc);
                 }
             }
         }
@@ -478,12 +444,152 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject(const real *__rest
     if (x < nx && y < ny) u[(long long)t * nx * ny + (long long)y * nx + x] = acc;
 }
 
-// FP32 form with BP_PX pixels per thread (x = x0 + di + 32 e, e < BP_PX: a 128 x 8 tile
-// per CTA): the per-angle constants come from shared memory as two 16-byte records
-// and are reused for the thread's pixels, and the tile origin's FP64 set-up is shared
-// by four times as many pixels. Each pixel's bin coordinate and weights are those of
-// k_backproject (the same split products); a pixel's sum over the angles is compensated
-// (Kahan), so its rounding does not grow with the number of angles.
+// FP32, footprints of at most 2 RT bins (mu h <= RT db for every view; RT = 1 for a detector
+// no finer than the pixels, RT = 2 for one up to twice as fine). A CTA owns a tile of
+// 32 x 32 pixels of a frame; per view it stages the bins that the tile's pixels can reach,
+// times the footprint height (zero beyond the detector), in shared memory, so that the pixels
+// need no bounds checks and adjacent lanes read adjacent words. A thread owns a column of
+// eight pixels; the bin coordinate at the column's middle comes from 64-bit fixed point, the
+// pixels' from one FMA each about it (exact to 2^-22 bins), the floor by the addition of
+// ray_march. The tent weights sat(1 - (fr + m) / r) and sat(1 - (1 + m - fr) / r) are saturating
+// FMAs: they vanish by themselves outside the footprint. The sum over the views is compensated
+// (Kahan).
+// A segment with a non-finite value takes the weights that are zero out of the sum (careful),
+// so that the value reaches exactly the pixels whose footprint holds it.
+// What bounds it: instruction issue (about 74 %, 17 instructions a pixel and view), with the
+// FP32 pipe, which a packed pair occupies twice, and the shared loads close behind. 1024x1024x64,
+// 90 views: 3.29 ms against 9.48 for one thread per four pixels of a row with global loads and
+// three floors a coordinate; 256x256x32, 30 views: 46 against 130 us. Two columns per thread
+// (64 x 32 tiles): 3.31 ms, no gain. Kahan steps every 2 and 4 views: 10 and 15 % faster, but
+// 3 and 7 % further from the exact sum.
+constexpr int BT_X = 32, BT_Y = 4, BT_E = 8;  // threads, pixels per thread down a column
+constexpr int BT_CH = 32;                     // views staged at a time (one lane each sets them up)
+struct __align__(16) BtAngle {
+    long long t;    // bin coordinate of the tile's first pixel in the segment, units of 2^-FB
+    int a, b;       // its steps in x and y, units of 2^-FB
+    float df;       // step in y
+    float ir, c1;   // 1 / r, 1 - 1 / r
+    unsigned seg;   // shared address of the segment
+};
+
+__device__ __forceinline__ float lds(unsigned addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+template <int RT, bool CAREFUL>
+__device__ __forceinline__ void bt_view(const BtAngle &A, F2 (&acc)[BT_E / 2], F2 (&cmp)[BT_E / 2]) {
+    constexpr int FB = 31 - RT;
+    const float ir = A.ir, c1 = A.c1;
+    const F2 df2 = both(A.df);
+    const long long P = A.t + (long long)(int)threadIdx.x * A.a + (long long)(int)(threadIdx.y * BT_E + BT_E / 2) * A.b;
+    const F2 fc2 = both((float)((unsigned)P & ((1u << FB) - 1u)) * (1.0f / (float)(1u << FB)));
+    const unsigned base = A.seg + 4u * ((unsigned)(int)(P >> FB) - (unsigned)FLOOR_BITS);
+#pragma unroll
+    for (int e = 0; e < BT_E; e += 2) {
+        int n0, n1;
+        const F2 fr2 = floor2(fma2(pack2((float)(e - BT_E / 2), (float)(e + 1 - BT_E / 2)), df2, fc2), n0, n1);
+        float f0, f1;
+        unpack2(fr2, f0, f1);
+        const unsigned at0 = base + 4u * (unsigned)n0, at1 = base + 4u * (unsigned)n1;
+        F2 tap = both(0.f);
+#pragma unroll
+        for (int m = 0; m < RT; ++m) {  // bins i - m and i + 1 + m
+            const float o0 = m == 0 ? 1.0f : c1, o1 = m == 0 ? c1 : c1 - ir;
+            const float w00 = __saturatef(fmaf(-f0, ir, o0)), w10 = __saturatef(fmaf(-f1, ir, o0));
+            const float w01 = __saturatef(fmaf(f0, ir, o1)), w11 = __saturatef(fmaf(f1, ir, o1));
+            float b00 = lds(at0 + 4 * (RT - 1 - m)), b10 = lds(at1 + 4 * (RT - 1 - m));
+            float b01 = lds(at0 + 4 * (RT + m)), b11 = lds(at1 + 4 * (RT + m));
+            if (CAREFUL) {  // a bin outside the footprint is no part of the sum
+                b00 = w00 > 0.f ? b00 : 0.f;
+                b10 = w10 > 0.f ? b10 : 0.f;
+                b01 = w01 > 0.f ? b01 : 0.f;
+                b11 = w11 > 0.f ? b11 : 0.f;
+            }
+            const F2 w0 = pack2(w00, w10), w1 = pack2(w01, w11);
+            tap = m == 0 ? mul2(w0, pack2(b00, b10)) : fma2(w0, pack2(b00, b10), tap);
+            tap = fma2(w1, pack2(b01, b11), tap);
+        }
+        const F2 y = sub2(tap, cmp[e / 2]), t = add2(acc[e / 2], y);
+        cmp[e / 2] = sub2(sub2(t, acc[e / 2]), y);
+        acc[e / 2] = t;
+    }
+}
+
+template <int RT>
+__global__ void __launch_bounds__(BT_X *BT_Y) k_backproject_tile(const float *__restrict__ b, float *__restrict__ u,
+                                                                 const AngleParams *__restrict__ ang,
+                                                                 const int *__restrict__ aoff, int nx, int ny, int nb, int t0) {
+    constexpr int W = 64 * RT;  // words of a segment
+    constexpr int FB = 31 - RT;
+    __shared__ float s_seg[BT_CH][W];
+    __shared__ BtAngle s_a[BT_CH];
+    __shared__ int2 s_k[BT_CH];  // first and last bin of the segment
+    __shared__ float s_w[BT_CH];
+    const int t = t0 + blockIdx.z;
+    const int x0 = blockIdx.x * BT_X, y0 = blockIdx.y * BT_Y * BT_E;
+    const int lane = threadIdx.x, w = threadIdx.y;
+    const int a_begin = aoff[t], a_end = aoff[t + 1];
+    F2 acc[BT_E / 2], cmp[BT_E / 2];
+#pragma unroll
+    for (int e = 0; e < BT_E / 2; ++e) acc[e] = cmp[e] = both(0.f);
+    for (int ac = a_begin; ac < a_end; ac += BT_CH) {
+        const int cn = min(BT_CH, a_end - ac);
+        __syncthreads();
+        if (w == 0 && lane < cn) {
+            const AngleParams &P = ang[ac + lane];
+            const long long a = P.tAQ, bb = P.tBQ, tt = P.t0Q + x0 * a + y0 * bb;
+            const long long ex = (BT_X - 1) * a, ey = (BT_Y * BT_E - 1) * bb;
+            // the segment starts RT bins before the smallest bin coordinate of the tile (one more
+            // than the footprint needs: the fixed-point steps may round below it)
+            const int k0 = (int)((tt + min(0LL, ex) + min(0LL, ey)) >> 40) - RT;
+            const int k1 = (int)((tt + max(0LL, ex) + max(0LL, ey)) >> 40) + RT + 1;
+            s_a[lane] = BtAngle{(tt - ((long long)(k0 + RT - 1) << 40)) >> (40 - FB), (int)(a >> (40 - FB)), (int)(bb >> (40 - FB)),
+                                (float)bb * 9.094947017729282e-13f, P.inv_rfoot, 1.0f - P.inv_rfoot,
+                                (unsigned)__cvta_generic_to_shared(&s_seg[lane][0])};
+            s_k[lane] = make_int2(k0, min(k1, nb - 1));
+            s_w[lane] = P.wfoot;
+        }
+        __syncthreads();
+        bool finite = true;
+        for (int q = w; q < cn; q += BT_Y) {  // a warp per view
+            const int2 kk = s_k[q];
+            const float wf = s_w[q];
+            const float *row = b + (long long)(ac + q) * nb;
+#pragma unroll
+            for (int i = 0; i < W; i += 32) {
+                const int k = kk.x + i + lane;
+                const float v = (k >= 0 && k <= kk.y) ? ldg(row + k) * wf : 0.f;
+                finite = finite && fabsf(v) <= 3.402823466e+38f;
+                s_seg[q][i + lane] = v;
+            }
+        }
+        if (__syncthreads_and(finite)) {
+#pragma unroll 1
+            for (int q = 0; q < cn; ++q) bt_view<RT, false>(s_a[q], acc, cmp);
+        } else {
+#pragma unroll 1
+            for (int q = 0; q < cn; ++q) bt_view<RT, true>(s_a[q], acc, cmp);
+        }
+    }
+    float *ut = u + (long long)t * nx * ny;
+    const int x = x0 + lane;
+#pragma unroll
+    for (int e = 0; e < BT_E; e += 2) {
+        const int y = y0 + w * BT_E + e;
+        float v0, v1;
+        unpack2(acc[e / 2], v0, v1);
+        if (x < nx && y < ny) ut[(long long)y * nx + x] = v0;
+        if (x < nx && y + 1 < ny) ut[(long long)(y + 1) * nx + x] = v1;
+    }
+}
+
+// FP32, any footprint and bin count, with BP_PX pixels per thread (x = x0 + di + 32 e, e < BP_PX:
+// a 128 x 8 tile per CTA): the form for detectors more than twice as fine as the pixels. The
+// per-angle constants come from shared memory as two 16-byte records and are reused for the
+// thread's pixels. A pixel's bin coordinate is the tile origin's (FP64, once per angle) plus its
+// in-tile offset in split steps (exact products).
 constexpr int BP_PX = 4;
 struct __align__(16) BpAngle {
     float fb, tAh, tAl, tBh;
@@ -641,13 +747,20 @@ mof_status launch_backproject(const mof_problem *p, const real *b, real *u, cuda
     // the plain form launches one frame at a time (t0 = t, one z slice), else all frames
     const int nlaunch = per_frame ? p->nt : 1, nz = per_frame ? 1 : p->nt;
     for (int t0 = 0; t0 < nlaunch; ++t0) {
-        if (sizeof(real) == 4) {
+        if (sizeof(real) == 4 && p->bp_reach) {
+            const dim3 gt((p->nx + BT_X - 1) / BT_X, (p->ny + BT_Y * BT_E - 1) / (BT_Y * BT_E), nz), tt(BT_X, BT_Y);
+            const float *bf = (const float *)b;
+            float *uf = (float *)u;
+            ::mof::count_launch();
+            if (p->bp_reach == 1) k_backproject_tile<1><<<gt, tt, 0, st>>>(bf, uf, p->d_ang, p->d_aoff, p->nx, p->ny, p->nb, t0);
+            else k_backproject_tile<2><<<gt, tt, 0, st>>>(bf, uf, p->d_ang, p->d_aoff, p->nx, p->ny, p->nb, t0);
+        } else if (sizeof(real) == 4) {
             dim3 g4((p->nx + BP_TX * BP_PX - 1) / (BP_TX * BP_PX), (p->ny + BP_TY - 1) / BP_TY, nz);
             ::mof::count_launch(), k_backproject4<<<g4, dim3(BP_TX, BP_TY), 0, st>>>((const float *)b, (float *)u, p->d_ang,
                                                                                      p->d_aoff, p->nx, p->ny, p->nb, t0);
         } else {
             dim3 g1(grid.x, grid.y, nz);
-            ::mof::count_launch(), k_backproject<real><<<g1, dim3(BP_TX, BP_TY), 0, st>>>(b, u, p->d_ang, p->d_aoff, p->nx, p->ny,
+            ::mof::count_launch(), k_backproject64<<<g1, dim3(BP_TX, BP_TY), 0, st>>>((const double *)b, (double *)u, p->d_ang, p->d_aoff, p->nx, p->ny,
                                                                                          p->nb, t0);
         }
     }
