@@ -290,14 +290,30 @@ mof_status mof_problem_create_fan(const mof_geometry *g, double source_distance,
     p->rs = source_distance;
     p->rd = detector_distance;
     p->fan_scale = (float)((source_distance + detector_distance) / g->bin_size);
+    // Over the frame (a disk of radius R about the centre) den = q . e >= dmin = rs - R and
+    // |q . f| <= R, so t = (q . f) / den has |t| <= R / dmin and |grad t| = |q| / den^2. A point
+    // h away along x or y projects to within h (|f_i| + |t| |e_i|) / (den - h) of t, and
+    // den / (den - h) <= dmin / (dmin - h).
+    const double R = half_diag, dmin = source_distance - R, tm = R / dmin, scale = p->fan_scale;
+    const double slope = std::sqrt(dmin * dmin + R * R) / (dmin * dmin);  // |grad t| at most
     std::vector<FanView> views(p->A);
     const double cx = 0.5 * (g->nx - 1) * g->pixel_size, cy = 0.5 * (g->ny - 1) * g->pixel_size;
     for (int a = 0; a < p->A; ++a) {
         const double th = g->angles[a], ex = -std::sin(th), ey = std::cos(th);
         // q = p - S, S = -rs e, p = (x h - cx, y h - cy)
         views[a] = FanView{(float)(-cx + source_distance * ex), (float)(-cy + source_distance * ey), (float)ex, (float)ey,
-                           (float)std::cos(th), (float)std::sin(th)};
+                           (float)std::cos(th), (float)std::sin(th), 0.0f};
+        views[a].reach = (float)(scale * g->pixel_size * dmin / (dmin - g->pixel_size) * (1.0 + 1e-5));
     }
+    // The tiled FP32 transpose stages the bins of a 32 x 32 tile (31 sqrt(2) pixels across) with
+    // the reach on both sides, and takes distances between a pixel and a visited ray modulo 64
+    // pixels: the ray is within the reach and two bins of the pixel's projection, a bin is at most
+    // (rs + R) / (scale h cos) pixels wide there, cos >= 1 / (sqrt(2) (1 + t)).
+    const double reach = scale * g->pixel_size * (1.0 + tm) * dmin / (dmin - g->pixel_size) / dmin;  // bins, at most
+    const double width = scale * slope * 31.0 * std::sqrt(2.0) * g->pixel_size + 2.0 * reach;
+    const double tdet = (0.5 * g->nb + 1.0) / scale;
+    const double binpx = (source_distance + R) / (scale * g->pixel_size) * std::sqrt(2.0) * (1.0 + std::fmax(tm, tdet));
+    p->fan_tile = width <= FAN_TILE_RAYS - 8 && (2.0 * reach + 3.0) * binpx <= 30.0;
     cudaError_t e = precision == MOF_FP64 ? upload_fan_rays<double>(p, g->angles) : upload_fan_rays<float>(p, g->angles);
     if (e == cudaSuccess) e = cudaMalloc(&p->d_fanview, sizeof(FanView) * p->A);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_fanview, views.data(), sizeof(FanView) * p->A, cudaMemcpyHostToDevice);

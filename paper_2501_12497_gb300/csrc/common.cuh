@@ -95,7 +95,12 @@ template <> struct FanRay<double> {
 // scale (q . f) / (q . e) + (nb - 1)/2, e the central ray direction, f the detector axis.
 struct FanView {
     float qx0, qy0, ex, ey, fx, fy;
+    // A pixel's two Joseph segments project to within reach max(|f_i| + |t| |e_i|) / (q . e) bins
+    // of its centre's projection t = (q . f) / (q . e) (not scaled), i = x, y
+    float reach;
 };
+// Rays that the tiled FP32 transpose stages per view of a 32 x 32 tile (mof_problem::fan_tile)
+constexpr int FAN_TILE_RAYS = 128;
 // Margin, in bins, of the transpose's FP32 search for the bins a pixel can reach (the host
 // rejects geometries whose rounding bound exceeds half of it)
 constexpr double FAN_PAD_BINS = 0.02;
@@ -117,6 +122,7 @@ struct mof_problem {
     int warp_mode = 0;                  // M(s): 0 bilinear, 1 rounding and clipping (Sec. 3)
     int bp_reach = 0;                   // parallel FP32 transpose: footprints within this many bins each side (1, 2), 0: any
     int fan = 0;                        // 1: fan beam with a flat detector
+    int fan_tile = 0;                   // 1: the tiled FP32 transpose applies
     double rs = 0, rd = 0;              // source and detector distances from the centre
     float fan_scale = 0;                // (rs + rd) / db
     void *d_fanray = nullptr;           // device FanRay<real>[A * nb] (fan only)

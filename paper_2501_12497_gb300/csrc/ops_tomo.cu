@@ -670,18 +670,174 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject4(const float *__re
 }
 
 // ---------------------------------------------------------- K2 fan beam
-// One thread per pixel. A ray steps over rows (or columns) and gives the pixel
-// a weight only at the step of the pixel's row (column), when its crossing
-// there is less than one pixel away; so the rays that reach the pixel are
-// those crossing the open segments of half-length h through its centre along
-// x and along y. Seen from the source, those segments cover the bins between
-// the central projections of their four end points (widened by FAN_PAD bins
-// for the FP32 evaluation of the bounds); for each such bin the forward entry
-// is re-evaluated with the forward's own arithmetic. Steps the forward march
-// skips have crossings more than a pixel outside the frame, so they cannot
-// reach a pixel and need no test here.
+// A ray steps over rows (or columns) and gives the pixel a weight only at the step of the
+// pixel's row (column), when its crossing there is less than one pixel away; so the rays that
+// reach the pixel are those crossing the open segments of half-length h through its centre
+// along x and along y. Steps the forward march skips have crossings more than a pixel outside
+// the frame, so they cannot reach a pixel and need no test here.
+//
+// FP32. A CTA owns a 32 x 32 pixel tile of a frame; per view it stages the rays that can reach
+// the tile in shared memory, each as its crossing at the tile's middle row (column) and its
+// step in fixed point (2^-26 pixels) and its datum times its length per step. A pixel takes
+// every ray whose bin lies within `half` bins of its central projection t = (q . f) / (q . e)
+// (q the pixel seen from the source): its segments project to within
+// h max(|f_x| + |t| |e_x|, |f_y| + |t| |e_y|) / (den - h) of t, with the tile's largest |t| and
+// the bound FanView::reach on the rest, widened by FAN_PAD bins for the FP32 evaluation. A ray's weight is sat(1 - |crossing - pixel|),
+// zero by itself for the rays that the bound lets in without need: the distance is exact in
+// 32-bit integers modulo 64 pixels (the host admits only geometries where a visited ray is
+// closer than 32). Every pixel of a tile and view visits the same number of rays, the most that
+// its bound allows. The sum over the views is compensated (Kahan).
+// A segment with a non-finite datum takes the weights that are zero out of the sum (careful).
+// What bounds it: instruction issue (80 %), about nine instructions per pixel, view and visited
+// ray (2 to 3 rays; 2.8 on average hold the pixel). fan 256x256x32, 30 views:
+// 133 us (error 3.2e-8) against 386 (1.1e-7) for one thread per pixel with four divisions per view
+// and each ray's entry re-evaluated from its 16-byte record.
 constexpr float FAN_PAD = (float)FAN_PAD_BINS;
+constexpr int FT_X = 32, FT_Y = 4, FT_E = 8;  // threads, pixels per thread down a column
+constexpr int FT_CH = 16;                     // views staged at a time
+constexpr int FT_W = FAN_TILE_RAYS;           // rays staged per view
+constexpr int FT_Q = 26;                      // fraction bits of the staged crossings
+struct FtView {
+    float fx, fy, ex, ey, qx0, qy0, reach;  // FanView
+    int k0, n;    // first staged bin, rays a pixel visits
+    unsigned seg; // shared address of the segment less 4 FLOOR_BITS
+    int steps;    // 1: every staged ray steps over rows, 0: over columns, 2: both
+};
 
+// the visits of one view to a thread's column; STEPS: FtView::steps
+template <int STEPS, bool CAREFUL>
+__device__ __forceinline__ void ft_view(const FtView &V, float h, float scale, float toff, int x, int y, int dx, int dy,
+                                        float (&acc)[FT_E], float (&cmp)[FT_E]) {
+    const float qx = fmaf((float)x, h, V.qx0), qy = fmaf((float)y, h, V.qy0);
+    const float num0 = fmaf(qx, V.fx, qy * V.fy), den0 = fmaf(qx, V.ex, qy * V.ey), dn = h * V.fy, dd = h * V.ey;
+    const int n = V.n;
+    const float off = toff - FAN_PAD - (float)V.k0, kmax = (float)(FT_W - n), reach = V.reach;
+    unsigned at[FT_E];
+    float tap[FT_E];
+#pragma unroll
+    for (int e = 0; e < FT_E; ++e) {
+        const float r = __fdividef(1.0f, fmaf((float)e, dd, den0));
+        const float t = fmaf(fmaf((float)e, dn, num0) * r, scale, fmaf(-reach, r, off));
+        // first visited bin relative to the segment, rounded up by the addition; held within the
+        // segment (a non-finite t visits its start)
+        const float k = __fadd_ru(fminf(fmaxf(t, 0.f), kmax), FLOOR_MAGIC);
+        at[e] = V.seg + 4u * (unsigned)__float_as_int(k);
+        tap[e] = 0.f;
+    }
+    // visit by visit, the column's eight pixels side by side (their chains are independent)
+#pragma unroll 1
+    for (int m = 0; m < n; ++m) {
+#pragma unroll
+        for (int e = 0; e < FT_E; ++e) {
+            const int c = __float_as_int(lds(at[e])), s = __float_as_int(lds(at[e] + 4 * FT_W));  // crossing (bit 0: steps over rows), step
+            const float v = lds(at[e] + 8 * FT_W);
+            int d;
+            if (STEPS == 1) d = (dy + e) * s + (c - (dx << FT_Q));
+            else if (STEPS == 0) d = dx * s + (c - ((dy + e) << FT_Q));
+            else d = (c & 1) ? (dy + e) * s + (c - (dx << FT_Q)) : dx * s + (c - ((dy + e) << FT_Q));
+            const float w = __saturatef(fmaf(-fabsf((float)d), 1.0f / (float)(1 << FT_Q), 1.0f));
+            if (!CAREFUL || w > 0.f) tap[e] = fmaf(w, v, tap[e]);
+            at[e] += 4;
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < FT_E; ++e) {
+        const float yv = __fsub_rn(tap[e], cmp[e]), tt = __fadd_rn(acc[e], yv);
+        cmp[e] = __fsub_rn(__fsub_rn(tt, acc[e]), yv);
+        acc[e] = tt;
+    }
+}
+
+__global__ void __launch_bounds__(FT_X *FT_Y) k_backproject_fan_tile(const float *__restrict__ b, float *__restrict__ u,
+                                                                     const FanRay<float> *__restrict__ rays,
+                                                                     const FanView *__restrict__ views,
+                                                                     const int *__restrict__ aoff, int nx, int ny, int nb,
+                                                                     float h, float scale) {
+    __shared__ float s_seg[FT_CH][3][FT_W];  // crossings and steps (integers), data
+    __shared__ FtView s_v[FT_CH];
+    const int t = blockIdx.z;
+    const int x0 = blockIdx.x * FT_X, y0 = blockIdx.y * FT_Y * FT_E;
+    const int lane = threadIdx.x, w = threadIdx.y;
+    const int x1 = min(x0 + FT_X, nx) - 1, y1 = min(y0 + FT_Y * FT_E, ny) - 1;
+    const int xm = x0 + FT_X / 2, ym = y0 + FT_Y * FT_E / 2;  // the staged crossings' row and column
+    const float toff = 0.5f * (float)(nb - 1);
+    float acc[FT_E], cmp[FT_E];
+#pragma unroll
+    for (int e = 0; e < FT_E; ++e) acc[e] = cmp[e] = 0.f;
+    const int a_end = aoff[t + 1];
+    for (int ac = aoff[t]; ac < a_end; ac += FT_CH) {
+        const int cn = min(FT_CH, a_end - ac);
+        __syncthreads();
+        if (w == 0 && lane < cn) {
+            // the extremes of t and of 1 / den over the tile lie at its corners
+            const FanView V = views[ac + lane];
+            float tlo = 3.4e38f, thi = -3.4e38f, rmax = 0.f;  // central projections and 1 / den at the corners
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float qx = fmaf((float)((c & 1) ? x1 : x0), h, V.qx0), qy = fmaf((float)((c & 2) ? y1 : y0), h, V.qy0);
+                const float r = 1.0f / fmaf(qx, V.ex, qy * V.ey), tc = fmaf(qx, V.fx, qy * V.fy) * r;
+                tlo = fminf(tlo, tc);
+                thi = fmaxf(thi, tc);
+                rmax = fmaxf(rmax, r);
+            }
+            const float tm = fmaxf(fabsf(tlo), fabsf(thi));
+            const float reach = V.reach * fmaxf(fmaf(tm, fabsf(V.ex), fabsf(V.fx)), fmaf(tm, fabsf(V.ey), fabsf(V.fy)));
+            const float half = fmaf(reach, rmax, 1.5f * FAN_PAD);
+            const int k0 = (int)floorf(fminf(fmaxf(fmaf(tlo, scale, toff) - half, -1e6f), 1e6f)) - 1;
+            s_v[lane] = FtView{V.fx, V.fy, V.ex, V.ey, V.qx0, V.qy0, reach, k0, min((int)(2.0f * half) + 1, FT_W / 2),
+                               (unsigned)__cvta_generic_to_shared(&s_seg[lane][0][0]) - 4u * (unsigned)FLOOR_BITS, 1};
+        }
+        __syncthreads();
+        bool finite = true;
+        for (int q = w; q < cn; q += FT_Y) {  // a warp per view
+            const int k0 = s_v[q].k0;
+            int any_r = 0, any_c = 0;
+            for (int i = lane; i < FT_W; i += 32) {
+                const int k = k0 + i;
+                int cr = 0, st = 0;
+                float v = 0.f;  // beyond the detector: no datum
+                if (k >= 0 && k < nb) {
+                    const long long o = (long long)(ac + q) * nb + k;
+                    const FanRay<float> F = rays[o];
+                    const int rows = (int)(F.f0q & 1);
+                    const long long c = (F.f0q >> 1) + (rows ? ym : xm) * F.dq - ((long long)(rows ? xm : ym) << 40);
+                    cr = ((int)(c >> (40 - FT_Q)) & ~1) | rows;
+                    st = (int)((F.dq + (1LL << (39 - FT_Q))) >> (40 - FT_Q));
+                    const float df = (float)F.dq * 9.094947017729282e-13f;
+                    v = ldg(b + o) * (h * sqrtf(fmaf(df, df, 1.0f)));
+                    any_r |= rows;
+                    any_c |= !rows;
+                }
+                finite = finite && fabsf(v) <= 3.402823466e+38f;
+                s_seg[q][0][i] = __int_as_float(cr);
+                s_seg[q][1][i] = __int_as_float(st);
+                s_seg[q][2][i] = v;
+            }
+            any_r = __any_sync(0xffffffffu, any_r);
+            any_c = __any_sync(0xffffffffu, any_c);
+            if (lane == 0) s_v[q].steps = any_r && any_c ? 2 : (any_c ? 0 : 1);
+        }
+        const bool careful = !__syncthreads_and(finite);
+        const int x = min(x0 + lane, x1), y = y0 + w * FT_E, dx = lane - FT_X / 2, dy = w * FT_E - FT_Y * FT_E / 2;
+        for (int q = 0; q < cn; ++q) {
+            const int steps = s_v[q].steps;
+            if (careful) ft_view<2, true>(s_v[q], h, scale, toff, x, y, dx, dy, acc, cmp);
+            else if (steps == 1) ft_view<1, false>(s_v[q], h, scale, toff, x, y, dx, dy, acc, cmp);
+            else if (steps == 0) ft_view<0, false>(s_v[q], h, scale, toff, x, y, dx, dy, acc, cmp);
+            else ft_view<2, false>(s_v[q], h, scale, toff, x, y, dx, dy, acc, cmp);
+        }
+    }
+    const int x = x0 + lane;
+#pragma unroll
+    for (int e = 0; e < FT_E; ++e) {
+        const int y = y0 + w * FT_E + e;
+        if (x < nx && y < ny) u[(long long)t * nx * ny + (long long)y * nx + x] = acc[e];
+    }
+}
+
+// Any geometry (and FP64): one thread per pixel; per view the bins between the central
+// projections of the four segment end points (widened by FAN_PAD bins), each re-evaluated with
+// the forward's own arithmetic.
 template <typename real>
 __global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject_fan(const real *__restrict__ b, real *__restrict__ u,
                                                                   const FanRay<real> *__restrict__ rays,
@@ -737,6 +893,14 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject_fan(const real *__
 template <typename real>
 mof_status launch_backproject(const mof_problem *p, const real *b, real *u, cudaStream_t st, bool per_frame) {
     dim3 grid((p->nx + BP_TX - 1) / BP_TX, (p->ny + BP_TY - 1) / BP_TY, p->nt);
+    if (p->fan && p->fan_tile && sizeof(real) == 4) {
+        const dim3 gt((p->nx + FT_X - 1) / FT_X, (p->ny + FT_Y * FT_E - 1) / (FT_Y * FT_E), p->nt);
+        ::mof::count_launch(), k_backproject_fan_tile<<<gt, dim3(FT_X, FT_Y), 0, st>>>(
+            (const float *)b, (float *)u, static_cast<const FanRay<float> *>(p->d_fanray), p->d_fanview, p->d_aoff, p->nx, p->ny,
+            p->nb, (float)p->h, p->fan_scale);
+        MOF_LAUNCH_CHECK();
+        return MOF_OK;
+    }
     if (p->fan) {
         ::mof::count_launch(), k_backproject_fan<real><<<grid, dim3(BP_TX, BP_TY), 0, st>>>(
             b, u, static_cast<const FanRay<real> *>(p->d_fanray), p->d_fanview, p->d_aoff, p->nx, p->ny, p->nb,

@@ -89,3 +89,33 @@ def test_non_finite_bin_reaches_its_own_footprint_only(db, bad):
     out = _apply(p, api.mof_apply_AT, d, p.n)
     assert not np.isfinite(out[w > 1e-4]).any()
     assert np.array_equal(out[w == 0], want[w == 0])
+
+
+# nx, ny, nt, na, nb, bin size, source and detector distance: the 1.5x magnification of the
+# workloads on tiles with remainders (views beyond one stage, fans that straddle 45 degrees), the
+# same turned to 45 degrees exactly, and a source too near for the tiled form
+FANS = [(33, 65, 2, 17, 100, 1.6, 140.0, 70.0), (64, 64, 2, 4, 97, 1.5, 128.0, 64.0), (200, 31, 2, 5, 260, 1.6, 400.0, 200.0),
+        (31, 31, 2, 33, 64, 1.2, 30.0, 3.0)]
+
+
+@pytest.mark.parametrize("case", FANS)
+def test_fan_transpose_at_tile_edges(case):
+    nx, ny, nt, na, nb, db, rs, rd = case
+    p, g = _pair((nx, ny, nt, na, nb, db), fan=(rs, rd))
+    d = np.random.default_rng(5).standard_normal(p.m).astype(np.float32)
+    assert _rel(_apply(p, api.mof_apply_AT, d, p.n), O.backproject(g, d.astype(np.float64)).ravel()) <= 1e-6
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_fan_non_finite_bin_reaches_its_own_rays_pixels_only(bad):
+    p, g = _pair((64, 48, 2, 5, 100, 1.6), fan=(140.0, 70.0))
+    d = np.random.default_rng(6).standard_normal(p.m).astype(np.float32)
+    k = 3 * 100 + 52
+    e = np.zeros(p.m)
+    e[k] = 1.0
+    w = O.backproject(g, e).ravel()
+    want = _apply(p, api.mof_apply_AT, d, p.n)
+    d[k] = bad
+    out = _apply(p, api.mof_apply_AT, d, p.n)
+    assert not np.isfinite(out[w > 1e-4]).any()
+    assert np.array_equal(out[w == 0], want[w == 0])
