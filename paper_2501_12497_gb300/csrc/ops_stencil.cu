@@ -54,14 +54,33 @@ __device__ __forceinline__ void warp_axis(int x, real v, int n, int &i0, int &i1
     i1 = min(i0 + 1, n - 1);
 }
 
+// FP32 form: the floor by an addition that rounds down to the integers (1.5 2^23), one
+// conversion less; v held within +-8192, beyond which every sample of a frame (at most 4096
+// pixels a side) is clipped. The same values as the general form.
+constexpr float FLOOR_MAGIC = 12582912.0f;
+constexpr int FLOOR_BITS = 0x4B400000;
+__device__ __forceinline__ void warp_axis(int x, float v, int n, int &i0, int &i1, float &w, int wm) {
+    const float vc = v == v ? fminf(fmaxf(v, -8192.f), 8192.f) : 0.f;  // NaN: identity sample
+    if (wm) {
+        i0 = min(max(x + (int)roundf(vc), 0), n - 1);
+        w = 0.f;
+    } else {
+        const float t = __fadd_rd(vc, FLOOR_MAGIC);
+        const int I = x + (__float_as_int(t) - FLOOR_BITS);
+        i0 = min(max(I, 0), n - 1);
+        w = (unsigned)I < (unsigned)(n - 1) ? vc - (t - FLOOR_MAGIC) : 0.f;
+    }
+    i1 = min(i0 + 1, n - 1);
+}
+
 template <typename real>
 __device__ __forceinline__ real bilinear(const real *__restrict__ f, int nx, int ny, int x, int y, real vx, real vy, int wm) {
     int x0, x1, y0, y1;
     real wx, wy;
     warp_axis(x, vx, nx, x0, x1, wx, wm);
     warp_axis(y, vy, ny, y0, y1, wy, wm);
-    const real a = ldg(f + (long long)y0 * nx + x0), b = ldg(f + (long long)y0 * nx + x1);
-    const real c = ldg(f + (long long)y1 * nx + x0), d = ldg(f + (long long)y1 * nx + x1);
+    const real a = ldg(f + (y0 * nx + x0)), b = ldg(f + (y0 * nx + x1));  // a frame holds at most 2^24 pixels
+    const real c = ldg(f + (y1 * nx + x0)), d = ldg(f + (y1 * nx + x1));
     const real top = (1 - wx) * a + wx * b, bot = (1 - wx) * c + wx * d;
     return (1 - wy) * top + wy * bot;
 }
@@ -138,17 +157,13 @@ __device__ __forceinline__ double fx_out(long long tot, int E, double f) {
 // most cb terms each
 template <typename real>
 __device__ __forceinline__ int fx_exponent(int ex, long long cb) { return 62 - (64 - __clzll(cb - 1)) - ex; }
-// bit pattern of |v| (ordered like the magnitudes; non-finite values above every finite one)
-__device__ __forceinline__ unsigned long long abs_bits(float v) { return (unsigned long long)(__float_as_uint(v) & 0x7fffffffu); }
-__device__ __forceinline__ unsigned long long abs_bits(double v) {
-    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
-}
-__device__ __forceinline__ bool bits_finite(unsigned long long b, float) { return b < 0x7f800000ull; }
+// magnitudes as bit patterns (mag_bits): non-finite values lie above every finite one
+__device__ __forceinline__ bool bits_finite(unsigned b, float) { return b < 0x7f800000u; }
 __device__ __forceinline__ bool bits_finite(unsigned long long b, double) { return b < 0x7ff0000000000000ull; }
 // exponent ex with |v| < 2^ex for the magnitude whose bits are b (b > 0, finite)
-__device__ __forceinline__ int bits_exp(unsigned long long b, float) {
+__device__ __forceinline__ int bits_exp(unsigned b, float) {
     int ex = 0;
-    frexpf(__uint_as_float((unsigned)b), &ex);
+    frexpf(__uint_as_float(b), &ex);
     return ex;
 }
 __device__ __forceinline__ int bits_exp(unsigned long long b, double) {
@@ -161,12 +176,12 @@ template <> struct FxLimits<float> { static constexpr int EMAX = 126, EMIN = -12
 template <> struct FxLimits<double> { static constexpr int EMAX = 1000, EMIN = -1000; };
 
 // A rectangle of candidate source pixels of one destination tile: w columns from x0,
-// rows from y0, its pixels numbered from `start` in the tile's flat candidate list;
-// magic = ceil(2^64 / w) turns a pixel's number into its row with one multiply-high.
+// rows from y0, its pixels numbered from `start` in the tile's flat candidate list; iw = 1 / w
+// turns a pixel's number (below BW BH) into its row by one multiplication of number + 1/2.
 struct SrcRect {
     int x0, y0, w, start;
-    unsigned long long magic;
-    int term, pad_;
+    float iw;
+    int term;
 };
 constexpr int MAXR = 64;  // rectangles per round of a destination tile
 
@@ -428,7 +443,10 @@ mof_status launch_tile_bounds(const mof_problem *p, const real *s, const real *s
 // rectangles of the velocity fields' source tiles, numbered c in [cursor, nc0 + nc1)
 // (the candidate tiles of term 0, then of term 1), until the list is full or the tiles
 // are exhausted; MODE 0 (bilinear footprints) or MODE 1 (single destinations). Writes the
-// number of rectangles and of their pixels and the next cursor to sh[0..2].
+// number of rectangles and of their pixels and the next cursor to sh[0..2], and to sh[3] a bound
+// on how many of the round's sources can reach any one pixel: per term, the extent of the
+// displacements of the tiles that contribute (MODE 0: a source p reaches q only with q - p - d
+// in {0, 1} per axis).
 struct TermTiles {
     const int4 *bnd;  // the field's source-tile bounds (its reach after them)
     int txa, tya, ntx, nc;
@@ -454,10 +472,12 @@ __device__ void build_rects(const TermTiles &T0, const TermTiles &T1, int cursor
     const int lane = threadIdx.x & 31;
     const int total = T0.nc + T1.nc, ext = MODE == 0 ? 1 : 0;
     int cnt = 0, npx = 0;
+    int xlo[2] = {INT_MAX, INT_MAX}, xhi[2] = {INT_MIN, INT_MIN}, ylo[2] = {INT_MAX, INT_MAX}, yhi[2] = {INT_MIN, INT_MIN};
     while (cursor < total && cnt <= MAXR - 32) {
         const int c = cursor + lane;
         bool valid = false;
         int rx0 = 0, ry0 = 0, w = 0, h = 0, term = 0;
+        int4 db = make_int4(0, 0, 0, 0);
         if (c < total) {
             term = c < T0.nc ? 0 : 1;
             const TermTiles &T = term ? T1 : T0;
@@ -472,7 +492,16 @@ __device__ void build_rects(const TermTiles &T0, const TermTiles &T1, int cursor
             w = rx1 - rx0 + 1;
             h = ry1 - ry0 + 1;
             valid = w > 0 && h > 0;
+            db = b;
         }
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            if (valid && term == e) {
+                xlo[e] = min(xlo[e], db.x);
+                xhi[e] = max(xhi[e], db.y);
+                ylo[e] = min(ylo[e], db.z);
+                yhi[e] = max(yhi[e], db.w);
+            }
         const unsigned m = __ballot_sync(0xffffffffu, valid);
         const int mine = valid ? w * h : 0;
         int incl = mine;
@@ -487,28 +516,40 @@ __device__ void build_rects(const TermTiles &T0, const TermTiles &T1, int cursor
             R.y0 = ry0;
             R.w = w;
             R.start = npx + incl - mine;
-            R.magic = w > 1 ? (~0ull) / (unsigned long long)w + 1ull : 0ull;
+            R.iw = 1.0f / (float)w;
             R.term = term;
         }
         cnt += __popc(m);
         npx += __shfl_sync(0xffffffffu, incl, 31);
         cursor += 32;
     }
+    int most = 0;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int ax = __reduce_min_sync(0xffffffffu, xlo[e]), bx = __reduce_max_sync(0xffffffffu, xhi[e]);
+        const int ay = __reduce_min_sync(0xffffffffu, ylo[e]), by = __reduce_max_sync(0xffffffffu, yhi[e]);
+        if (ax <= bx) most += min(bx - ax + 1 + ext, 1024) * min(by - ay + 1 + ext, 1024);
+    }
     if (lane == 0) {
         sh[0] = cnt;
         sh[1] = npx;
         sh[2] = cursor;
+        sh[3] = most;
     }
 }
 
 // pixel number k of the current round -> (term, px, py); r is the caller's running rectangle
-// index (k only grows within a thread, so the search resumes where it stopped)
-__device__ __forceinline__ void rect_pixel(const SrcRect *rect, int nrect, int k, int &r, int &term, int &px, int &py) {
-    while (r + 1 < nrect && rect[r + 1].start <= k) ++r;
+// index, next the number where the following one starts (k only grows within a thread, so the
+// search resumes where it stopped; r = -1, next = 0 at the start)
+__device__ __forceinline__ void rect_pixel(const SrcRect *rect, int nrect, int k, int &r, int &next, int &term, int &px, int &py) {
+    while (next <= k) {
+        ++r;
+        next = r + 1 < nrect ? rect[r + 1].start : INT_MAX;
+    }
     const SrcRect &R = rect[r];
-    const unsigned long long loc = (unsigned long long)(k - R.start);
-    const int row = R.magic ? (int)__umul64hi(loc, R.magic) : (int)loc;
-    px = R.x0 + (int)loc - row * R.w;
+    const int loc = k - R.start;
+    const int row = (int)(((float)loc + 0.5f) * R.iw);
+    px = R.x0 + loc - row * R.w;
     py = R.y0 + row;
     term = R.term;
 }
@@ -520,10 +561,139 @@ __device__ __forceinline__ void rect_pixel(const SrcRect *rect, int nrect, int k
 // with `temporal`, L_t^T w_t L_t x, all times scale * lam, plus y_add) as a scatter into
 // the tile: every source p whose bilinear footprint can touch D (the candidate rectangles
 // of the two velocity fields) adds w * r(p) to the pixels of its footprint inside D. The
-// terms are summed exactly in 64-bit fixed point (shared-memory integer atomics), so the
-// result does not depend on the order of the additions. Pass 0 finds the largest term
-// magnitude of the tile (it sets the fixed-point scale), pass 1 scatters. A non-finite
-// term makes the tile's outputs NaN.
+// terms are summed exactly in fixed point, so the result does not depend on the order of
+// the additions. Pass 0 finds the largest term magnitude of the tile (it sets the
+// fixed-point scale), pass 1 scatters. A non-finite term makes the tile's outputs NaN.
+//
+// FP32, and the candidates fit one round of the lists (they do unless the displacements vary by
+// many pixels within a tile): pass 0 keeps each candidate's position and value in shared memory
+// for pass 1, and a term x, scaled below 2^48, is added as x = h 2^24 + l in two 32-bit integer
+// sums (native shared-memory reductions; 64-bit ones are compare-and-swap loops). A pixel gets
+// at most FAST_MOST terms from the candidates and eight of its own, so neither sum overflows. The
+// sums have a border of one pixel around the tile: a candidate whose first corner lies in or
+// next to the tile adds all four corners without further tests. Else (and in FP64) the sums are
+// 64-bit, and every corner is tested.
+// What bounds it: instruction issue (62 %) and the latency of its loads, 8 warps of 16 per SM
+// resident. 1024x1024x64 with displacements of up to 3 pixels: Theta^T W Theta 5.12 -> 3.09 ms
+// (scatter 3.8 -> 2.1, rows 0.90 -> 0.64), Mhat^T 3.29 -> 2.03 ms against 64-bit sums for every tile,
+// each candidate's number divided by its rectangle's width in 64 bits, and its values read twice.
+constexpr int FAST_NC = 3072, FAST_MOST = 118;
+constexpr int FAST_W = BW + 2, FAST_N = FAST_W * (BH + 2);
+
+// x = h 2^24 + l for |x| < 2^48
+__device__ __forceinline__ void fx_split(float x, int &h, int &l) {
+    h = __float2int_rn(x * 5.9604644775390625e-08f);
+    l = __float2int_rn(fmaf((float)h, -16777216.0f, x));
+}
+// bit pattern of |v| as the element's unsigned type (ordered like the magnitudes)
+__device__ __forceinline__ unsigned mag_bits(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned long long mag_bits(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+// sums of a pixel's own terms: FP32 with the additions' rounding errors, FP64 in fixed point later
+template <typename real> struct OwnSum;
+template <> struct OwnSum<float> {
+    DFAcc a;
+    __device__ __forceinline__ void add(float v) { a.add(v); }
+    __device__ __forceinline__ void fixed(float sc, int &h, int &l) const {
+        int h1, l1;
+        fx_split(a.hi * sc, h, l);
+        fx_split(a.lo * sc, h1, l1);
+        h += h1;
+        l += l1;
+    }
+    __device__ __forceinline__ long long fixed(float sc) const { return fx_term(a.hi * sc) + fx_term(a.lo * sc); }
+};
+template <> struct OwnSum<double> {
+    double v[8];
+    int n = 0;
+    __device__ __forceinline__ void add(double x) { v[n++] = x; }
+    __device__ __forceinline__ void fixed(double, int &, int &) const {}
+    __device__ __forceinline__ long long fixed(double sc) const {
+        long long t = 0;
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (e < n) t += fx_term(v[e] * sc);
+        return t;
+    }
+};
+
+// weighted difference g / sqrt(gk^2 + eps^2)
+__device__ __forceinline__ double wdiff(double g, double gk, double eps2) { return g / sqrt(gk * gk + eps2); }
+// FP32: the reciprocal square root's approximation and one Newton step (within an ulp of the
+// exact 1 / sqrt), times g: as accurate as the rounded square root and division, a third of
+// their instructions
+__device__ __forceinline__ float wdiff(float g, float gk, float eps2) {
+    const float v = fmaf(gk, gk, eps2), y = rsqrtf(v);
+    const float e = fmaf(-v * y, y, 1.0f);
+    return g * (v < 3.0e38f && y < 3.0e38f ? fmaf(0.5f * e, y, y) : y);
+}
+
+// What a tile's scatter works on
+template <typename real>
+struct WarpTile {
+    const real *val0, *val1, *v0, *v1;  // terms 0 and 1: values and velocities
+    TermTiles T0, T1;
+    int X0, X1, Y0, Y1, nx, ny, wm;
+    long long ns;
+};
+
+// One 64-bit pass over all rounds of candidates: pass 0 raises mb, pass 1 adds into acc. Returns
+// the number of candidates. All threads call.
+template <typename real, typename bits_t>
+__device__ __noinline__ long long warpT_pass64(const WarpTile<real> &W, int pass, real sc, bits_t &mb, long long *acc,
+                                               SrcRect *rect, int *sh) {
+    const int tid = threadIdx.x;
+    long long count = 0;
+    int cursor = 0;
+    do {
+        __syncthreads();  // the previous round's rectangles are consumed
+        if (tid < 32) build_rects<0>(W.T0, W.T1, cursor, W.X0, W.X1, W.Y0, W.Y1, W.nx, W.ny, rect, sh);
+        __syncthreads();
+        const int nrect = sh[0], npx = sh[1];
+        cursor = sh[2];
+        count += npx;
+        int ri = -1, next = 0;
+        for (int k = tid; k < npx; k += BT) {
+            int term, px, py;
+            rect_pixel(rect, nrect, k, ri, next, term, px, py);
+            const long long i = (long long)py * W.nx + px;
+            const real val = term ? W.val1[i] : W.val0[i];
+            if (pass == 0) {
+                mb = max(mb, mag_bits(val));
+                continue;
+            }
+            const real *vv = term ? W.v1 : W.v0;
+            int x0, x1, y0, y1;
+            real wx, wy;
+            warp_axis(px, vv[i], W.nx, x0, x1, wx, W.wm);
+            warp_axis(py, vv[W.ns + i], W.ny, y0, y1, wy, W.wm);
+            // footprint corners with their axis weights (x1 == x0 only where the sample sits
+            // on the last column, with wx = 0: one corner of weight (1 - wx) + wx); the
+            // scaled value times the y weight, then times the x weight
+            const bool xs = x1 == x0, ys = y1 == y0;
+            const real ax0 = xs ? (1 - wx) + wx : 1 - wx, ay0 = ys ? (1 - wy) + wy : 1 - wy;
+            const real vs = -(val * sc);
+#pragma unroll
+            for (int cy = 0; cy < 2; ++cy) {
+                const int yc = cy ? y1 : y0;
+                const real ay = cy ? wy : ay0;
+                if ((cy && ys) || yc < W.Y0 || yc > W.Y1 || ay == (real)0) continue;
+                const real vy = vs * ay;
+#pragma unroll
+                for (int cx = 0; cx < 2; ++cx) {
+                    const int xc = cx ? x1 : x0;
+                    const real ax = cx ? wx : ax0;
+                    if ((cx && xs) || xc < W.X0 || xc > W.X1 || ax == (real)0) continue;
+                    atomicAdd(reinterpret_cast<unsigned long long *>(&acc[(yc - W.Y0) * BW + (xc - W.X0)]),
+                              (unsigned long long)fx_term(vy * ax));
+                }
+            }
+        }
+    } while (cursor < W.T0.nc + W.T1.nc);
+    return count;
+}
+
 template <typename real, bool REGN>
 __global__ void __launch_bounds__(BT) k_warpT_tile(const real *__restrict__ r, const real *__restrict__ s,
                                                    const real *__restrict__ sr, const int *__restrict__ bnd_s,
@@ -531,138 +701,186 @@ __global__ void __launch_bounds__(BT) k_warpT_tile(const real *__restrict__ r, c
                                                    const real *__restrict__ x, const real *__restrict__ uk, real eps2,
                                                    double scale, const double *__restrict__ lam, const real *__restrict__ y_add,
                                                    int temporal, real *__restrict__ out) {
-    __shared__ long long acc[BW * BH];
+    constexpr bool F32 = sizeof(real) == 4;
+    using bits_t = decltype(mag_bits(real()));
+    // 64-bit sums, or the high and the low 32-bit sums with their border
+    __shared__ long long acc[F32 && FAST_N > BW * BH ? FAST_N : BW * BH];
     __shared__ SrcRect rect[MAXR];
-    __shared__ int sh[3];
-    __shared__ unsigned long long s_max;
-    __shared__ long long s_total;
+    __shared__ int sh[4];
+    __shared__ bits_t s_max;
     __shared__ real s_sc;  // scale * lam, once per block (FP64 kept out of the threads)
+    __shared__ float s_val[F32 ? FAST_NC : 1];
+    __shared__ int s_pos[F32 ? FAST_NC : 1];  // x | y << 12 | term << 24
     const int t = blockIdx.z, tid = threadIdx.x;
-    const int X0 = blockIdx.x * BW, Y0 = blockIdx.y * BH;
-    const int X1 = min(X0 + BW - 1, nx - 1), Y1 = min(Y0 + BH - 1, ny - 1);
-    const long long ns = (long long)nx * ny;
+    WarpTile<real> W;
+    W.X0 = blockIdx.x * BW;
+    W.Y0 = blockIdx.y * BH;
+    W.X1 = min(W.X0 + BW - 1, nx - 1);
+    W.Y1 = min(W.Y0 + BH - 1, ny - 1);
+    W.nx = nx;
+    W.ny = ny;
+    W.wm = wm;
+    W.ns = (long long)nx * ny;
+    const long long ns = W.ns;
+    const int X0 = W.X0, X1 = W.X1, Y0 = W.Y0, Y1 = W.Y1;
     const int txn = (nx + BW - 1) / BW, tyn = (ny + BH - 1) / BH;
     // term 0: rows r1 of pair t (sources on frame t+1, velocity sr_t); term 1: rows r0 of
     // pair t-1 (sources on frame t-1, velocity s_{t-1})
-    TermTiles T0{nullptr, 0, 0, 1, 0}, T1{nullptr, 0, 0, 1, 0};
-    if (t < np) T0 = term_tiles(bnd_sr + 4LL * t * (tiles + 1), tiles, txn, tyn, X0, X1, Y0, Y1, nx, ny);
-    if (t > 0) T1 = term_tiles(bnd_s + 4LL * (t - 1) * (tiles + 1), tiles, txn, tyn, X0, X1, Y0, Y1, nx, ny);
-    const real *val0 = r + (np + t) * ns, *val1 = r + (long long)(t - 1) * ns;
-    const real *v0 = sr + 2LL * t * ns, *v1 = s + 2LL * (t - 1) * ns;
-    for (int l = tid; l < BW * BH; l += BT) acc[l] = 0;
+    W.T0 = W.T1 = TermTiles{nullptr, 0, 0, 1, 0};
+    if (t < np) W.T0 = term_tiles(bnd_sr + 4LL * t * (tiles + 1), tiles, txn, tyn, X0, X1, Y0, Y1, nx, ny);
+    if (t > 0) W.T1 = term_tiles(bnd_s + 4LL * (t - 1) * (tiles + 1), tiles, txn, tyn, X0, X1, Y0, Y1, nx, ny);
+    W.val0 = r + (np + t) * ns;
+    W.val1 = r + (long long)(t - 1) * ns;
+    W.v0 = sr + 2LL * t * ns;
+    W.v1 = s + 2LL * (t - 1) * ns;
+    if (tid < 32) build_rects<0>(W.T0, W.T1, 0, X0, X1, Y0, Y1, nx, ny, rect, sh);
+    for (int l = tid; l < (int)(sizeof(acc) / sizeof(acc[0])); l += BT) acc[l] = 0;
     if (tid == 0) {
         s_max = 0;
-        s_total = 0;
         s_sc = REGN ? (real)(lam ? scale * *lam : scale) : (real)1;
     }
 
     // the pixel's own terms: the identity parts of Mhat^T and (REGN) the weighted differences
     constexpr int NOWN = REGN ? 8 : 2;
-    real own[BPT][NOWN];
-    unsigned long long mb = 0;
+    OwnSum<real> own[BPT];
+    bits_t mb = 0;
 #pragma unroll
     for (int k = 0; k < BPT; ++k) {
         const int l = tid + k * BT, xx = X0 + (l % BW), yy = Y0 + l / BW;
-#pragma unroll
-        for (int e = 0; e < NOWN; ++e) own[k][e] = 0;
         if (xx > X1 || yy > Y1) continue;
-        const long long i = (long long)yy * nx + xx;
-        if (t < np) own[k][0] = r[t * ns + i];
-        if (t > 0) own[k][1] = r[(np + t - 1) * ns + i];
+        const int i = yy * nx + xx;
+        auto term = [&](real v) {
+            mb = max(mb, mag_bits(v));
+            own[k].add(v);
+        };
+        if (t < np) term(r[t * ns + i]);
+        if (t > 0) term(r[(np + t - 1) * ns + i]);
         if (REGN) {
-            const real *f = x + t * ns, *kk = uk + t * ns;
-            auto wd = [&](const real *fa, const real *ka, long long j, long long step) -> real {
-                const real g = fa[j + step] - fa[j], gk = ka[j + step] - ka[j];
-                return g / sqrt(gk * gk + eps2);
-            };
-            if (xx > 0) own[k][2] = wd(f, kk, i - 1, 1);
-            if (xx < nx - 1) own[k][3] = -wd(f, kk, i, 1);
-            if (yy > 0) own[k][4] = wd(f, kk, i - nx, nx);
-            if (yy < ny - 1) own[k][5] = -wd(f, kk, i, nx);
+            const real *f = x + t * ns + i, *kk = uk + t * ns + i;
+            const real f0 = *f, k0 = *kk;
+            if (xx > 0) term(wdiff(f0 - f[-1], k0 - kk[-1], eps2));
+            if (xx < nx - 1) term(-wdiff(f[1] - f0, kk[1] - k0, eps2));
+            if (yy > 0) term(wdiff(f0 - f[-nx], k0 - kk[-nx], eps2));
+            if (yy < ny - 1) term(-wdiff(f[nx] - f0, kk[nx] - k0, eps2));
             if (temporal) {
-                if (t > 0) own[k][6] = wd(f - ns, kk - ns, i, ns);
-                if (t < np) own[k][7] = -wd(f, kk, i, ns);
+                if (t > 0) term(wdiff(f0 - f[-ns], k0 - kk[-ns], eps2));
+                if (t < np) term(-wdiff(f[ns] - f0, kk[ns] - k0, eps2));
             }
         }
-#pragma unroll
-        for (int e = 0; e < NOWN; ++e) mb = max(mb, abs_bits(own[k][e]));
     }
-
+    // the tile's largest magnitude from the threads' mb, and the fixed-point scale of E
+    auto tile_max = [&]() {
+        bits_t m = mb;
+        if constexpr (F32) {
+            m = __reduce_max_sync(0xffffffffu, m);
+        } else {
+            const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(m >> 32));
+            const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(m >> 32) == hi ? (unsigned)m : 0u);
+            m = ((bits_t)hi << 32) | lo;
+        }
+        if ((tid & 31) == 0) atomicMax(&s_max, m);
+        __syncthreads();
+        return s_max;
+    };
+    auto clamp_E = [](int E) { return min(max(E, FxLimits<real>::EMIN), FxLimits<real>::EMAX); };
+    __syncthreads();
     real sc = 0;
     int E = 0;
-    bool finite = true;
-    for (int pass = 0; pass < 2; ++pass) {
-        int cursor = 0;
-        do {
-            __syncthreads();  // the previous round's rectangles are consumed
-            if (tid < 32) build_rects<0>(T0, T1, cursor, X0, X1, Y0, Y1, nx, ny, rect, sh);
-            __syncthreads();
+    bool finite = true, fast = false;
+    if constexpr (F32) fast = sh[2] >= W.T0.nc + W.T1.nc && sh[1] <= FAST_NC && sh[3] <= FAST_MOST;
+    if (fast) {
+        if constexpr (F32) {
             const int nrect = sh[0], npx = sh[1];
-            cursor = sh[2];
-            if (pass == 0 && tid == 0) s_total += npx;
-            int ri = 0;
-            for (int k = tid; k < npx; k += BT) {
-                int term, px, py;
-                rect_pixel(rect, nrect, k, ri, term, px, py);
-                const long long i = (long long)py * nx + px;
-                const real val = term ? val1[i] : val0[i];
-                if (pass == 0) {
-                    mb = max(mb, abs_bits(val));
-                    continue;
+            int ri = -1, next = 0;
+            constexpr int U = 4;  // candidates with their loads in flight
+            for (int k0 = tid; k0 < npx; k0 += U * BT) {
+                float val[U];
+                int pos[U];
+#pragma unroll
+                for (int e = 0; e < U; ++e) {
+                    val[e] = 0.f;
+                    if (k0 + e * BT >= npx) continue;
+                    int term, px, py;
+                    rect_pixel(rect, nrect, k0 + e * BT, ri, next, term, px, py);
+                    val[e] = ldg((term ? W.val1 : W.val0) + (py * nx + px));
+                    pos[e] = px | py << 12 | term << 24;
                 }
-                const real *vv = term ? v1 : v0;
-                int x0, x1, y0, y1;
-                real wx, wy;
-                warp_axis(px, vv[i], nx, x0, x1, wx, wm);
-                warp_axis(py, vv[ns + i], ny, y0, y1, wy, wm);
-                // footprint corners with their axis weights (x1 == x0 only where the sample sits
-                // on the last column, with wx = 0: one corner of weight (1 - wx) + wx); the
-                // scaled value times the y weight, then times the x weight
-                const bool xs = x1 == x0, ys = y1 == y0;
-                const real ax0 = xs ? (1 - wx) + wx : 1 - wx, ay0 = ys ? (1 - wy) + wy : 1 - wy;
-                const real vs = -(val * sc);
 #pragma unroll
-                for (int cy = 0; cy < 2; ++cy) {
-                    const int yc = cy ? y1 : y0;
-                    const real ay = cy ? wy : ay0;
-                    if ((cy && ys) || yc < Y0 || yc > Y1 || ay == (real)0) continue;
-                    const real vy = vs * ay;
-#pragma unroll
-                    for (int cx = 0; cx < 2; ++cx) {
-                        const int xc = cx ? x1 : x0;
-                        const real ax = cx ? wx : ax0;
-                        if ((cx && xs) || xc < X0 || xc > X1 || ax == (real)0) continue;
-                        atomicAdd(reinterpret_cast<unsigned long long *>(&acc[(yc - Y0) * BW + (xc - X0)]),
-                                  (unsigned long long)fx_term(vy * ax));
-                    }
+                for (int e = 0; e < U; ++e) {
+                    if (k0 + e * BT >= npx) continue;
+                    s_val[k0 + e * BT] = val[e];
+                    s_pos[k0 + e * BT] = pos[e];
+                    mb = max(mb, mag_bits(val[e]));
                 }
             }
-        } while (cursor < T0.nc + T1.nc);
-        if (pass == 0) {
-            // the tile's largest magnitude (warp maximum of the 64-bit patterns in two 32-bit
-            // halves, then the CTA maximum) and the fixed-point scale 2^E
-            const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(mb >> 32));
-            const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(mb >> 32) == hi ? (unsigned)mb : 0u);
-            if ((tid & 31) == 0) atomicMax(&s_max, ((unsigned long long)hi << 32) | lo);
-            __syncthreads();
-            const unsigned long long M = s_max;
+            const bits_t M = tile_max();
             finite = bits_finite(M, real(0));
-            E = fx_exponent<real>(M ? bits_exp(M, real(0)) : 0, 4 * s_total + NOWN + 1);
-            E = min(max(E, FxLimits<real>::EMIN), FxLimits<real>::EMAX);
+            E = clamp_E(48 - (M ? bits_exp(M, real(0)) : 0));
             fx_pow2(E, sc);
-            if (!finite) break;
+            int *hi = reinterpret_cast<int *>(acc), *lo = hi + FAST_N;
+            const unsigned nw = X1 - X0 + 1, nh = Y1 - Y0 + 1;
+            // the next candidate's velocity is loaded while this one's terms are added
+            float vx = 0.f, vy = 0.f;
+            auto fetch = [&](int k) {
+                const int pos = s_pos[k];
+                const float *vv = (pos >> 24 ? W.v1 : W.v0) + (((pos >> 12) & 4095) * nx + (pos & 4095));
+                vx = ldg(vv);
+                vy = ldg(vv + ns);
+            };
+            if (finite && tid < npx) fetch(tid);
+            for (int k = tid; finite && k < npx; k += BT) {
+                const int pos = s_pos[k], px = pos & 4095, py = (pos >> 12) & 4095;
+                int x0, x1, y0, y1;
+                float wx, wy;
+                const float cvx = vx, cvy = vy;
+                if (k + BT < npx) fetch(k + BT);
+                warp_axis(px, cvx, nx, x0, x1, wx, wm);
+                warp_axis(py, cvy, ny, y0, y1, wy, wm);
+                // corners with their axis weights (a clipped axis has wx = 0: its second corner adds
+                // zero); the scaled value times the y weight, then times the x weight
+                const int cx = x0 - X0 + 1, cy = y0 - Y0 + 1;
+                if ((unsigned)cx > nw || (unsigned)cy > nh) continue;
+                const float vs = -(s_val[k] * sc), ux = 1.0f - wx, b0 = vs * (1.0f - wy), b1 = vs * wy;
+                int *ph = hi + cy * FAST_W + cx, *pl = ph + FAST_N;
+                int h, l;
+                fx_split(b0 * ux, h, l);
+                atomicAdd(ph, h);
+                atomicAdd(pl, l);
+                fx_split(b0 * wx, h, l);
+                atomicAdd(ph + 1, h);
+                atomicAdd(pl + 1, l);
+                fx_split(b1 * ux, h, l);
+                atomicAdd(ph + FAST_W, h);
+                atomicAdd(pl + FAST_W, l);
+                fx_split(b1 * wx, h, l);
+                atomicAdd(ph + FAST_W + 1, h);
+                atomicAdd(pl + FAST_W + 1, l);
+            }
         }
+    } else {
+        const long long count = warpT_pass64<real, bits_t>(W, 0, sc, mb, acc, rect, sh);
+        const bits_t M = tile_max();
+        finite = bits_finite(M, real(0));
+        E = clamp_E(fx_exponent<real>(M ? bits_exp(M, real(0)) : 0, 4 * count + NOWN + 1));
+        fx_pow2(E, sc);
+        if (finite) warpT_pass64<real, bits_t>(W, 1, sc, mb, acc, rect, sh);
     }
     __syncthreads();
     const real f_out = s_sc;
 #pragma unroll
     for (int k = 0; k < BPT; ++k) {
-        const int l = tid + k * BT, xx = X0 + (l % BW), yy = Y0 + l / BW;
+        const int l = tid + k * BT, lx = l % BW, ly = l / BW, xx = X0 + lx, yy = Y0 + ly;
         if (xx > X1 || yy > Y1) continue;
         const long long o = t * ns + (long long)yy * nx + xx;
-        long long tot = acc[l];
-#pragma unroll
-        for (int e = 0; e < NOWN; ++e) tot += fx_term(own[k][e] * sc);
+        long long tot;
+        if (fast) {
+            const int *hi = reinterpret_cast<const int *>(acc) + (ly + 1) * FAST_W + lx + 1;
+            int h, g;
+            own[k].fixed(sc, h, g);
+            tot = ((long long)(hi[0] + h) << 24) + (hi[FAST_N] + g);
+        } else {
+            tot = acc[l] + own[k].fixed(sc);
+        }
         real res = fx_out(tot, E, f_out);
         if (!finite) res = (real)NAN;
         out[o] = (REGN && y_add) ? y_add[o] + res : res;
@@ -700,8 +918,8 @@ __device__ __forceinline__ void bilinear_grad(const real *__restrict__ f, int nx
     real wx, wy;
     warp_axis(x, vx, nx, x0, x1, wx, 0);
     warp_axis(y, vy, ny, y0, y1, wy, 0);
-    const real a = ldg(f + (long long)y0 * nx + x0), b = ldg(f + (long long)y0 * nx + x1);
-    const real c = ldg(f + (long long)y1 * nx + x0), d = ldg(f + (long long)y1 * nx + x1);
+    const real a = ldg(f + (y0 * nx + x0)), b = ldg(f + (y0 * nx + x1));
+    const real c = ldg(f + (y1 * nx + x0)), d = ldg(f + (y1 * nx + x1));
     gx = axis_moves(x, vx, nx) ? (1 - wy) * (b - a) + wy * (d - c) : (real)0;
     gy = axis_moves(y, vy, ny) ? (1 - wx) * (c - a) + wx * (d - b) : (real)0;
 }
@@ -990,7 +1208,22 @@ mof_status launch_flow_linT(const mof_problem *p, const real *ux, const real *uy
 }
 
 // ============================================================ K5 Theta^T W Theta
-// Stage 1: q = W_M (Mhat x), W_M = ((Mhat uk)^2 + eps^2)^(-1/2), per flow row.
+// Stage 1: q = W_M (Mhat x), W_M = ((Mhat uk)^2 + eps^2)^(-1/2), per flow row. Both images are
+// sampled at the same points, whose coordinates and weights are formed once.
+template <typename real>
+__device__ __forceinline__ void flow_row(const real *__restrict__ fx, const real *__restrict__ fk, real cx, real ck, int nx, int ny,
+                                         int x, int y, real vx, real vy, int wm, real eps2, real &q) {
+    int x0, x1, y0, y1;
+    real wx, wy;
+    warp_axis(x, vx, nx, x0, x1, wx, wm);
+    warp_axis(y, vy, ny, y0, y1, wy, wm);
+    const int o00 = y0 * nx + x0, o01 = y0 * nx + x1, o10 = y1 * nx + x0, o11 = y1 * nx + x1;
+    const real ux = 1 - wx, uy = 1 - wy;
+    const real bx = uy * (ux * ldg(fx + o00) + wx * ldg(fx + o01)) + wy * (ux * ldg(fx + o10) + wx * ldg(fx + o11));
+    const real bk = uy * (ux * ldg(fk + o00) + wx * ldg(fk + o01)) + wy * (ux * ldg(fk + o10) + wx * ldg(fk + o11));
+    q = wdiff(cx - bx, ck - bk, eps2);
+}
+
 template <typename real>
 __global__ void k_regn_flow_rows(const real *__restrict__ x, const real *__restrict__ uk, const real *__restrict__ s,
                                  const real *__restrict__ sr, real eps2, real *__restrict__ q, int nx, int ny, int np,
@@ -999,14 +1232,12 @@ __global__ void k_regn_flow_rows(const real *__restrict__ x, const real *__restr
     if (xx >= nx || y >= ny) return;
     const long long ns = (long long)nx * ny, i = (long long)y * nx + xx;
     const real *sp = s + 2LL * p * ns, *srp = sr + 2LL * p * ns;
-    const real svx = sp[i], svy = sp[ns + i], rvx = srp[i], rvy = srp[ns + i];
     const real *x0 = x + p * ns, *x1 = x0 + ns, *k0 = uk + p * ns, *k1 = k0 + ns;
-    const real fx = x0[i] - bilinear(x1, nx, ny, xx, y, svx, svy, wm);
-    const real fk = k0[i] - bilinear(k1, nx, ny, xx, y, svx, svy, wm);
-    const real bx = x1[i] - bilinear(x0, nx, ny, xx, y, rvx, rvy, wm);
-    const real bk = k1[i] - bilinear(k0, nx, ny, xx, y, rvx, rvy, wm);
-    q[p * ns + i] = fx / sqrt(fk * fk + eps2);
-    q[(np + p) * ns + i] = bx / sqrt(bk * bk + eps2);
+    real a, b;
+    flow_row(x1, k1, x0[i], k0[i], nx, ny, xx, y, sp[i], sp[ns + i], wm, eps2, a);
+    flow_row(x0, k0, x1[i], k1[i], nx, ny, xx, y, srp[i], srp[ns + i], wm, eps2, b);
+    q[p * ns + i] = a;
+    q[(np + p) * ns + i] = b;
 }
 
 // Stage 2: y = y_add + scale * lam * (Psi^T W_Psi Psi x [+ L_t^T W_t L_t x] + Mhat^T q), the
