@@ -540,11 +540,12 @@ mof_status mof_reverse_flow(mof_problem *p, const void *s, void *sr, void *strea
     g_err[0] = 0;
     MOF_TRY(check_problem(p));
     if (!s || !sr) return fail(MOF_EINVAL, "null array");
-    void *rad = nullptr, *dest = nullptr;
+    void *rad = nullptr;
     MOF_TRY(apply_scratch(p, SCR_RADIUS, &rad));
+    if (p->precision != MOF_FP64) return launch_reverse_flow<float>(p, CF(s), (int *)rad, nullptr, F(sr), S(stream));
+    void *dest = nullptr;
     MOF_TRY(apply_scratch(p, SCR_DEST, &dest));
-    if (p->precision == MOF_FP64) return launch_reverse_flow<double>(p, CD(s), (int *)rad, (int *)dest, D(sr), S(stream));
-    return launch_reverse_flow<float>(p, CF(s), (int *)rad, (int *)dest, F(sr), S(stream));
+    return launch_reverse_flow<double>(p, CD(s), (int *)rad, (int *)dest, D(sr), S(stream));
 }
 
 mof_status mof_apply_reg_normal(mof_problem *p, const void *x, const void *uk, const void *s, const void *sr, double eps,

@@ -154,6 +154,7 @@ template <typename real> mof_status launch_downsample(const mof_problem *p, int 
 template <typename real> mof_status launch_upsample_velocity(const mof_problem *p, int a, const real *sc, real *s, cudaStream_t st);
 template <typename real> mof_status launch_flow_lin(const mof_problem *p, const real *ux, const real *uy, const real *ut, const real *s, real *r, cudaStream_t st);
 template <typename real> mof_status launch_flow_linT(const mof_problem *p, const real *ux, const real *uy, const real *r, real *gs, cudaStream_t st);
+// dest_scratch: (nt - 1) ns ints in FP64 (null in FP32)
 template <typename real> mof_status launch_reverse_flow(const mof_problem *p, const real *s, int *bnd_scratch, int *dest_scratch, real *sr, cudaStream_t st);
 // Weighted regulariser normal operator: y = y_add + scale * Theta^T W Theta x,
 // W from uk; q_scratch holds 2*(nt-1)*ns weighted flow rows. lam_dev (may be

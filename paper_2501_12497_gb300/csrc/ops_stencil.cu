@@ -102,6 +102,14 @@ __device__ __forceinline__ int round_axis(int x, real v, int n) {
     return I < 0 ? 0 : (I > n - 1 ? n - 1 : I);
 }
 
+// FP32 form, as warp_axis
+__device__ __forceinline__ int round_axis(int x, float v, int n) {
+    const float vc = v == v ? fminf(fmaxf(v, -8192.f), 8192.f) : 0.f;
+    const float t = __fadd_rd(vc, FLOOR_MAGIC), fr = vc - (t - FLOOR_MAGIC);
+    const int I = x + (__float_as_int(t) - FLOOR_BITS);
+    return min(max(I + (I >= 0 ? fr >= 0.5f : fr > 0.5f), 0), n - 1);
+}
+
 // ---------------------------------------------------------------- tiles of the transposes
 // The warp transposes (Mhat^T, the flow part of Theta^T W Theta) and the reverse flow
 // work on BW x BH pixel tiles, one CTA of BT threads per tile (BPT pixels per thread).
@@ -357,7 +365,7 @@ __global__ void k_zero_reach(int *__restrict__ bnd_a, int *__restrict__ bnd_b, i
 // Bounds of one source tile of velocity field f (fields f < nf from va, the next nf
 // from vb): {min, max} over its pixels p of x0(p) - px and y0(p) - py, with x0, y0 the
 // first pixel of the bilinear footprint {x0, x0 or x0 + 1} of M(v) (MODE 0), or the
-// reverse flow's destination (MODE 1, which also stores it in dest). The field's reach
+// reverse flow's destination (MODE 1, stored in dest where that is given). The field's reach
 // max(-min, max + 1) (MODE 0; max(-min, max) in MODE 1) is raised with one integer
 // atomicMax per tile and axis (exact and order independent).
 template <typename real, int MODE>
@@ -386,7 +394,7 @@ __global__ void __launch_bounds__(BT) k_src_bounds(const real *__restrict__ va, 
             dy = y0 - y;
         } else {
             const int qx = round_axis(x, vx[i], nx), qy = round_axis(y, vy[i], ny);
-            dest[(long long)f * ns + i] = qy * nx + qx;
+            if (dest) dest[(long long)f * ns + i] = qy * nx + qx;
             dx = qx - x;
             dy = qy - y;
         }
@@ -950,9 +958,55 @@ __global__ void k_flow_ds(const real *__restrict__ u, const real *__restrict__ s
     gsr[(2 * t + 1) * ns + i] = -g1 * gy;
 }
 
+// FP32 form of k_flow_ds with four consecutive pixels per thread (16-byte vectors of the
+// streamed arrays, as k_flow4); the same arithmetic per pixel. Bound by DRAM (0.9 of the copy rate):
+// 1024x1024x64 476 us against 566 pixel by pixel.
+__device__ __forceinline__ void slope32(const float *__restrict__ f, int nx, int ny, int x, int y, float vx, float vy, float &gx,
+                                        float &gy) {
+    int x0, x1, y0, y1;
+    float wx, wy;
+    warp_axis(x, vx, nx, x0, x1, wx, 0);
+    warp_axis(y, vy, ny, y0, y1, wy, 0);
+    const float a = ldg(f + (y0 * nx + x0)), b = ldg(f + (y0 * nx + x1)), c = ldg(f + (y1 * nx + x0)), d = ldg(f + (y1 * nx + x1));
+    // the sample moves where its cell is the unclipped one: x + v in [0, n - 1)
+    const float cx = fminf(fmaxf(vx, -8192.f), 8192.f), cy = fminf(fmaxf(vy, -8192.f), 8192.f);
+    const int ix = x + (__float_as_int(__fadd_rd(cx, FLOOR_MAGIC)) - FLOOR_BITS), iy = y + (__float_as_int(__fadd_rd(cy, FLOOR_MAGIC)) - FLOOR_BITS);
+    gx = (unsigned)ix < (unsigned)(nx - 1) && vx == vx ? (1 - wy) * (b - a) + wy * (d - c) : 0.f;
+    gy = (unsigned)iy < (unsigned)(ny - 1) && vy == vy ? (1 - wx) * (c - a) + wx * (d - b) : 0.f;
+}
+__global__ void __launch_bounds__(V4X *V4Y) k_flow_ds4(const float *__restrict__ u, const float *__restrict__ s,
+                                                       const float *__restrict__ sr, const float *__restrict__ gr,
+                                                       float *__restrict__ gs, float *__restrict__ gsr, int nx, int ny, int np) {
+    const int x = 4 * (blockIdx.x * V4X + threadIdx.x), y = blockIdx.y * V4Y + threadIdx.y, t = blockIdx.z;
+    if (x >= nx || y >= ny) return;
+    const long long ns = (long long)nx * ny, i = (long long)y * nx + x, o = 2 * t * ns + i;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const float4 v4x = ldcs4((h ? sr : s) + o), v4y = ldcs4((h ? sr : s) + o + ns), g4 = ldcs4(gr + (h * np + t) * ns + i);
+        const float vx[4] = {v4x.x, v4x.y, v4x.z, v4x.w}, vy[4] = {v4y.x, v4y.y, v4y.z, v4y.w}, g[4] = {g4.x, g4.y, g4.z, g4.w};
+        float ox[4], oy[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            float gx, gy;
+            slope32(u + (t + 1 - h) * ns, nx, ny, x + k, y, vx[k], vy[k], gx, gy);
+            ox[k] = -g[k] * gx;
+            oy[k] = -g[k] * gy;
+        }
+        stcs4((h ? gsr : gs) + o, make_float4(ox[0], ox[1], ox[2], ox[3]));
+        stcs4((h ? gsr : gs) + o + ns, make_float4(oy[0], oy[1], oy[2], oy[3]));
+    }
+}
+
 template <typename real>
 mof_status launch_flow_ds(const mof_problem *p, const real *u, const real *s, const real *sr, const real *gr, real *gs,
                           real *gsr, cudaStream_t st) {
+    if (sizeof(real) == 4 && p->nx % 4 == 0 && !p->warp_mode && al16(u) && al16(s) && al16(sr) && al16(gr) && al16(gs) && al16(gsr)) {
+        ::mof::count_launch(), k_flow_ds4<<<grid4(p->nx, p->ny, p->nt - 1), dim3(V4X, V4Y), 0, st>>>(
+            (const float *)u, (const float *)s, (const float *)sr, (const float *)gr, (float *)gs, (float *)gsr, p->nx, p->ny,
+            p->nt - 1);
+        MOF_LAUNCH_CHECK();
+        return MOF_OK;
+    }
     ::mof::count_launch(), k_flow_ds<real><<<grid2d(p->nx, p->ny, p->nt - 1), dim3(TX, TY), 0, st>>>(u, s, sr, gr, gs, gsr, p->nx,
                                                                                                    p->ny, p->nt - 1, p->warp_mode);
     MOF_LAUNCH_CHECK();
@@ -961,24 +1015,42 @@ mof_status launch_flow_ds(const mof_problem *p, const real *u, const real *s, co
 
 // ============================================================ K6 reverse flow
 // s'(q) = -(mean of s(p) over the sources p with dest(p) = q), dest(p) = round(p + s(p))
-// clipped (k_src_bounds, MODE 1). One CTA per BW x BH destination tile: warp 0 takes the
-// union of the displacement bounds of the source tiles whose destinations can fall into
-// the tile; each pixel then scans the sources of its window in row-major order and sums
-// their velocities in FP64 in that order, so the result is that of a sequential pass over
-// the sources.
+// clipped. One CTA per BW x BH destination tile: its threads run over the sources that can
+// reach the tile (the candidate rectangles of k_src_bounds, MODE 1) and enter each source that
+// lands in the tile into its pixel's list (a shared-memory counter and the first REV_LIST
+// sources); each pixel then averages its sources in row-major order. One or two arrivals in
+// the element type (the mean of one or two values rounds as the FP64 mean does), FP64 sums from
+// the third, so the result is that of a sequential pass over the sources. A pixel with more
+// arrivals than its list (where the flow leaves the frame) scans the window of sources that the
+// tile's displacements allow.
+// FP32 rounds the destinations here; FP64 (whose pipe would bound the pass) takes them from
+// dest, where the bounds kernel stored them.
+// What bounds it: instruction issue and the two passes over the velocities. 1024x1024x64: 730 us
+// with the bounds (bounds 190, tiles 520) against 961 for a scan of every pixel's window of
+// destinations; 256x256x32: 44 against 54 us.
+constexpr int REV_LIST = 4;
 template <typename real>
-__global__ void __launch_bounds__(BT) k_rev_gather(const real *__restrict__ s, const int *__restrict__ dest,
-                                                   const int *__restrict__ bnd, real *__restrict__ sr, int nx, int ny,
-                                                   int tiles) {
+__global__ void __launch_bounds__(BT) k_rev_tile(const real *__restrict__ s, const int *__restrict__ dest, const int *__restrict__ bnd,
+                                                 real *__restrict__ sr, int nx, int ny, int tiles) {
+    __shared__ SrcRect rect[MAXR];
+    __shared__ int sh[4];
     __shared__ int4 ub;
+    __shared__ int s_cnt[BW * BH];
+    __shared__ int s_src[REV_LIST][BW * BH];
     const int p = blockIdx.z, tid = threadIdx.x;
     const int X0 = blockIdx.x * BW, Y0 = blockIdx.y * BH;
     const int X1 = min(X0 + BW - 1, nx - 1), Y1 = min(Y0 + BH - 1, ny - 1);
     const int txn = (nx + BW - 1) / BW, tyn = (ny + BH - 1) / BH;
-    if (tid < 32) {
-        const TermTiles T = term_tiles(bnd + 4LL * p * (tiles + 1), tiles, txn, tyn, X0, X1, Y0, Y1, nx, ny);
+    const long long ns = (long long)nx * ny;
+    const real *sx = s + 2LL * p * ns, *sy = sx + ns;
+    constexpr bool F32 = sizeof(real) == 4;
+    const int *dp = F32 ? nullptr : dest + p * ns;
+    const TermTiles T = term_tiles(bnd + 4LL * p * (tiles + 1), tiles, txn, tyn, X0, X1, Y0, Y1, nx, ny);
+    const TermTiles none{nullptr, 0, 0, 1, 0};
+    for (int l = tid; l < BW * BH; l += BT) s_cnt[l] = 0;
+    if (tid >= 32 && tid < 64) {  // the union of the displacements of the source tiles that can reach the tile
         int dxmin = INT_MAX, dxmax = INT_MIN, dymin = INT_MAX, dymax = INT_MIN;
-        for (int j = tid; j < T.nc; j += 32) {
+        for (int j = tid - 32; j < T.nc; j += 32) {
             const int tx = T.txa + j % T.ntx, ty = T.tya + j / T.ntx;
             const int4 b = __ldg(T.bnd + ty * txn + tx);
             const int S0 = tx * BW, S1 = min(S0 + BW - 1, nx - 1), R0 = ty * BH, R1 = min(R0 + BH - 1, ny - 1);
@@ -994,59 +1066,94 @@ __global__ void __launch_bounds__(BT) k_rev_gather(const real *__restrict__ s, c
         dxmax = __reduce_max_sync(0xffffffffu, dxmax);
         dymin = __reduce_min_sync(0xffffffffu, dymin);
         dymax = __reduce_max_sync(0xffffffffu, dymax);
-        if (tid == 0) ub = make_int4(dxmin, dxmax, dymin, dymax);
+        if (tid == 32) ub = make_int4(dxmin, dxmax, dymin, dymax);
     }
+    int cursor = 0;
+    do {
+        __syncthreads();
+        if (tid < 32) build_rects<1>(T, none, cursor, X0, X1, Y0, Y1, nx, ny, rect, sh);
+        __syncthreads();
+        const int nrect = sh[0], npx = sh[1];
+        cursor = sh[2];
+        int ri = -1, next = 0;
+        constexpr int U = 4;  // sources with their loads in flight
+        for (int k0 = tid; k0 < npx; k0 += U * BT) {
+            float vx[U], vy[U];
+            int px[U], py[U], to[U];
+#pragma unroll
+            for (int e = 0; e < U; ++e) {
+                px[e] = -1;
+                if (k0 + e * BT >= npx) continue;
+                int term;
+                rect_pixel(rect, nrect, k0 + e * BT, ri, next, term, px[e], py[e]);
+                const int i = py[e] * nx + px[e];
+                if constexpr (F32) {
+                    vx[e] = ldg(sx + i);
+                    vy[e] = ldg(sy + i);
+                } else {
+                    to[e] = ldg(dp + i);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < U; ++e) {
+                if (px[e] < 0) continue;
+                int qx, qy;
+                if constexpr (F32) {
+                    qx = round_axis(px[e], vx[e], nx);
+                    qy = round_axis(py[e], vy[e], ny);
+                } else {
+                    qy = to[e] / nx;
+                    qx = to[e] - qy * nx;
+                }
+                if (qx < X0 || qx > X1 || qy < Y0 || qy > Y1) continue;
+                const int l = (qy - Y0) * BW + qx - X0, c = atomicAdd(&s_cnt[l], 1);
+                if (c < REV_LIST) s_src[c][l] = py[e] * nx + px[e];
+            }
+        }
+    } while (cursor < T.nc);
     __syncthreads();
-    const int4 bd = ub;
-    const long long ns = (long long)nx * ny;
-    const real *sx = s + 2LL * p * ns, *sy = sx + ns;
-    const int *dp = dest + p * ns;
     real *rx = sr + 2LL * p * ns, *ry = rx + ns;
 #pragma unroll
     for (int k = 0; k < BPT; ++k) {
         const int l = tid + k * BT, x = X0 + (l % BW), y = Y0 + l / BW;
         if (x > X1 || y > Y1) continue;
-        const long long q = (long long)y * nx + x;
-        // the first two arrivals in the element type, FP64 sums from the third: the mean of
-        // one or two values (x, or (x0 + x1) / 2 with an exact halving) rounds as the FP64
-        // mean does, so FP64 work is left to the pixels where three or more sources collide
-        real a0 = 0, a1 = 0, b0 = 0, b1 = 0;
-        double ax = 0.0, ay = 0.0;
-        int cnt = 0;
-        if (bd.x <= bd.y) {  // some source tile can reach this tile
-            const int ylo = max(0, y - bd.w), yhi = min(ny - 1, y - bd.z);
-            const int xlo = max(0, x - bd.y), xhi = min(nx - 1, x - bd.x);
-            for (int py = ylo; py <= yhi; ++py)
-                for (int px = xlo; px <= xhi; ++px) {
-                    const long long i = (long long)py * nx + px;
-                    if (ldg(dp + i) == (int)q) {
+        const int q = y * nx + x, cnt = s_cnt[l];
+        real ox = 0, oy = 0;
+        if (cnt == 1) {
+            const int i = s_src[0][l];
+            ox = -ldg(sx + i);
+            oy = -ldg(sy + i);
+        } else if (cnt == 2) {
+            const int i = s_src[0][l], j = s_src[1][l];
+            ox = -((ldg(sx + i) + ldg(sx + j)) * (real)0.5);
+            oy = -((ldg(sy + i) + ldg(sy + j)) * (real)0.5);
+        } else if (cnt > 2) {
+            double ax = 0.0, ay = 0.0;
+            if (cnt <= REV_LIST) {  // in source order: the smallest source beyond the last one taken
+                int last = -1;
+                for (int c = 0; c < cnt; ++c) {
+                    int i = INT_MAX;
+#pragma unroll
+                    for (int e = 0; e < REV_LIST; ++e) {
+                        const int v = e < cnt ? s_src[e][l] : INT_MAX;
+                        i = v > last ? min(i, v) : i;
+                    }
+                    ax += (double)ldg(sx + i);
+                    ay += (double)ldg(sy + i);
+                    last = i;
+                }
+            } else {
+                const int4 bd = ub;
+                for (int py = max(0, y - bd.w); py <= min(ny - 1, y - bd.z); ++py)
+                    for (int px = max(0, x - bd.y); px <= min(nx - 1, x - bd.x); ++px) {
+                        const int i = py * nx + px;
                         const real vx = ldg(sx + i), vy = ldg(sy + i);
-                        if (cnt == 0) {
-                            a0 = vx;
-                            b0 = vy;
-                        } else if (cnt == 1) {
-                            a1 = vx;
-                            b1 = vy;
-                        } else {
-                            if (cnt == 2) {  // in source order, as a sequential FP64 sum
-                                ax = (double)a0 + (double)a1;
-                                ay = (double)b0 + (double)b1;
-                            }
+                        if (F32 ? round_axis(px, vx, nx) == x && round_axis(py, vy, ny) == y : ldg(dp + i) == q) {
                             ax += (double)vx;
                             ay += (double)vy;
                         }
-                        ++cnt;
                     }
-                }
-        }
-        real ox = 0, oy = 0;
-        if (cnt == 1) {
-            ox = -a0;
-            oy = -b0;
-        } else if (cnt == 2) {
-            ox = -((a0 + a1) * (real)0.5);
-            oy = -((b0 + b1) * (real)0.5);
-        } else if (cnt > 2) {
+            }
             ox = (real)(-ax / cnt);
             oy = (real)(-ay / cnt);
         }
@@ -1064,7 +1171,7 @@ mof_status launch_reverse_flow(const mof_problem *p, const real *s, int *bnd, in
     ::mof::count_launch(), k_src_bounds<real, 1><<<grid_tiles(p, np), BT, 0, st>>>(s, s, np, p->nx, p->ny, 0, bnd, bnd,
                                                                                   tiles_x(p), tiles, dest);
     MOF_LAUNCH_CHECK();
-    ::mof::count_launch(), k_rev_gather<real><<<grid_tiles(p, np), BT, 0, st>>>(s, dest, bnd, sr, p->nx, p->ny, tiles);
+    ::mof::count_launch(), k_rev_tile<real><<<grid_tiles(p, np), BT, 0, st>>>(s, dest, bnd, sr, p->nx, p->ny, tiles);
     MOF_LAUNCH_CHECK();
     return MOF_OK;
 }
@@ -1104,7 +1211,115 @@ __global__ void k_of_fields(const real *__restrict__ u, int dr, real *__restrict
     ut[i] = st / (box * box);
 }
 
-// The same fields from shared-memory tiles: a CTA owns a 32 x 8 tile of every pair and
+// dr = 1 without shared memory: a warp takes 32 V consecutive columns of one pair and marches
+// down `rows` rows, with the rows y - 1, y, y + 1 of the image and of u_{p+1} - u_p in registers; the
+// neighbours of a lane's V columns come from the adjacent lanes. Each image row is read twice
+// (as frame p and as frame p + 1 of pair p - 1, the second time from L2) plus two halo rows per strip.
+// ux and uy take their terms in the order of k_of_fields; ut sums three differences per row,
+// then three rows. V = 4 needs rows of a multiple of 4 pixels and 16-byte aligned arrays.
+// What bounds it: DRAM (62 % of the copy rate with the first pass over u in the count). 1024x1024x64:
+// 250 us against 461 for shared-memory tiles that walk the frames in order; 256x256x32: 17 against
+// 52 us; 181x149x9: 9 against 17 us.
+constexpr int FW = 4;  // warps per CTA
+template <typename real, int V>
+__global__ void __launch_bounds__(32 * FW) k_of_fields_rows(const real *__restrict__ u, real *__restrict__ ux,
+                                                            real *__restrict__ uy, real *__restrict__ ut, int nx, int ny,
+                                                            int rows) {
+    const int lane = threadIdx.x, p = blockIdx.z;
+    const int x = (blockIdx.x * 32 + lane) * V, y0 = (blockIdx.y * FW + threadIdx.y) * rows;
+    if (y0 >= ny) return;  // whole warps
+    const bool on = x < nx;
+    const int xc = on ? x : nx - V;
+    const long long ns = (long long)nx * ny;
+    const real *a = u + p * ns, *b = a + ns;
+    const real half = (real)0.5, three = (real)3;
+    // row yy of the image (with its left and right neighbours) and of the difference
+    auto load = [&](int yy, real (&f)[V + 2], real (&d)[V + 2]) {
+        const int i = min(max(yy, 0), ny - 1) * nx + xc;
+        real g[V + 2];
+        if constexpr (V == 4 && sizeof(real) == 4) {
+            const float4 q = ld4(a + i), r = ld4(b + i);
+            f[1] = q.x; f[2] = q.y; f[3] = q.z; f[4] = q.w;
+            g[1] = r.x; g[2] = r.y; g[3] = r.z; g[4] = r.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+                f[k + 1] = a[i + k];
+                g[k + 1] = b[i + k];
+            }
+        }
+        f[0] = __shfl_up_sync(0xffffffffu, f[V], 1);
+        g[0] = __shfl_up_sync(0xffffffffu, g[V], 1);
+        f[V + 1] = __shfl_down_sync(0xffffffffu, f[1], 1);
+        g[V + 1] = __shfl_down_sync(0xffffffffu, g[1], 1);
+        if (lane == 0 && xc > 0) {
+            f[0] = a[i - 1];
+            g[0] = b[i - 1];
+        }
+        if (lane == 31 && xc + V < nx) {
+            f[V + 1] = a[i + V];
+            g[V + 1] = b[i + V];
+        }
+        if (xc == 0) {  // reflected about the edge
+            f[0] = f[1];
+            g[0] = g[1];
+        }
+        if (xc + V >= nx) {
+            f[V + 1] = f[V];
+            g[V + 1] = g[V];
+        }
+#pragma unroll
+        for (int k = 0; k < V + 2; ++k) d[k] = g[k] - f[k];
+    };
+    real f0[V + 2], f1[V + 2], f2[V + 2], d[V + 2], s0[V], s1[V], s2[V];
+    auto sum3 = [&](real (&o)[V]) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) o[k] = d[k] + d[k + 1] + d[k + 2];
+    };
+    load(y0 - 1, f0, d);
+    sum3(s0);
+    load(y0, f1, d);
+    sum3(s1);
+    const int ye = min(y0 + rows, ny);
+    for (int y = y0; y < ye; ++y) {
+        load(y + 1, f2, d);
+        sum3(s2);
+        real gx[V], gy[V], gt[V];
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            gx[k] = ((f0[k + 2] - f0[k]) * half + (f1[k + 2] - f1[k]) * half + (f2[k + 2] - f2[k]) * half) / three;
+            gy[k] = ((f2[k] - f0[k]) * half + (f2[k + 1] - f0[k + 1]) * half + (f2[k + 2] - f0[k + 2]) * half) / three;
+            gt[k] = (s0[k] + s1[k] + s2[k]) / (three * three);
+        }
+        if (on) {
+            const long long o = p * ns + (long long)y * nx + x;
+            if constexpr (V == 4 && sizeof(real) == 4) {
+                st4(ux + o, make_float4(gx[0], gx[1], gx[2], gx[3]));
+                st4(uy + o, make_float4(gy[0], gy[1], gy[2], gy[3]));
+                st4(ut + o, make_float4(gt[0], gt[1], gt[2], gt[3]));
+            } else {
+#pragma unroll
+                for (int k = 0; k < V; ++k) {
+                    ux[o + k] = gx[k];
+                    uy[o + k] = gy[k];
+                    ut[o + k] = gt[k];
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < V + 2; ++k) {
+            f0[k] = f1[k];
+            f1[k] = f2[k];
+        }
+#pragma unroll
+        for (int k = 0; k < V; ++k) {
+            s0[k] = s1[k];
+            s1[k] = s2[k];
+        }
+    }
+}
+
+// dr = 2 from shared-memory tiles: a CTA owns a 32 x 8 tile of every pair and
 // walks the frames in order, so each frame's tile (with its reflected halo of DR pixels)
 // is loaded once and serves as frame t + 1 of pair t and frame t of pair t + 1; the sums
 // take the terms in the order of k_of_fields (identical results).
@@ -1157,9 +1372,20 @@ mof_status launch_of_fields(const mof_problem *p, const real *u, int dr, real *u
     const int np = p->nt - 1;
     if (np <= 0) return MOF_OK;
     // each halo element is the reflected pixel of its own coordinate, as in k_of_fields
-    if (dr == 1)
-        ::mof::count_launch(), k_of_fields_tiled<real, 1><<<dim3((p->nx + TX - 1) / TX, (p->ny + TY - 1) / TY), dim3(TX, TY), 0, st>>>(
-            u, ux, uy, ut, p->nx, p->ny, np);
+    if (dr == 1) {
+        const bool vec = sizeof(real) == 4 && p->nx % 4 == 0 && al16(u) && al16(ux) && al16(uy) && al16(ut);
+        const int gx = (p->nx + (vec ? 127 : 31)) / (vec ? 128 : 32);
+        // strips of 16 rows (two halo rows each) where they give every SM 16 warps, else of 4 or 2
+        // (256x256x32: 17 us with 4 rows, 33 with 16; 181x149x9: 9 and 19)
+        int rows = 16;
+        while (rows > 2 && (long long)gx * np * ((p->ny + rows - 1) / rows) < 152LL * 16) rows = rows == 16 ? 4 : 2;
+        const dim3 grid(gx, (p->ny + FW * rows - 1) / (FW * rows), np), tb(32, FW);
+        ::mof::count_launch();
+        if (vec)
+            k_of_fields_rows<float, 4><<<grid, tb, 0, st>>>((const float *)u, (float *)ux, (float *)uy, (float *)ut, p->nx, p->ny, rows);
+        else
+            k_of_fields_rows<real, 1><<<grid, tb, 0, st>>>(u, ux, uy, ut, p->nx, p->ny, rows);
+    }
     else if (dr == 2)
         ::mof::count_launch(), k_of_fields_tiled<real, 2><<<dim3((p->nx + TX - 1) / TX, (p->ny + TY - 1) / TY), dim3(TX, TY), 0, st>>>(
             u, ux, uy, ut, p->nx, p->ny, np);

@@ -351,7 +351,8 @@ static mof_status ensure_ws(mof_problem *p, const mof_solver_params &prm, int n_
         w->rad_s = a.take<int>(bints);
         w->rad_sr = a.take<int>(bints);
         w->rad_rev = a.take<int>(bints);
-        w->dest = a.take<int>(P * ns);
+        w->dest = a.take<int>(sizeof(real) == 8 ? P * ns : 0);  // reverse-flow destinations (FP64)
+        if (sizeof(real) == 4) w->dest = nullptr;
         w->GH = a.take<double>((size_t)Kmax * Kmax);
         w->GT = a.take<double>((size_t)Kmax * Kmax);
         w->gH = a.take<double>(Kmax);
