@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(SDT) k_sub_dot(const real *__restrict__ V, lon
 // r and q and Ups^T b, the two 1 KB segments of those pixels, and the segments of u_x and u_y,
 // completing on one mbarrier (bounded wait). The chunk partials (3 Kmax + 4 per chunk,
 // FP32 16-element partials accumulated with their rounding errors, FP64 across lanes) are
-// reduced by k_of_pass_reduce. With x' = r - V d the new vector is v = x' / ||x'|| and its Gram
+// reduced by k_of_pass_finish. With x' = r - V d the new vector is v = x' / ||x'|| and its Gram
 // column follows from these without another pass over the basis (k_of_pass_finish):
 //   G_A[i][v] = (V^T y)_i / ||x'||,   G_L[i][v] = ((V^T q)_i - (G_L d)_i) / ||x'||,
 //   g[v] = x'^T Ups^T b / ||x'||,     G_A[v][v] = x'^T y / ||x'||^2,
@@ -409,10 +409,10 @@ long long of_pass_chunks(long long ns, int elem_bytes) { return (ns * elem_bytes
 int of_pass_stride(int Kmax) { return 3 * Kmax + 4; }
 
 template <typename real>
-__global__ void __launch_bounds__(OP_T) k_of_proj_gram_pass(const real *__restrict__ V, long long ns, int Kmax,
+__global__ void __launch_bounds__(OP_T) k_of_proj_gram_pass(const real *V, long long ns, int Kmax,
                                                            const int *__restrict__ K, const int *__restrict__ act,
-                                                           const double *__restrict__ d, real *x, const real *__restrict__ q,
-                                                           const real *__restrict__ AtB, const real *__restrict__ ux,
+                                                           const double *__restrict__ d, const real *__restrict__ x,
+                                                           const real *__restrict__ q, real *to, const real *__restrict__ AtB, const real *__restrict__ ux,
                                                            const real *__restrict__ uy, double *__restrict__ partial,
                                                            int nchunk, int *__restrict__ err, int kcap) {
     constexpr int PX = opx<real>(), CH = 2 * PX;  // elements of one vector in the tile
@@ -485,13 +485,16 @@ __global__ void __launch_bounds__(OP_T) k_of_proj_gram_pass(const real *__restri
 #pragma unroll
         for (int e = 0; e < EPT; ++e) xx[e] = (pix0 + e < len) ? xx[e] - acc[e] : (real)0;
         *reinterpret_cast<vec_t *>(sx + i0) = xv;
-        real *ob = x + b * 2 * ns + (i0 < PX ? 0 : ns) + p0 + pix0;
-        if (pix0 + EPT <= len) {
-            *reinterpret_cast<vec_t *>(ob) = xv;
-        } else {
+        // into the slot behind the basis, where an append finds it (a full basis appends nothing)
+        if (K[b] < Kmax) {
+            real *ob = to + ((long long)b * Kmax + Kb) * 2 * ns + (i0 < PX ? 0 : ns) + p0 + pix0;
+            if (pix0 + EPT <= len) {
+                *reinterpret_cast<vec_t *>(ob) = xv;
+            } else {
 #pragma unroll
-            for (int e = 0; e < EPT; ++e)
-                if (pix0 + e < len) ob[e] = xx[e];
+                for (int e = 0; e < EPT; ++e)
+                    if (pix0 + e < len) ob[e] = xx[e];
+            }
         }
     }
     __syncthreads();
@@ -578,25 +581,6 @@ __global__ void __launch_bounds__(OP_T) k_of_proj_gram_pass(const real *__restri
             out[(long long)(2 * Kmax + j) * nchunk] = o3;
         }
     }
-}
-
-// sums of the chunk partials of k_of_proj_gram_pass in FP64 (one warp per output, lanes over
-// its contiguous chunks, fixed order): res[b][0..3 Kmax + 4)
-__global__ void k_of_pass_reduce(const double *__restrict__ partial, int nchunk, int Kmax, const int *__restrict__ K,
-                                 const int *__restrict__ act, double *__restrict__ res) {
-    const int b = blockIdx.y;
-    if (act && !act[b]) return;
-    const int stride = 3 * Kmax + 4, Kb = min(K[b], Kmax);
-    const int o = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (o >= stride) return;
-    const int j = o < 3 * Kmax ? o % Kmax : 0;
-    if (o < 3 * Kmax && j >= Kb) return;
-    const double *src = partial + ((long long)b * stride + o) * nchunk;
-    double sum = 0.0;
-#pragma unroll 8
-    for (int c = lane; c < nchunk; c += 32) sum += src[c];
-    sum = warp_sum(sum);
-    if (lane == 0) res[(long long)b * stride + o] = sum;
 }
 
 // ||x[b]||^2 per chunk
@@ -921,47 +905,74 @@ void Krylov<real>::append(const BasisRef<real> &B, int *Kmut, const real *x, lon
     ::mof::count_launch(), k_append<real><<<dim3(blocks, B.B), KT, 0, st>>>(B.V, B.N, B.Kmax, slot, inv, x, xstride, stage);
 }
 
-// Per pair (one warp): the append decision on ||x'|| (as k_append_prep), and for an appended
-// vector v = x' / ||x'||, its Gram columns G_A, G_L, g, its Euclidean overlaps Mg and the slot
-// and scale of k_append (see k_of_proj_gram_pass for the formulas).
+// The chunk partials of k_of_proj_gram_pass summed in FP64 (one warp per output, lanes over its
+// contiguous chunks, fixed order): res[b][0..3 Kmax + 4). The last CTA of a pair to finish
+// (counter done[b], left at zero) takes the append decision on ||x'|| (as k_append_prep) and
+// writes, for an appended vector v = x' / ||x'||, its Gram columns G_A, G_L, g, its Euclidean
+// overlaps Mg, and its slot and scale for k_of_combine (see k_of_proj_gram_pass for the formulas).
+constexpr int PF_T = 256;
 template <typename real>
-__global__ void k_of_pass_finish(const double *__restrict__ res, const double *__restrict__ d, int Kmax, int *__restrict__ K,
-                                 const int *__restrict__ act, const double *__restrict__ scale, double tol,
-                                 int *__restrict__ grow, double *__restrict__ GA, double *__restrict__ GL,
-                                 double *__restrict__ g, double *__restrict__ Mg, double *__restrict__ nrm2_out,
-                                 int *__restrict__ appended, int *__restrict__ slot, real *__restrict__ inv) {
-    const int b = blockIdx.x, lane = threadIdx.x;
+__global__ void __launch_bounds__(PF_T) k_of_pass_finish(const double *__restrict__ partial, int nchunk, double *res,
+                                                         const double *__restrict__ d, int Kmax, int *__restrict__ K,
+                                                         const int *__restrict__ act, const double *__restrict__ scale, double tol,
+                                                         int *__restrict__ grow, double *GA, double *GL, double *g, double *Mg,
+                                                         double *__restrict__ nrm2_out, int *__restrict__ appended,
+                                                         int *__restrict__ slot, real *__restrict__ inv, int *done) {
+    __shared__ double s_gd[64], s_sum[2];
+    __shared__ int s_last;
+    const int b = blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (act && !act[b]) {
-        if (lane == 0) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
             slot[b] = -1;
             if (appended) appended[b] = 0;
         }
         return;
     }
     const int stride = 3 * Kmax + 4, Kb = min(K[b], Kmax);
-    const double *rs = res + (long long)b * stride;
-    const double *c2 = rs, *ay = rs + Kmax, *aq = rs + 2 * Kmax, *sc = rs + 3 * Kmax;
+    double *rs = res + (long long)b * stride;
+    const int o = blockIdx.x * (PF_T / 32) + w;
+    if (o < stride && (o >= 3 * Kmax || o % Kmax < Kb)) {
+        const double *src = partial + ((long long)b * stride + o) * nchunk;
+        double sum = 0.0;
+#pragma unroll 8
+        for (int c = lane; c < nchunk; c += 32) sum += src[c];
+        sum = warp_sum(sum);
+        if (lane == 0) rs[o] = sum;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(done + b, 1) == (int)gridDim.x - 1;
+        if (s_last) done[b] = 0;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const volatile double *c2 = rs, *ay = rs + Kmax, *aq = rs + 2 * Kmax, *sc = rs + 3 * Kmax;
     const double *db = d + (long long)b * Kmax;
     const long long KK = (long long)Kmax * Kmax;
     double *A = GA + b * KK, *L = GL + b * KK, *M = Mg + b * KK;
     const double nr2 = sc[0];
     const bool ok = append_ok(grow[b], Kb, Kmax, nr2, scale, b, tol);
-    // (G_L d)_i and d^T (V^T q) - d^T G_L d for the new column of G_L
-    double dq = 0.0, dGd = 0.0;
-    for (int i = lane; i < Kb; i += 32) {
+    // (G_L d)_i (one warp per row), then d^T (V^T q) and d^T G_L d for the new column of G_L
+    for (int i = w; i < Kb; i += PF_T / 32) {
         double gd = 0.0;
-        for (int k = 0; k < Kb; ++k) gd += L[(long long)i * Kmax + k] * db[k];
-        dq += db[i] * aq[i];
-        dGd += db[i] * gd;
+        for (int k = lane; k < Kb; k += 32) gd += L[(long long)i * Kmax + k] * db[k];
+        gd = warp_sum(gd);
+        if (lane == 0) s_gd[i] = gd;
     }
-    dq = warp_sum(dq);
-    dGd = warp_sum(dGd);
+    __syncthreads();
+    if (w < 2) {
+        double t = 0.0;
+        for (int i = lane; i < Kb; i += 32) t += db[i] * (w == 0 ? aq[i] : s_gd[i]);
+        t = warp_sum(t);
+        if (lane == 0) s_sum[w] = t;
+    }
+    __syncthreads();
+    const double ib = 1.0 / sqrt(nr2), ib2 = 1.0 / nr2;
     if (ok) {
-        const double ib = 1.0 / sqrt(nr2), ib2 = 1.0 / nr2;
-        for (int i = lane; i < Kb; i += 32) {
-            double gd = 0.0;
-            for (int k = 0; k < Kb; ++k) gd += L[(long long)i * Kmax + k] * db[k];
-            const double va = ay[i] * ib, vl = (aq[i] - gd) * ib, vm = c2[i] * ib;
+        for (int i = threadIdx.x; i < Kb; i += PF_T) {
+            const double va = ay[i] * ib, vl = (aq[i] - s_gd[i]) * ib, vm = c2[i] * ib;
             A[(long long)i * Kmax + Kb] = va;
             A[(long long)Kb * Kmax + i] = va;
             L[(long long)i * Kmax + Kb] = vl;
@@ -969,41 +980,148 @@ __global__ void k_of_pass_finish(const double *__restrict__ res, const double *_
             M[(long long)i * Kmax + Kb] = vm;
             M[(long long)Kb * Kmax + i] = vm;
         }
-        __syncwarp();
-        if (lane == 0) {
+        if (threadIdx.x == 0) {
             A[(long long)Kb * Kmax + Kb] = sc[1] * ib2;
-            L[(long long)Kb * Kmax + Kb] = (sc[2] - dq + dGd) * ib2;
+            L[(long long)Kb * Kmax + Kb] = (sc[2] - s_sum[0] + s_sum[1]) * ib2;
             M[(long long)Kb * Kmax + Kb] = 1.0;
             g[(long long)b * Kmax + Kb] = sc[3] * ib;
         }
     }
-    if (lane == 0) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
         nrm2_out[b] = nr2;
         slot[b] = ok ? Kb : -1;
-        inv[b] = ok ? (real)(1.0 / sqrt(nr2)) : (real)0;
+        inv[b] = ok ? (real)ib : (real)0;
         if (ok) K[b] = Kb + 1;
         else grow[b] = 0;
         if (appended) appended[b] = ok;
     }
 }
 
-// q[b] = L^T L r[b] on both components (the graph Laplacian with free boundary, one thread
-// per pixel and component)
+// s[b] = sum_j V[b][j] z[b][j] for Solve-OF, with the scale of a vector appended by
+// k_of_pass_finish: slot[b] (-1: none) holds x' still, which becomes x' inv[b] here on its way
+// through (one pass over the vector less than a separate append). 16 bytes per thread.
 template <typename real>
-__global__ void k_of_lap(const real *__restrict__ r, real *__restrict__ q, int nx, int ny, const int *__restrict__ act) {
-    const int b = blockIdx.z >> 1, c = blockIdx.z & 1;
-    if (act && !act[b]) return;
-    const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
-    if (x >= nx || y >= ny) return;
-    const long long ns = (long long)nx * ny, i = (long long)y * nx + x;
-    const real *f = r + (2LL * b + c) * ns;
-    const real v0 = f[i];
+__global__ void __launch_bounds__(CT) k_of_combine(real *__restrict__ V, long long N, int Kmax, const int *__restrict__ K,
+                                                   const double *__restrict__ z, const int *__restrict__ slot,
+                                                   const real *__restrict__ inv, real *__restrict__ out) {
+    using vec_t = typename std::conditional<sizeof(real) == 4, float4, double2>::type;
+    constexpr int EPT = 16 / sizeof(real);
+    __shared__ real sc[64];
+    const int b = blockIdx.y, Kb = min(K[b], Kmax), sl = slot[b];
+    for (int j = threadIdx.x; j < Kb; j += CT) sc[j] = (real)z[(long long)b * Kmax + j];
+    __syncthreads();
+    const long long i = ((long long)blockIdx.x * CT + threadIdx.x) * EPT;
+    if (i >= N) return;
+    real *Vb = V + (long long)b * Kmax * N + i;
+    real acc[EPT];
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) acc[e] = 0;
+    const int Kd = sl >= 0 ? Kb - 1 : Kb;  // a new vector is the last one
+    int j = 0;
+    for (; j + 3 < Kd; j += 4) {
+        vec_t q[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) q[c] = __ldcs(reinterpret_cast<const vec_t *>(Vb + (long long)(j + c) * N));
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int e = 0; e < EPT; ++e) acc[e] += reinterpret_cast<const real *>(&q[c])[e] * sc[j + c];
+    }
+    for (; j < Kd; ++j) {
+        const vec_t q = __ldcs(reinterpret_cast<const vec_t *>(Vb + (long long)j * N));
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) acc[e] += reinterpret_cast<const real *>(&q)[e] * sc[j];
+    }
+    if (sl >= 0) {
+        const real iv = inv[b];
+        vec_t q = *reinterpret_cast<const vec_t *>(Vb + (long long)Kd * N);
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) {
+            real &v = reinterpret_cast<real *>(&q)[e];
+            v *= iv;
+            acc[e] += v * sc[Kd];
+        }
+        *reinterpret_cast<vec_t *>(Vb + (long long)Kd * N) = q;
+    }
+    *reinterpret_cast<vec_t *>(out + (long long)b * N + i) = *reinterpret_cast<vec_t *>(acc);
+}
+
+template <typename real>
+mof_status launch_of_combine(const BasisRef<real> &B, const double *z, double *aux, real *out, cudaStream_t st) {
+    const int *slot = reinterpret_cast<const int *>(aux);
+    const real *inv = reinterpret_cast<const real *>(aux + B.B);
+    const long long per = CT * (16 / (int)sizeof(real));
+    ::mof::count_launch(), k_of_combine<real><<<dim3((unsigned)((B.N + per - 1) / per), B.B), CT, 0, st>>>(B.V, B.N, B.Kmax, B.K, z, slot,
+                                                                                                      inv, out);
+    MOF_LAUNCH_CHECK();
+    return MOF_OK;
+}
+
+// r = Ups^T Ups s - Ups^T b + gamma (L(+)L)^T (L(+)L) s (the normal-equation residual of Alg. 2)
+// and q = L^T L r on both components (graph Laplacians with free boundary) in one pass: a CTA
+// forms r on its 32 x 8 tile and a border of one pixel from s with a border of two.
+template <typename real>
+__device__ __forceinline__ real lap5(real c, bool l, real fl, bool r, real fr, bool u, real fu, bool d, real fd) {
     real v = 0;
-    if (x > 0) v += v0 - f[i - 1];
-    if (x < nx - 1) v += v0 - f[i + 1];
-    if (y > 0) v += v0 - f[i - nx];
-    if (y < ny - 1) v += v0 - f[i + nx];
-    q[(2LL * b + c) * ns + i] = v;
+    if (l) v += c - fl;
+    if (r) v += c - fr;
+    if (u) v += c - fu;
+    if (d) v += c - fd;
+    return v;
+}
+template <typename real>
+__global__ void __launch_bounds__(256) k_of_resid_lap(const real *__restrict__ ux, const real *__restrict__ uy,
+                                                      const real *__restrict__ AtB, const real *__restrict__ s,
+                                                      const double *__restrict__ gam, real *__restrict__ r, real *__restrict__ q,
+                                                      int nx, int ny, const int *__restrict__ act) {
+    constexpr int W = 32, H = 8;
+    __shared__ real S[2][H + 4][W + 4], R[2][H + 2][W + 2];
+    __shared__ real s_g;
+    const int b = blockIdx.z;
+    if (!act[b]) return;
+    const int x0 = blockIdx.x * W, y0 = blockIdx.y * H, tid = threadIdx.y * W + threadIdx.x;
+    const long long ns = (long long)nx * ny;
+    const real *sb = s + b * 2 * ns;
+    if (tid == 0) s_g = (real)gam[b];
+    for (int e = tid; e < 2 * (H + 4) * (W + 4); e += 256) {
+        const int c = e / ((H + 4) * (W + 4)), m = e - c * (H + 4) * (W + 4), ly = m / (W + 4), lx = m - ly * (W + 4);
+        const int x = x0 + lx - 2, y = y0 + ly - 2;
+        S[c][ly][lx] = (x >= 0 && x < nx && y >= 0 && y < ny) ? sb[c * ns + y * nx + x] : (real)0;
+    }
+    __syncthreads();
+    const real g = s_g;
+    for (int e = tid; e < (H + 2) * (W + 2); e += 256) {
+        const int ly = e / (W + 2), lx = e - ly * (W + 2), x = x0 + lx - 1, y = y0 + ly - 1;
+        if (x < 0 || x >= nx || y < 0 || y >= ny) continue;
+        const int i = y * nx + x;
+        const real ax = ux[b * ns + i], ay = uy[b * ns + i];
+        const real v0 = S[0][ly + 1][lx + 1], v1 = S[1][ly + 1][lx + 1], a = ax * v0 + ay * v1;
+        const bool l = x > 0, rr = x < nx - 1, u = y > 0, d = y < ny - 1;
+        const real q0 = lap5(v0, l, S[0][ly + 1][lx], rr, S[0][ly + 1][lx + 2], u, S[0][ly][lx + 1], d, S[0][ly + 2][lx + 1]);
+        const real q1 = lap5(v1, l, S[1][ly + 1][lx], rr, S[1][ly + 1][lx + 2], u, S[1][ly][lx + 1], d, S[1][ly + 2][lx + 1]);
+        R[0][ly][lx] = ax * a - AtB[b * 2 * ns + i] + g * q0;
+        R[1][ly][lx] = ay * a - AtB[b * 2 * ns + ns + i] + g * q1;
+    }
+    __syncthreads();
+    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, lx = threadIdx.x + 1, ly = threadIdx.y + 1;
+    if (x >= nx || y >= ny) return;
+    const long long i = b * 2 * ns + y * nx + x;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const real v = R[c][ly][lx];
+        r[i + c * ns] = v;
+        q[i + c * ns] = lap5(v, x > 0, R[c][ly][lx - 1], x < nx - 1, R[c][ly][lx + 1], y > 0, R[c][ly - 1][lx], y < ny - 1, R[c][ly + 1][lx]);
+    }
+}
+
+template <typename real>
+mof_status launch_of_resid_lap(int nb, int nx, int ny, const real *ux, const real *uy, const real *AtB, const real *s,
+                               const double *gam, real *r, real *q, const int *act, cudaStream_t st) {
+    ::mof::count_launch(), k_of_resid_lap<real><<<dim3((nx + 31) / 32, (ny + 7) / 8, nb), dim3(32, 8), 0, st>>>(ux, uy, AtB, s, gam, r, q,
+                                                                                                            nx, ny, act);
+    MOF_LAUNCH_CHECK();
+    return MOF_OK;
 }
 
 template <typename real>
@@ -1013,11 +1131,10 @@ bool of_pass_applicable(long long ns, const void *V, const void *x) {
 }
 
 template <typename real>
-mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long long ns, int nx, int ny, const double *d, real *x,
-                                    real *q, const real *AtB, const real *ux, const real *uy, double *partial,
-                                    double *res, int *err, int kcap, const double *scale, double tol, int *grow,
-                                    double *GA, double *GL, double *g, double *Mg, double *nrm2_out, int *appended,
-                                    double *aux, cudaStream_t st) {
+mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long long ns, const double *d, const real *x, const real *q,
+                                    const real *AtB, const real *ux, const real *uy, double *partial, double *res, int *err,
+                                    int kcap, const double *scale, double tol, int *grow, double *GA, double *GL, double *g,
+                                    double *Mg, double *nrm2_out, int *appended, double *aux, int *done, cudaStream_t st) {
     static std::atomic<bool> configured{false};
     if (!configured.load()) {
         if (cudaFuncSetAttribute(k_of_proj_gram_pass<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, 140 * 1024) !=
@@ -1028,32 +1145,30 @@ mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long lon
     const int nc = (int)of_pass_chunks(ns, (int)sizeof(real));
     const int kc = kcap > 0 ? std::min(kcap, B.Kmax) : B.Kmax;
     const size_t smem = (size_t)(kc + 5) * 2048;
-    const dim3 lg((nx + 31) / 32, (ny + 7) / 8, 2 * B.B);
-    ::mof::count_launch(), k_of_lap<real><<<lg, dim3(32, 8), 0, st>>>(x, q, nx, ny, B.act);
-    ::mof::count_launch(), k_of_proj_gram_pass<real><<<dim3(nc, B.B), OP_T, smem, st>>>(B.V, ns, B.Kmax, B.K, B.act, d, x, q, AtB,
+    ::mof::count_launch(), k_of_proj_gram_pass<real><<<dim3(nc, B.B), OP_T, smem, st>>>(B.V, ns, B.Kmax, B.K, B.act, d, x, q, B.V, AtB,
                                                                                      ux, uy, partial, nc, err, kc);
     const int stride = of_pass_stride(B.Kmax);
-    ::mof::count_launch(), k_of_pass_reduce<<<dim3((stride + 7) / 8, B.B), 256, 0, st>>>(partial, nc, B.Kmax, B.K, B.act, res);
     int *slot = reinterpret_cast<int *>(aux);
     real *inv = reinterpret_cast<real *>(aux + B.B);
-    ::mof::count_launch(), k_of_pass_finish<real><<<B.B, 32, 0, st>>>(res, d, B.Kmax, Kmut, B.act, scale, tol, grow, GA, GL, g,
-                                                                     Mg, nrm2_out, appended, slot, inv);
-    const int blocks = (int)std::min<long long>(1024, (B.N + KT - 1) / KT);
-    ::mof::count_launch(), k_append<real><<<dim3(blocks, B.B), KT, 0, st>>>(B.V, B.N, B.Kmax, slot, inv, x, B.N, nullptr);
+    ::mof::count_launch(), k_of_pass_finish<real><<<dim3((stride + PF_T / 32 - 1) / (PF_T / 32), B.B), PF_T, 0, st>>>(
+        partial, nc, res, d, B.Kmax, Kmut, B.act, scale, tol, grow, GA, GL, g, Mg, nrm2_out, appended, slot, inv, done);
     MOF_LAUNCH_CHECK();
     return MOF_OK;
 }
 
 template bool of_pass_applicable<float>(long long, const void *, const void *);
 template bool of_pass_applicable<double>(long long, const void *, const void *);
-template mof_status launch_of_proj_gram_pass<float>(const BasisRef<float> &, int *, long long, int, int, const double *, float *,
-                                                    float *, const float *, const float *, const float *, double *, double *,
-                                                    int *, int, const double *, double, int *, double *, double *, double *,
-                                                    double *, double *, int *, double *, cudaStream_t);
-template mof_status launch_of_proj_gram_pass<double>(const BasisRef<double> &, int *, long long, int, int, const double *, double *,
-                                                     double *, const double *, const double *, const double *, double *,
-                                                     double *, int *, int, const double *, double, int *, double *, double *,
-                                                     double *, double *, double *, int *, double *, cudaStream_t);
+#define MOF_INST_OF(real)                                                                                                      \
+    template mof_status launch_of_proj_gram_pass<real>(const BasisRef<real> &, int *, long long, const double *, const real *, \
+                                                       const real *, const real *, const real *, const real *, double *,      \
+                                                       double *, int *, int, const double *, double, int *, double *,         \
+                                                       double *, double *, double *, double *, int *, double *, int *,        \
+                                                       cudaStream_t);                                                          \
+    template mof_status launch_of_combine<real>(const BasisRef<real> &, const double *, double *, real *, cudaStream_t);       \
+    template mof_status launch_of_resid_lap<real>(int, int, int, const real *, const real *, const real *, const real *,       \
+                                                  const double *, real *, real *, const int *, cudaStream_t);
+MOF_INST_OF(float)
+MOF_INST_OF(double)
 
 template struct Krylov<float>;
 template struct Krylov<double>;

@@ -977,8 +977,8 @@ __global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
         warp_trsv(Um, lds, invs, x0, x1, K, false);  // Rs y = w
         warp_trsv(Rm, lds, invd, x0, x1, K, false);  // R z = y
         const bool bad = (lane < K && !isfinite(x0)) || (lane + 32 < K && !isfinite(x1));
-        if (lane < K) z[lane] = x0;
-        if (lane + 32 < K) z[lane + 32] = x1;
+        if (lane < K) z[lane] = gh[lane] = x0;
+        if (lane + 32 < K) z[lane + 32] = gh[lane + 32] = x1;
         if (__any_sync(0xffffffffu, bad) || s_fail) {
             if (lane == 0) atomicOr(a.err, 2);
         }
@@ -987,6 +987,57 @@ __global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
             a.flag[b] = s_flag;
         }
     }
+    if (!a.proj) return;
+
+    // ---------------------------------------------- 6. proj = Mg^-1 ((G_A + lam G_L) z - g)
+    // by the inverse Cholesky factor of Mg: matrix-vector products instead of two triangular
+    // solves (each a chain of K dependent FP64 steps); a new vector adds one row
+    double *Li = a.Linv + (long long)b * ld * ld, *zs = gh, *cv = theta, *lv = c2;
+    const double *Mg = a.Mg + (long long)b * ld * ld;
+    const int n0 = a.nL[b];
+    for (int e = tid; e < K * K; e += ST) {
+        const int i = e / K, j = e - (e / K) * K;
+        AT(Tm, i, j) = (j <= i && i < n0) ? Li[i * ld + j] : 0.0;
+    }
+    __syncthreads();
+    // out_i = sum_k M(i, k) v_k, a warp per row, lanes over k
+    auto matvec = [&](double *out, int n, auto &&row) {
+        for (int i = wid; i < n; i += NW) {
+            double t = 0.0;
+            for (int k = lane; k < n; k += 32) t += row(i, k);
+            t = warp_sum(t);
+            if (lane == 0) out[i] = t;
+        }
+        __syncthreads();
+    };
+    for (int r = n0; r < K; ++r) {  // Linv of [L 0; l^T d]: the row [-(l^T Linv) / d, 1 / d], l = Linv Mg[:, r]
+        matvec(lv, r, [&](int i, int k) { return k <= i ? AT(Tm, i, k) * Mg[k * ld + r] : 0.0; });
+        matvec(cv, r, [&](int i, int k) { return k >= i ? AT(Tm, k, i) * lv[k] : 0.0; });
+        if (wid == 0) {
+            double t = 0.0;
+            for (int k = lane; k < r; k += 32) t += lv[k] * lv[k];
+            t = warp_sum(t);
+            const double id = 1.0 / sqrt(fmax(Mg[r * ld + r] - t, 1e-300));
+            for (int k = lane; k < r; k += 32) Li[r * ld + k] = AT(Tm, r, k) = -cv[k] * id;
+            if (lane == 0) Li[r * ld + r] = AT(Tm, r, r) = id;
+        }
+        __syncthreads();
+    }
+    // the Grams are symmetric: entry (i, k) is read as (k, i)'s mirror, lanes over k
+    for (int i = wid; i < K; i += NW) {
+        double sa = 0.0, sl = 0.0;
+        for (int k = lane; k < K; k += 32) {
+            sa += GA[i * ld + k] * zs[k];
+            sl += GL[i * ld + k] * zs[k];
+        }
+        warp_sum2(sa, sl);
+        if (lane == 0) cv[i] = sa + lam * sl - g[i];
+    }
+    __syncthreads();
+    matvec(lv, K, [&](int i, int k) { return k <= i ? AT(Tm, i, k) * cv[k] : 0.0; });
+    matvec(zs, K, [&](int i, int k) { return k >= i ? AT(Tm, k, i) * lv[k] : 0.0; });
+    for (int i = tid; i < K; i += ST) a.proj[(long long)b * ld + i] = zs[i];
+    if (tid == 0) a.nL[b] = K;
 #undef AT
 #undef AF
 }

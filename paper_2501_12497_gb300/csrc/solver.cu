@@ -136,8 +136,8 @@ struct WS {
     // ---- Solve-OF (P pairs)
     real *ux, *uy, *ut, *bof, *Vof, *Uof, *AtB, *wv, *wu, *y1, *y2, *sof, *vnew_of, *q_of;
     double *GA, *GL, *gof, *zof, *gam, *nrm_of, *coef_of, *coefU_of, *scale_of, *alpha_of, *alpha1_of, *beta_of,
-        *beta1_of, *bb_of, *Mg_of, *pres_of;
-    int *Kv_of, *Ku_of, *grow_of, *gkb_of, *act_of, *app_of, *flag_of;
+        *beta1_of, *bb_of, *Mg_of, *Linv_of, *pres_of;
+    int *Kv_of, *Ku_of, *grow_of, *gkb_of, *act_of, *app_of, *flag_of, *nL_of, *done_of;
     real *wf_of = nullptr, *wl_of = nullptr;  // IRLS weights of Solve-OF with p = q = 1 (P ns, 4 P ns)
     double *rn_of = nullptr;                  // norm^2 of its residual before orthogonalisation (P)
     int pq1 = 0;                              // workspace holds the p = q = 1 arrays
@@ -399,6 +399,7 @@ static mof_status ensure_ws(mof_problem *p, const mof_solver_params &prm, int n_
         w->nrm_of = a.take<double>(P);
         w->coef_of = a.take<double>((size_t)P * Kof);
         w->Mg_of = a.take<double>((size_t)P * Kof * Kof);
+        w->Linv_of = a.take<double>((size_t)P * Kof * Kof);
         w->pres_of = a.take<double>((size_t)P * of_pass_stride(Kof));
         w->q_of = a.take<real>((size_t)P * N2);
         w->coefU_of = a.take<double>((size_t)P * (prm.of_ell + 1));
@@ -415,6 +416,8 @@ static mof_status ensure_ws(mof_problem *p, const mof_solver_params &prm, int n_
         w->act_of = a.take<int>(P);
         w->app_of = a.take<int>(P);
         w->flag_of = a.take<int>(P);
+        w->nL_of = a.take<int>(P);
+        w->done_of = a.take<int>(P);
         w->wf_of = a.take<real>(w->pq1 ? P * ns : 0);
         w->wl_of = a.take<real>(w->pq1 ? 4 * P * ns : 0);
         w->rn_of = a.take<double>(w->pq1 ? P : 0);
@@ -610,57 +613,20 @@ __global__ void k_of_resid(const real *__restrict__ ux, const real *__restrict__
 // onto the stored basis's span; so the second update pass over the basis (x' - V c2) is never
 // applied to the vectors. The span, the Grams of the stored vectors and everything the small
 // solver computes from them (z, the parameter, s = V z) are those of the basis CGS twice
-// would store, up to rounding.
-__global__ void k_of_mg_init(double *__restrict__ Mg, int ld, const int *__restrict__ act, int B) {
+// would store, up to rounding. The small solver forms d by the inverse of Mg's Cholesky factor,
+// one row longer with every append (48 us per iteration of 7 pairs in FP64 for a factorisation and
+// two triangular solves in one warp; 6 us of the small solve as matrix-vector products).
+// Also the inverse Cholesky factor of Mg over the first K vectors (I) and no appended vector
+// waiting for its scale (slot = -1).
+__global__ void k_of_mg_init(double *__restrict__ Mg, double *__restrict__ Linv, int *__restrict__ nL, const int *__restrict__ K,
+                             int *__restrict__ slot, int ld, const int *__restrict__ act, int B) {
     const int b = blockIdx.x;
-    if (b >= B || (act && !act[b])) return;
-    double *M = Mg + (long long)b * ld * ld;
-    for (int e = threadIdx.x; e < ld * ld; e += blockDim.x) M[e] = (e / ld == e % ld) ? 1.0 : 0.0;
-}
-
-// c[b] <- Mg[b]^-1 c[b] over the first K[b] entries: Cholesky in shared memory by one warp
-// (lanes over rows), then the two triangular solves. Mg is near I (unit diagonal, off
-// diagonal the stored vectors' residual overlaps), so the factorisation is well conditioned.
-__global__ void __launch_bounds__(32) k_of_mg_solve(const double *__restrict__ Mg, double *__restrict__ c, int ld,
-                                                    const int *__restrict__ K, const int *__restrict__ act) {
-    extern __shared__ double mg_sm[];  // [ld][ld + 1] Cholesky factor (lower), then [ld] the right side
-    const int b = blockIdx.x, lane = threadIdx.x;
+    if (b >= B) return;
+    if (threadIdx.x == 0) slot[b] = -1;
     if (act && !act[b]) return;
-    const int Kb = min(K[b], ld), L = ld + 1;
-    double *Lm = mg_sm, *y = mg_sm + (long long)ld * L;
-    const double *M = Mg + (long long)b * ld * ld;
-    double *cb = c + (long long)b * ld;
-    for (int e = lane; e < Kb * Kb; e += 32) Lm[(e / Kb) * L + e % Kb] = M[(e / Kb) * ld + e % Kb];
-    for (int i = lane; i < Kb; i += 32) y[i] = cb[i];
-    __syncwarp();
-    for (int j = 0; j < Kb; ++j) {
-        // column j: rows i >= j, s_i = M[i][j] - sum_{k<j} L[i][k] L[j][k]
-        for (int i = j + lane; i < Kb; i += 32) {
-            double sum = Lm[i * L + j];
-            for (int k = 0; k < j; ++k) sum -= Lm[i * L + k] * Lm[j * L + k];
-            Lm[i * L + j] = sum;
-        }
-        __syncwarp();
-        const double d = sqrt(fmax(Lm[j * L + j], 1e-300));
-        for (int i = j + 1 + lane; i < Kb; i += 32) Lm[i * L + j] /= d;
-        __syncwarp();
-        if (lane == 0) Lm[j * L + j] = d;
-        __syncwarp();
-    }
-    if (lane == 0) {  // L y = c, then L^T d = y (K <= 64 sequential steps)
-        for (int i = 0; i < Kb; ++i) {
-            double t = y[i];
-            for (int k = 0; k < i; ++k) t -= Lm[i * L + k] * y[k];
-            y[i] = t / Lm[i * L + i];
-        }
-        for (int i = Kb - 1; i >= 0; --i) {
-            double t = y[i];
-            for (int k = i + 1; k < Kb; ++k) t -= Lm[k * L + i] * y[k];
-            y[i] = t / Lm[i * L + i];
-        }
-    }
-    __syncwarp();
-    for (int i = lane; i < Kb; i += 32) cb[i] = y[i];
+    double *M = Mg + (long long)b * ld * ld, *L = Linv + (long long)b * ld * ld;
+    for (int e = threadIdx.x; e < ld * ld; e += blockDim.x) M[e] = L[e] = (e / ld == e % ld) ? 1.0 : 0.0;
+    if (threadIdx.x == 0) nL[b] = min(K[b], ld);
 }
 
 // After an append (appended[b]; K[b] already counts the new vector): the new column of Mg,
@@ -1462,7 +1428,6 @@ __global__ void k_report(double *__restrict__ rep, int *__restrict__ iter, const
 }
 
 static inline int fb(long long n) { return (int)std::min<long long>(152 * 8, (n + 255) / 256); }
-static inline size_t mg_solve_smem(int ld) { return sizeof(double) * ((size_t)ld * (ld + 1) + ld); }
 
 // ============================================================ Solve-OF
 template <typename real>
@@ -1478,29 +1443,28 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
         MOF_TRY(launch_of_fields<real>(p, u, prm.of_dr, w.ux, w.uy, w.ut, st));
         ::mof::count_launch(), k_of_rhs<real><<<dim3(fb(ns), P), 256, 0, st>>>(w.ux, w.uy, w.ut, w.bof, w.AtB, ns);
     }
-    // The pairs are split into groups, each running its whole Solve-OF (GKB start,
-    // initial Gram columns, GKS iterations) on its own stream: a group's small
-    // FP64 solves occupy one SM per pair and are latency bound, and its GKB steps
-    // are short launches, so the groups fill the GPU together. Every kernel works
-    // per pair, so the grouping does not change the result.
-    // the plain form: one pair per group, all on the solver's stream one after another
-    const int G = prm.plain ? P : std::max(1, std::min(prm.of_streams > 0 ? prm.of_streams : AUTO_OF_STREAMS, P));
-    const long long part_pair = of_partial_per_pair(p, Kof, w.of_ell);
-    if (!prm.plain) MOF_CUDA(cudaEventRecord(w.gfork, st));
-    for (int gi = 0; gi < G; ++gi) {
-        const int b0 = (int)((long long)gi * P / G), nb = (int)((long long)(gi + 1) * P / G) - b0;
-        const cudaStream_t gst = prm.plain ? st : w.gs[gi];
-        if (!prm.plain) MOF_CUDA(cudaStreamWaitEvent(gst, w.gfork, 0));
+    // Golub-Kahan start and initial Gram columns of all pairs together: short launches, bound by
+    // bandwidth on large frames and by latency on small ones. Then the pairs are split into groups,
+    // each running its GKS iterations on its own stream: a group's small FP64 solves occupy one SM
+    // per pair and are latency bound, and the other groups' passes fill the GPU meanwhile. Every
+    // kernel works per pair, so the grouping does not change the result. The plain form takes one
+    // pair after another, all on the solver's stream.
+    const long long part_pair = of_partial_per_pair(p, Kof, w.of_ell), KK = (long long)Kof * Kof;
+    const bool pq1 = prm.of_pq == 1;
+    auto krylov = [&](int b0) {
         Krylov<real> kg;
         kg.partial = w.partial + b0 * part_pair;
         kg.err = w.err;
         kg.aux = w.kaux + 2LL * b0;
-        const long long KK = (long long)Kof * Kof;
-        real *Vg = w.Vof + (long long)b0 * Kof * N2, *sg = s_out + (long long)b0 * N2, *wvg = w.wv + (long long)b0 * N2;
+        return kg;
+    };
+    auto start = [&](int b0, int nb, cudaStream_t gst) -> mof_status {
+        const Krylov<real> kg = krylov(b0);
+        real *Vg = w.Vof + (long long)b0 * Kof * N2, *wvg = w.wv + (long long)b0 * N2;
         real *Ug = w.Uof + (long long)b0 * ldU * ns, *wug = w.wu + (long long)b0 * ns;
         const real *uxg = w.ux + (long long)b0 * ns, *uyg = w.uy + (long long)b0 * ns, *AtBg = w.AtB + (long long)b0 * N2;
         const real *bofg = w.bof + (long long)b0 * ns;
-        int *Kvg = w.Kv_of + b0, *Kug = w.Ku_of + b0, *actg = w.act_of + b0, *appg = w.app_of + b0, *gkbg = w.gkb_of + b0;
+        int *Kvg = w.Kv_of + b0, *Kug = w.Ku_of + b0, *actg = w.act_of + b0, *gkbg = w.gkb_of + b0;
         double *nrmg = w.nrm_of + b0, *bbg = w.bb_of + b0;
         const int pb = (nb + 63) / 64;
         BasisRef<real> BV{Vg, N2, Kof, nb, Kvg, gkbg};
@@ -1525,23 +1489,32 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
                                 gst);
             }
         }
-        const dim3 gg((p->nx + 31) / 32, (p->ny + 7) / 8, nb);
-        BasisRef<real> BAg{Vg, N2, Kof, nb, Kvg, actg};
-        const int gram_ctas = (int)((ns + ofc<real>() - 1) / ofc<real>());
-        const int gram_red = (2 * Kof + 1 + 7) / 8;
-        const real *bofg2 = w.bof + (long long)b0 * ns;
-        const bool pq1 = prm.of_pq == 1;
-        real *wfg = pq1 ? w.wf_of + (long long)b0 * ns : nullptr, *wlg = pq1 ? w.wl_of + (long long)b0 * 4 * ns : nullptr;
         if (!pq1) {
             Scope sc(tm, "of_gram", gst);
+            const int gram_ctas = (int)((ns + ofc<real>() - 1) / ofc<real>()), gram_red = (2 * Kof + 1 + 7) / 8;
             const int ncol = std::min(prm.of_ell, Kof);
-            ::mof::count_launch(), k_of_gram_cols<real><<<dim3(gram_ctas, nb, ncol), OFG_T, 0, gst>>>(Vg, Kof, Kvg, actg, 0, uxg, uyg, bofg2,
+            ::mof::count_launch(), k_of_gram_cols<real><<<dim3(gram_ctas, nb, ncol), OFG_T, 0, gst>>>(Vg, Kof, Kvg, actg, 0, uxg, uyg, bofg,
                                                                                                    p->nx, p->ny, kg.partial);
             ::mof::count_launch(), k_of_gram_reduce<<<dim3(gram_red, nb, ncol), 256, 0, gst>>>(kg.partial, gram_ctas, Kof, Kvg, actg, 0,
                                                                                              w.GA + b0 * KK, w.GL + b0 * KK,
                                                                                              w.gof + (long long)b0 * Kof);
         }
-        ::mof::count_launch(), k_of_mg_init<<<nb, 256, 0, gst>>>(w.Mg_of + (long long)b0 * KK, Kof, actg, nb);
+        return MOF_OK;
+    };
+    auto iterate = [&](int b0, int nb, cudaStream_t gst) -> mof_status {
+        const Krylov<real> kg = krylov(b0);
+        real *Vg = w.Vof + (long long)b0 * Kof * N2, *sg = s_out + (long long)b0 * N2, *wvg = w.wv + (long long)b0 * N2;
+        const real *uxg = w.ux + (long long)b0 * ns, *uyg = w.uy + (long long)b0 * ns, *AtBg = w.AtB + (long long)b0 * N2;
+        const real *bofg = w.bof + (long long)b0 * ns;
+        int *Kvg = w.Kv_of + b0, *actg = w.act_of + b0, *appg = w.app_of + b0;
+        const int pb = (nb + 63) / 64;
+        const dim3 gg((p->nx + 31) / 32, (p->ny + 7) / 8, nb);
+        BasisRef<real> BAg{Vg, N2, Kof, nb, Kvg, actg};
+        const int gram_ctas = (int)((ns + ofc<real>() - 1) / ofc<real>());
+        const int gram_red = (2 * Kof + 1 + 7) / 8;
+        real *wfg = pq1 ? w.wf_of + (long long)b0 * ns : nullptr, *wlg = pq1 ? w.wl_of + (long long)b0 * 4 * ns : nullptr;
+        ::mof::count_launch(), k_of_mg_init<<<nb, 256, 0, gst>>>(w.Mg_of + b0 * KK, w.Linv_of + b0 * KK, w.nL_of + b0, Kvg,
+                                                                  reinterpret_cast<int *>(kg.aux), Kof, actg, nb);
         // the one-pass projection with the Gram column needs 16-byte aligned component segments
         const bool pass_ok = !pq1 && Kof <= 64 && of_pass_applicable<real>(ns, Vg, wvg);
         SmallArgs sa{};
@@ -1558,6 +1531,9 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
         sa.z = w.zof + (long long)b0 * Kof;
         sa.flag = w.flag_of + b0;
         sa.err = w.err;
+        sa.Mg = w.Mg_of + b0 * KK;
+        sa.Linv = w.Linv_of + b0 * KK;
+        sa.nL = w.nL_of + b0;
         BasisRef<real> BS{Vg, N2, Kof, nb, Kvg, nullptr};
         const int wg_ctas = (int)std::min<long long>(WG_CTAS, (ns + WG_P - 1) / WG_P);
         for (int it = 0; it < prm.of_iters; ++it) {
@@ -1565,58 +1541,59 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
                 // MM-GKS: IRLS weights of the current velocity (zero at the start), then the
                 // weighted Grams of the whole basis
                 Scope sc(tm, "of_irls", gst);
-                ::mof::count_launch(), k_of_irls_weights<real><<<gg, blk2, 0, gst>>>(uxg, uyg, bofg2, it == 0 ? nullptr : sg,
+                ::mof::count_launch(), k_of_irls_weights<real><<<gg, blk2, 0, gst>>>(uxg, uyg, bofg, it == 0 ? nullptr : sg,
                                                                                    (real)(prm.eps * prm.eps), wfg, wlg, p->nx,
                                                                                    p->ny, actg);
                 ::mof::count_launch(), k_of_wgram<real><<<dim3(wg_ctas, nb), WG_T, wg_smem<real>(Kof), gst>>>(
-                    Vg, Kof, Kvg, actg, uxg, uyg, bofg2, wfg, wlg, p->nx, p->ny, kg.partial);
+                    Vg, Kof, Kvg, actg, uxg, uyg, bofg, wfg, wlg, p->nx, p->ny, kg.partial);
                 ::mof::count_launch(), k_of_wgram_reduce<<<dim3((wg_pstride(Kof) + 7) / 8, nb), 256, 0, gst>>>(
                     kg.partial, wg_ctas, Kof, Kvg, actg, w.GA + b0 * KK, w.GL + b0 * KK, w.gof + (long long)b0 * Kof,
                     w.bb_of + b0);
             }
             {
+                // with the projection coefficients d = Mg^-1 V^T r of the residual that follows
                 Scope sc(tm, "of_small", gst);
+                sa.proj = it == prm.of_iters - 1 ? nullptr : w.coef_of + (long long)b0 * Kof;
                 MOF_TRY(launch_small_solve(sa, gst));
             }
             {
                 Scope sc(tm, "of_combine", gst);
-                kg.combine(BS, sa.z, Kof, sg, N2, gst);
+                if (pass_ok) MOF_TRY(launch_of_combine<real>(BS, sa.z, kg.aux, sg, gst));
+                else kg.combine(BS, sa.z, Kof, sg, N2, gst);
             }
             if (it == prm.of_iters - 1) break;
             if (pq1) {
                 Scope sc(tm, "of_resid", gst);
-                ::mof::count_launch(), k_of_resid_w<real><<<gg, blk2, 0, gst>>>(uxg, uyg, bofg2, sg, wfg, wlg, sa.lam, wvg, p->nx,
+                ::mof::count_launch(), k_of_resid_w<real><<<gg, blk2, 0, gst>>>(uxg, uyg, bofg, sg, wfg, wlg, sa.lam, wvg, p->nx,
                                                                               p->ny, actg);
                 // the growth test compares with the residual's own norm (the weights rescale it)
                 kg.norm2(wvg, N2, N2, nb, w.rn_of + b0, gst);
                 ::mof::count_launch(), k_sqrt_into<<<pb, 64, 0, gst>>>(w.rn_of + b0, w.scale_of + b0, nb);
+            } else if (pass_ok) {
+                Scope sc(tm, "of_resid", gst);
+                MOF_TRY(launch_of_resid_lap<real>(nb, p->nx, p->ny, uxg, uyg, AtBg, sg, sa.lam, wvg, w.q_of + (long long)b0 * N2, actg,
+                                                  gst));
             } else {
                 Scope sc(tm, "of_resid", gst);
                 ::mof::count_launch(), k_of_resid<real><<<gg, blk2, 0, gst>>>(uxg, uyg, AtBg, sg, sa.lam, wvg, p->nx, p->ny, actg);
             }
             {
                 // Projection of the residual onto the complement of the stored basis's span in
-                // one pass over the basis: V^T r from the Grams, d = Mg^-1 V^T r, then the fused
-                // pass x' = r - V d with c2 = V^T x' and ||x'||^2; the append stores x'/||x'|| and
-                // c2 / ||x'|| becomes the new column of Mg (see k_of_mg_init).
+                // one pass over the basis: x' = r - V d with c2 = V^T x' and ||x'||^2; the append
+                // stores x'/||x'|| and c2 / ||x'|| becomes the new column of Mg (see k_of_mg_init).
                 double *cg = w.coef_of + (long long)b0 * Kof;
                 double *Mgg = w.Mg_of + (long long)b0 * KK;
-                {
-                    Scope sc(tm, "of_reorth", gst);
-                    ::mof::count_launch(), k_of_proj_gram<<<nb, 32, 0, gst>>>(sa.GA, sa.GL, sa.g, sa.z, sa.lam, Kvg, actg, Kof, cg);
-                    ::mof::count_launch(), k_of_mg_solve<<<nb, 32, mg_solve_smem(Kof), gst>>>(Mgg, cg, Kof, Kvg, actg);
-                }
                 // at GKS iteration it the basis holds at most of_ell + it vectors (one append per iteration)
                 const int kcap = std::min(Kof, prm.of_ell + it);
                 if (pass_ok) {
                     // p = q = 2: the projection, the new vector's Gram columns and the append in
                     // one pass over the basis (no separate Gram-column pass after it)
                     Scope sc(tm, "of_subdot", gst);
-                    MOF_TRY(launch_of_proj_gram_pass<real>(BAg, Kvg, ns, p->nx, p->ny, cg, wvg, w.q_of + (long long)b0 * N2, AtBg,
-                                                           uxg, uyg, kg.partial, w.pres_of + (long long)b0 * of_pass_stride(Kof),
-                                                           w.err, kcap, w.scale_of + b0, tol, w.grow_of + b0, w.GA + b0 * KK,
-                                                           w.GL + b0 * KK,
-                                                           w.gof + (long long)b0 * Kof, Mgg, w.nrm_of + b0, appg, kg.aux, gst));
+                    MOF_TRY(launch_of_proj_gram_pass<real>(BAg, Kvg, ns, cg, wvg, w.q_of + (long long)b0 * N2, AtBg, uxg, uyg,
+                                                           kg.partial, w.pres_of + (long long)b0 * of_pass_stride(Kof), w.err, kcap,
+                                                           w.scale_of + b0, tol, w.grow_of + b0, w.GA + b0 * KK, w.GL + b0 * KK,
+                                                           w.gof + (long long)b0 * Kof, Mgg, w.nrm_of + b0, appg, kg.aux,
+                                                           w.done_of + b0, gst));
                     continue;
                 }
                 bool fused;
@@ -1639,17 +1616,33 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
             }
             if (!pq1) {
                 Scope sc(tm, "of_gram", gst);
-                ::mof::count_launch(), k_of_gram_cols<real><<<dim3(gram_ctas, nb, 1), OFG_T, 0, gst>>>(Vg, Kof, Kvg, appg, 1, uxg, uyg, bofg2,
+                ::mof::count_launch(), k_of_gram_cols<real><<<dim3(gram_ctas, nb, 1), OFG_T, 0, gst>>>(Vg, Kof, Kvg, appg, 1, uxg, uyg, bofg,
                                                                                                     p->nx, p->ny, kg.partial);
                 ::mof::count_launch(), k_of_gram_reduce<<<dim3(gram_red, nb, 1), 256, 0, gst>>>(kg.partial, gram_ctas, Kof, Kvg, appg, 1,
                                                                                               w.GA + b0 * KK, w.GL + b0 * KK,
                                                                                               w.gof + (long long)b0 * Kof);
             }
         }
-        if (!prm.plain) MOF_CUDA(cudaEventRecord(w.gdone[gi], gst));
+        return MOF_OK;
+    };
+    if (prm.plain) {
+        for (int b = 0; b < P; ++b) {
+            MOF_TRY(start(b, 1, st));
+            MOF_TRY(iterate(b, 1, st));
+        }
+        MOF_LAUNCH_CHECK();
+        return MOF_OK;
     }
-    if (!prm.plain)
-        for (int gi = 0; gi < G; ++gi) MOF_CUDA(cudaStreamWaitEvent(st, w.gdone[gi], 0));
+    MOF_TRY(start(0, P, st));
+    const int G = std::max(1, std::min(prm.of_streams > 0 ? prm.of_streams : AUTO_OF_STREAMS, P));
+    MOF_CUDA(cudaEventRecord(w.gfork, st));
+    for (int gi = 0; gi < G; ++gi) {
+        const int b0 = (int)((long long)gi * P / G), nb = (int)((long long)(gi + 1) * P / G) - b0;
+        MOF_CUDA(cudaStreamWaitEvent(w.gs[gi], w.gfork, 0));
+        MOF_TRY(iterate(b0, nb, w.gs[gi]));
+        MOF_CUDA(cudaEventRecord(w.gdone[gi], w.gs[gi]));
+        MOF_CUDA(cudaStreamWaitEvent(st, w.gdone[gi], 0));
+    }
     MOF_LAUNCH_CHECK();
     return MOF_OK;
 }

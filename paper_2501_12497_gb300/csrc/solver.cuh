@@ -105,20 +105,26 @@ struct Krylov {
                 const double *scale, double tol, int *grow, int *appended, real *stage, cudaStream_t st) const;
 };
 
-// Solve-OF (p = q = 2) GKS step after the projection coefficients d: the graph Laplacian q of
-// the residual x, then one pass over the basis forming x' = x - V d (in x) with the dot
-// products that give the new vector's Gram columns, the append decision, the new columns of
-// G_A, G_L, g and Mg, and the append of x'/||x'|| (krylov.cu, k_of_proj_gram_pass).
-// partial: [B][chunks][3 Kmax + 4] doubles; res: [B][3 Kmax + 4]; q: [B][2 ns] scratch.
+// Solve-OF (p = q = 2) GKS step. launch_of_resid_lap: the residual r at s and its graph
+// Laplacian q. launch_of_proj_gram_pass, after the projection coefficients d: one pass over the
+// basis forming x' = r - V d (into the slot behind the basis) with the dot products that give the
+// new vector's Gram columns, then the append decision and the new columns of G_A, G_L, g and Mg.
+// launch_of_combine: s = V z, scaling a vector appended since the last call to x' / ||x'||.
+// partial: [B][chunks][3 Kmax + 4] doubles; res: [B][3 Kmax + 4]; aux: 2 B doubles (the slot and
+// scale between an append and the next combine); done: [B] ints, zero between calls.
 long long of_pass_chunks(long long ns, int elem_bytes);
 int of_pass_stride(int Kmax);
 template <typename real> bool of_pass_applicable(long long ns, const void *V, const void *x);
 template <typename real>
-mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long long ns, int nx, int ny, const double *d, real *x,
-                                    real *q, const real *AtB, const real *ux, const real *uy, double *partial,
-                                    double *res, int *err, int kcap, const double *scale, double tol, int *grow,
-                                    double *GA, double *GL, double *g, double *Mg, double *nrm2_out, int *appended,
-                                    double *aux, cudaStream_t st);
+mof_status launch_of_resid_lap(int nb, int nx, int ny, const real *ux, const real *uy, const real *AtB, const real *s,
+                               const double *gam, real *r, real *q, const int *act, cudaStream_t st);
+template <typename real>
+mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long long ns, const double *d, const real *x, const real *q,
+                                    const real *AtB, const real *ux, const real *uy, double *partial, double *res, int *err,
+                                    int kcap, const double *scale, double tol, int *grow, double *GA, double *GL, double *g,
+                                    double *Mg, double *nrm2_out, int *appended, double *aux, int *done, cudaStream_t st);
+template <typename real>
+mof_status launch_of_combine(const BasisRef<real> &B, const double *z, double *aux, real *out, cudaStream_t st);
 
 // Bound of the device waits on tile copies for the current device (polls; < 0: the
 // default); used by mof_debug_set_wait_limit.
@@ -143,6 +149,15 @@ struct SmallArgs {
     double *z;             // [B][ld] out
     int *flag;             // [B] out: DP flag
     int *err;              // error word (|= 1: factorisation failed, 2: non-finite)
+    // Projection of the residual at z onto the stored basis (null: none). With r the residual of
+    // the normal equations at V z, V^T r = (G_A + lam G_L) z - g exactly, so the coefficients
+    // proj = Mg^-1 V^T r of its orthogonal projection need no pass over V. Mg [B][ld][ld] is the
+    // basis's Euclidean Gram, Linv the inverse of its Cholesky factor over the first nL[b]
+    // vectors, which the call brings up to K[b].
+    const double *Mg;
+    double *Linv;
+    int *nL;
+    double *proj;          // [B][ld] out
 };
 mof_status launch_small_solve(const SmallArgs &a, cudaStream_t st);
 // Raise the kernel's dynamic shared-memory limit for leading dimension ld
