@@ -825,7 +825,7 @@ __global__ void __launch_bounds__(BT) k_warpT_tile(const real *__restrict__ r, c
             finite = bits_finite(M, real(0));
             E = clamp_E(48 - (M ? bits_exp(M, real(0)) : 0));
             fx_pow2(E, sc);
-            int *hi = reinterpret_cast<int *>(acc), *lo = hi + FAST_N;
+            int *hi = reinterpret_cast<int *>(acc);
             const unsigned nw = X1 - X0 + 1, nh = Y1 - Y0 + 1;
             // the next candidate's velocity is loaded while this one's terms are added
             float vx = 0.f, vy = 0.f;

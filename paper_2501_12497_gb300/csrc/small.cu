@@ -23,8 +23,8 @@
 //      trace(I - S) = sum (1 - f_i), with closed-form derivatives in lam;
 //   4. picks lam on the bracket 10^[log10 rho - 12, log10 rho + 12]:
 //      GCV: the first minimum of a 200-point log grid (ties to the smaller
-//      lam), every point evaluated in FP64 (one thread per point), then
-//      refined between its two grid neighbours by
+//      lam): an FP32 scan leaves the points that can be it, FP64 decides among
+//      those; then refined between its two grid neighbours by
 //      safeguarded Newton steps on dG/dlog10(lam) = 0 (FP32 steps, then FP64
 //      steps, which stop after a Newton step below 1e-6 -- the next would be
 //      below ~1e-12 -- or once the derivative is at its rounding level), kept
@@ -45,10 +45,18 @@
 // upper triangle), keeps the serial parts (pivots, rotation angles,
 // substitutions, Newton steps) in one warp, and evaluates in FP32 what a
 // later FP64 step corrects (the Jacobi warm start, the lambda grids).
+//
+// The solves of one Solve-OF (p = q = 2) differ by one basis vector each: from the second on steps 1
+// and 2 are replaced by the update of the bordered eigenproblem below (rho that of the first), and z
+// comes from X with one step of refinement. All blocks of a call run side by side, one per SM, so a
+// call lasts as long as one block; 31 pairs at 256^2, basis 10 to 29, mean of 20 calls: 190 us when
+// every call factored anew and scanned the grid in FP64, 80 us now (of about 61 + 42 + 34 thousand
+// clocks for update, lambda and the rest at K = 20, the FP64 pipe is busy or waited for in all).
 #include "solver.cuh"
 
 #include <atomic>
 #include <cfloat>
+#include <cmath>
 
 namespace mof {
 
@@ -59,7 +67,7 @@ constexpr int NW = ST / 32;
 constexpr int GRID_POINTS = 200;
 constexpr int NEWTON_MAX = 60;
 constexpr int NEWTON32_MAX = 30;
-constexpr int NREF = 5;  // FP64 re-evaluated grid points around the FP32 minimum
+constexpr int NREF = 5;  // grid points around the minimum that decide whether it is flat
 constexpr double BRACKET_DECADES = 12.0;
 constexpr double THETA_TINY = 1e-14;
 constexpr int JACOBI32_MAX_SWEEPS = 12;
@@ -124,6 +132,50 @@ __device__ __forceinline__ void warp_sum6(double s[6]) {
     s[3] = __shfl_sync(0xffffffffu, y, 24);
     s[4] = __shfl_sync(0xffffffffu, y, 4);
     s[5] = __shfl_sync(0xffffffffu, y, 20);
+}
+
+// 1 / x from the FP32 reciprocal by two Newton steps, |x| within the normal FP32 range
+__device__ __forceinline__ double rcp_newton(double x) {  // 1 / x, |x| within the normal FP32 range
+    double r = (double)__frcp_rn((float)x);
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+// Sums over k < m of f(i, k) (and of f2) for the rows i < n <= 64: the rows over the lanes, k over
+// the CTA's warps, the warps' partial sums in part (2 ST doubles). A reduction over lanes would
+// take five dependent FP64 additions per row, the costly part on a pipe that a warp holds for
+// 64 cycles per instruction. out(i, sum, sum2) is called by one thread per row. All threads
+// call; ends with a barrier.
+template <typename F, typename O>
+__device__ __forceinline__ void row_sums2(int n, int m, double *part, F &&f, O &&out) {
+    const int tid = threadIdx.x, RS = n <= 32 ? 32 : 64, parts = ST / RS, i = tid & (RS - 1);
+    double x = 0.0, y = 0.0;
+    if (i < n)
+        for (int k = tid / RS; k < m; k += parts) f(i, k, x, y);
+    part[tid] = x;
+    part[ST + tid] = y;
+    __syncthreads();
+    if (tid < n) {
+        for (int q = 1; q < parts; ++q) {
+            x += part[q * RS + tid];
+            y += part[ST + q * RS + tid];
+        }
+        out(tid, x, y);
+    }
+    __syncthreads();
+}
+template <typename F, typename O>
+__device__ __forceinline__ void row_sums(int n, int m, double *part, F &&f, O &&out) {
+    const int tid = threadIdx.x, RS = n <= 32 ? 32 : 64, parts = ST / RS, i = tid & (RS - 1);
+    double x = 0.0;
+    if (i < n)
+        for (int k = tid / RS; k < m; k += parts) x += f(i, k);
+    part[tid] = x;
+    __syncthreads();
+    if (tid < n) {
+        for (int q = 1; q < parts; ++q) x += part[q * RS + tid];
+        out(tid, x);
+    }
+    __syncthreads();
 }
 
 // ------------------------------------------------------------ dense kernels
@@ -527,7 +579,9 @@ __device__ __forceinline__ void lam_terms6(const SP &S, R mu, R s[6]) {
             s[3] += R(1);
             continue;
         }
-        const R inv = R(1) / d;
+        R inv;
+        if constexpr (sizeof(R) == 8) inv = rcp_newton(d);  // d within [1e-13, 1e13]
+        else inv = R(1) / d;
         const R g = mu * a * inv, g1 = a * th * inv * inv, g2 = R(-2) * a * g1 * inv;
         s[0] += c * g * g;
         s[1] += R(2) * c * g * g1;
@@ -567,7 +621,7 @@ __device__ __forceinline__ void lam_terms_nd(const Spec &S, double mu, double &N
     D = 0.0;
     for (int i = threadIdx.x & 31; i < S.K; i += 32) {
         const double th = S.theta[i], a = 1.0 - th, d = th + mu * a;
-        const double g = d > 0.0 ? mu * a / d : 1.0;
+        const double g = d > 0.0 ? mu * a * rcp_newton(d) : 1.0;
         N += S.c2[i] * g * g;
         D += g;
     }
@@ -624,12 +678,504 @@ __device__ __forceinline__ R newton_step(R t, R f, R f1, R &A, R &B) {
     return tn;
 }
 
+// mu 10^dt for a small dt (|dt ln 10| < 3e-3: the series to x^5 is exact to 1e-18), else exp10
+__device__ __forceinline__ double scale_pow10(double mu, double dt) {
+    const double x = dt * LN10;
+    if (fabs(x) > 3e-3) return mu * exp10(dt);
+    return mu * fma(x, fma(x, fma(x, fma(x, fma(x, 1.0 / 120.0, 1.0 / 24.0), 1.0 / 6.0), 0.5), 1.0), 1.0);
+}
+
+// Choice of lam by GCV on rho 10^[-12, 12], mu = lam / rho_mu (theta and c2 belong to the scaling
+// rho_mu; ratio = rho / rho_mu). The first minimum of the grid (ties to the smaller lam) is that of
+// the FP64 values: an FP32 scan, whose values are exact to 1e-5 (sums of at most 64 positive terms
+// with a few roundings each), leaves the points within 1e-4 of its minimum, and those are compared
+// in FP64, one warp per point with the terms over the lanes; many such points (a plateau) take one
+// thread each. Then safeguarded Newton steps on dG/dt = 0 between the neighbours, t = log10 mu:
+// FP32 steps to a starting point, then FP64 steps that carry mu itself (an FP64 exponential per step
+// would cost as much as the step); where the five FP64 values around the minimum agree to 1e-13
+// the grid point stands. The result is sh.mu. All threads call; ends with a barrier.
+struct GcvShared {
+    float val[GRID_POINTS];   // FP32 grid (0: not usable)
+    double grid[GRID_POINTS]; // FP64 values of the candidates, else DBL_MAX
+    int cand[GRID_POINTS];
+    float wmin[NW];
+    int count, ig, check;
+    double mu;
+};
+// the grid 10^(-12 + 24 i / 199), passed to the kernel as a parameter
+struct GcvGrid {
+    double v[GRID_POINTS];
+};
+
+__device__ void gcv_lambda(const Spec &S, const SpecF &SF, const GcvGrid &grid, double ratio, GcvShared &sh) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    constexpr float stepf = (float)(2.0 * BRACKET_DECADES / (GRID_POINTS - 1)), lof = (float)-BRACKET_DECADES;
+    const float ratiof = (float)ratio;
+    float v = 3.4e38f;
+    if (tid < GRID_POINTS) {
+        float N, D;
+        grid_nd(SF, exp10f(fmaf((float)tid, stepf, lof)) * ratiof, N, D);
+        const float g = N / (D * D);
+        const bool ok = N > 1e-36f && D * D > 1e-36f && g < 3e38f;
+        sh.val[tid] = ok ? g : 0.0f;
+        if (ok) v = g;
+        sh.grid[tid] = DBL_MAX;
+    }
+    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (lane == 0) sh.wmin[wid] = v;
+    if (tid == 0) sh.count = 0;
+    __syncthreads();
+    v = sh.wmin[0];
+    for (int w = 1; w < NW; ++w) v = fminf(v, sh.wmin[w]);
+    if (tid < GRID_POINTS && sh.val[tid] <= v * 1.0001f) sh.cand[atomicAdd(&sh.count, 1)] = tid;
+    __syncthreads();
+    auto value = [&](int gi) {  // by a warp, the terms over its lanes
+        double N, D;
+        lam_terms_nd(S, grid.v[gi] * ratio, N, D);
+        warp_sum2(N, D);
+        return gcv_value(N, D);
+    };
+    if (sh.count <= 4 * NW) {
+        for (int c = wid; c < sh.count; c += NW) {
+            const double g = value(sh.cand[c]);
+            if (lane == 0) sh.grid[sh.cand[c]] = g;
+        }
+    } else if (tid < sh.count) {
+        const int gi = sh.cand[tid];
+        const double mu = grid.v[gi] * ratio;
+        double N = 0.0, D = 0.0;
+        for (int i = 0; i < S.K; ++i) {
+            const double th = S.theta[i], am = 1.0 - th, d = th + mu * am;
+            const double g = d > 0.0 ? mu * am / d : 1.0;
+            N += S.c2[i] * g * g;
+            D += g;
+        }
+        sh.grid[gi] = gcv_value(N, D);
+    }
+    __syncthreads();
+    if (wid == 0) {
+        double bv = DBL_MAX;
+        int ig = GRID_POINTS;
+        for (int gi = lane; gi < GRID_POINTS; gi += 32)
+            if (sh.grid[gi] < bv) {
+                bv = sh.grid[gi];
+                ig = gi;
+            }
+        for (int o = 16; o > 0; o >>= 1) {
+            const double bo = __shfl_xor_sync(0xffffffffu, bv, o);
+            const int io = __shfl_xor_sync(0xffffffffu, ig, o);
+            if (bo < bv || (bo == bv && io < ig)) {
+                bv = bo;
+                ig = io;
+            }
+        }
+        if (ig >= GRID_POINTS) ig = 0;
+        // flat to rounding only if the FP32 neighbours are within their error of it
+        bool check = true;
+        for (int w = -(NREF / 2); w <= NREF / 2; ++w) {
+            const float q = sh.val[min(max(ig + w, 0), GRID_POINTS - 1)];
+            if (q > v * 1.0001f) check = false;
+        }
+        if (lane == 0) {
+            sh.ig = ig;
+            sh.check = check;
+        }
+    }
+    __syncthreads();
+    const int ig = sh.ig;
+    if (sh.check) {
+        for (int w = wid; w < NREF; w += NW) {
+            const int gi = min(max(ig + w - NREF / 2, 0), GRID_POINTS - 1);
+            if (sh.grid[gi] != DBL_MAX) continue;
+            const double g = value(gi);
+            __syncwarp();
+            if (lane == 0) sh.grid[gi] = g;
+        }
+        __syncthreads();
+    }
+    if (wid == 0) {
+        const double bv = sh.grid[ig];
+        bool flat = false;
+        if (sh.check) {
+            double vmax = bv;
+            for (int w = -(NREF / 2); w <= NREF / 2; ++w) vmax = fmax(vmax, sh.grid[min(max(ig + w, 0), GRID_POINTS - 1)]);
+            flat = vmax - bv <= 1e-13 * bv;
+        }
+        const double mu0 = grid.v[ig] * ratio;
+        double mu = mu0;
+        if (!flat) {
+            // t is relative to the grid point, the bracket its neighbours
+            const float Af = ig > 0 ? -stepf : 0.f, Bf = ig < GRID_POINTS - 1 ? stepf : 0.f, muf = (float)mu0;
+            float tf = 0.f, Af0 = Af, Bf0 = Bf;
+            for (int it = 0; it < NEWTON32_MAX; ++it) {
+                float s[6], d1, d2;
+                const float m = exp10f(tf) * muf;
+                lam_terms6<float>(SF, m, s);
+                for (int k = 0; k < 6; ++k) s[k] = warp_sum_t(s[k]);
+                gcv_dt<float>(s, m, d1, d2);
+                if (d1 == 0.0f || !(d1 == d1)) break;
+                if (fabsf(d1) <= 1e-5f * gcv_dt_scale<float>(s, m)) break;  // at the rounding level
+                const float tn = newton_step<float>(tf, d1, d2, Af0, Bf0);
+                const float dt = fabsf(tn - tf);
+                tf = tn;
+                if (dt <= 1e-6f || Bf0 - Af0 <= 1e-6f) break;
+            }
+            double t = (double)tf, A1 = (double)Af, B1 = (double)Bf;
+            if (!(t > A1 && t < B1)) t = 0.0;
+            mu = mu0 * (t == 0.0 ? 1.0 : (double)exp10f(tf));  // t follows mu to FP32 accuracy: it only brackets
+            for (int it = 0; it < NEWTON_MAX; ++it) {
+                double s6[6];
+                lam_terms6<double>(S, mu, s6);
+                warp_sum6(s6);
+                // derivatives of G in mu times D^2: G1 D^2 = N1 - 2 N D1 / D, G2 D^2 = N2 - 4 N1 D1 / D -
+                // 2 N D2 / D + 6 N (D1 / D)^2, and in t: d1 = G1 mu ln10, d2 = (G2 mu + G1) mu ln10^2
+                const double iD = rcp_newton(s6[3]), u = s6[4] * iD, w = s6[0] * u;
+                const double g1 = s6[1] - 2.0 * w;
+                if (g1 == 0.0 || !(g1 == g1) || fabs(g1) <= 1e-12 * (fabs(s6[1]) + fabs(2.0 * w))) break;  // at the rounding level
+                const double g2 = s6[2] - u * (4.0 * s6[1] - 6.0 * w) - 2.0 * s6[0] * s6[5] * iD, q = fma(g2, mu, g1) * LN10;
+                if (g1 > 0.0) B1 = t;
+                else A1 = t;
+                double tn = t - g1 / q;
+                const bool pure = q > 0.0 && tn > A1 && tn < B1;
+                if (!pure) tn = 0.5 * (A1 + B1);
+                const double dt = fabs(tn - t);
+                mu = scale_pow10(mu, tn - t);
+                t = tn;
+                if (dt <= 1e-10 || B1 - A1 <= 1e-10) break;
+                if (pure && dt <= 1e-6) break;  // quadratic: the next step is ~1e-12
+            }
+            double N, D;
+            lam_terms_nd(S, mu, N, D);
+            warp_sum2(N, D);
+            if (!(gcv_value(N, D) <= bv)) mu = mu0;
+        }
+        if (lane == 0) sh.mu = mu;
+    }
+    __syncthreads();
+}
+
+// ------------------------------------------------------------ bordered eigenproblem
+// A GKS iteration appends one vector, so its Grams are the previous ones with one more row and
+// column. With Y the generalised eigenvectors of the previous pair scaled to Y^T (G_A + rho G_L) Y
+// = I (rho that of the first, full solve), Y^T G_A Y = diag(d), the new problem in the basis
+// [Y, w / nu], w = e_n - Y m, m = Y^T (new column of G_A + rho G_L), nu^2 = its new diagonal entry
+// - ||m||^2, is the bordered diagonal matrix [diag(d) c; c^T gam], whose eigenvalues are the
+// roots of the secular equation F(x) = x - gam - sum c_i^2 / (x - d_i) = 0, one between any two
+// neighbouring poles and one beyond each end. A root is held as its distance mu from the nearest
+// pole, found in FP32 by interpolation with two poles (four threads per root) and then by FP64
+// Newton steps on mu F. The borders c that have exactly the computed roots follow from
+// c_i^2 = prod_j (x_j - d_i) / prod_{j != i} (d_j - d_i) (Loewner; Gu and Eisenstat 1995), so
+// the eigenvectors c_i / (x_j - d_i) are orthogonal to rounding however close the roots are.
+// One product of n x n matrices updates Y; all else is O(n^2). Entries with |c_i| at the rounding
+// level of the matrix are eigenpairs already. Poles closer than that, a nearly dependent new
+// vector or a root that did not converge leave the call to the full solve.
+constexpr int BE_NV = 14;        // vectors of the bordered solve in shared memory
+constexpr int BE_PART = 2 * ST;  // doubles of its partial sums
+struct BorderShared {
+    double gam, eta, inu, tol;
+    int p, bad;
+};
+
+// One interpolation step of a root in FP32 by four adjacent lanes (sub = 0..3, all of the warp
+// call): poles de[i] (relative to the origin pole o), squared borders z2[i], the first k poles left
+// of the root; e = origin - gam. Returns F, the proposal in x and the size of F's terms.
+__device__ float be_step32(const float *de, const float *z2, int p, int k, int o, float e, float m, int sub, float &x, float &size) {
+    float P = 0.f, Pp = 0.f, R = 0.f, Rp = 0.f;
+#pragma unroll 4
+    for (int i = sub; i < p; i += 4) {
+        const float q = __fdividef(1.0f, m - de[i]), t = z2[i] * q, t2 = t * q;
+        const bool left = i < k;
+        P -= left ? t : 0.f;
+        Pp += left ? t2 : 0.f;
+        R -= left ? 0.f : t;
+        Rp += left ? 0.f : t2;
+    }
+#pragma unroll
+    for (int w = 1; w < 4; w <<= 1) {
+        P += __shfl_xor_sync(0xffffffffu, P, w);
+        Pp += __shfl_xor_sync(0xffffffffu, Pp, w);
+        R += __shfl_xor_sync(0xffffffffu, R, w);
+        Rp += __shfl_xor_sync(0xffffffffu, Rp, w);
+    }
+    const float F = e + m + P + R;
+    size = fabsf(e) + fabsf(m) + fabsf(P) + fabsf(R);
+    if (k == 0 || k == p) {  // one pole, at the origin: x^2 + C x = a
+        const float a = (k == 0 ? Rp : Pp) * m * m, C = e + (k == 0 ? R : P) + a / m;
+        const float ds = sqrtf(fmaf(C, C, 4.0f * a));
+        if (k == 0) x = C >= 0.f ? -0.5f * (C + ds) : 2.0f * a / (C - ds);
+        else x = C <= 0.f ? 0.5f * (ds - C) : 2.0f * a / (C + ds);
+        return F;
+    }
+    const float dL = de[k - 1], dR = de[k];
+    const float a = Pp * (m - dL) * (m - dL), pc = P + a / (m - dL);
+    const float b = (1.0f + Rp) * (dR - m) * (dR - m), qc = m + R - b / (dR - m);
+    const float C = e + pc + qc, W = o == k - 1 ? dR : dL, t = o == k - 1 ? a : b;
+    const float B = fmaf(C, W, a + b), ds = sqrtf(fmaxf(fmaf(B, B, -4.0f * C * t * W), 0.f));
+    x = B > 0.f ? 2.0f * t * W / (B + ds) : (B - ds) / (2.0f * C);
+    return F;
+}
+
+// Updates Y (K - 1 x K - 1 in Ym, the result K x K in Yo; row stride lds) with its eigenvalues d
+// and the components gh = Y^T g to K, for the new last row and column of G_A, G_L and entry of g.
+// Q: K x K scratch; v: BE_NV vectors of lds; part: BE_PART doubles. False: not possible (d, gh, Ym are
+// as they were).
+__device__ bool be_update(const double *GA, const double *GL, const double *g, int ld, int K, double rho, double *Ym, double *Yo,
+                          double *Q, int lds, double *d, double *gh, double *v, double *part, BorderShared &sh) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, n = K - 1;
+    double *av = v, *mv = v + lds, *ah = v + 2 * lds, *mh = v + 3 * lds, *c = v + 4 * lds, *yw = v + 5 * lds;
+    double *D = v + 6 * lds, *Z = v + 7 * lds, *Z2 = av, *mu = v + 8 * lds, *ct = v + 9 * lds, *nrm = v + 10 * lds, *nd = v + 11 * lds;
+    int *map = reinterpret_cast<int *>(v + 12 * lds), *org = map + lds;
+    float *zf = reinterpret_cast<float *>(v + 13 * lds);
+    float *df = reinterpret_cast<float *>(Q);  // [root][pole], free until Q is formed
+    for (int i = tid; i < n; i += ST) {
+        const double x = GA[i * ld + n];
+        av[i] = x;
+        mv[i] = fma(rho, GL[i * ld + n], x);
+    }
+    if (tid == 0) sh.bad = 0;
+    __syncthreads();
+    row_sums2(n, n, part,  // Y^T (new columns)
+              [&](int j, int r, double &x, double &y) {
+                  const double q = Ym[r * lds + j];
+                  x += q * av[r];
+                  y += q * mv[r];
+              },
+              [&](int j, double x, double y) {
+                  ah[j] = x;
+                  mh[j] = y;
+              });
+    row_sums(n, n, part, [&](int r, int j) { return Ym[r * lds + j] * mh[j]; }, [&](int r, double x) { yw[r] = x; });  // Y m
+    if (wid == 0) {
+        double mm = 0.0, ma = 0.0, tm = 0.0, mg = 0.0;
+        for (int i = lane; i < n; i += 32) {
+            const double m = mh[i];
+            mm += m * m;
+            ma += m * ah[i];
+            tm += d[i] * m * m;
+            mg += m * gh[i];
+        }
+        warp_sum2(mm, ma);
+        warp_sum2(tm, mg);
+        const double al = GA[n * ld + n], mnn = fma(rho, GL[n * ld + n], al), nu2 = mnn - mm;
+        const bool ok = nu2 > 1e-8 * mnn && isfinite(nu2);
+        const double inu = ok ? rsqrt(nu2) : 0.0, gam = (al - 2.0 * ma + tm) * inu * inu;
+        float big = fabsf((float)gam);
+        for (int i = lane; i < n; i += 32) {
+            const double x = (ah[i] - d[i] * mh[i]) * inu;
+            c[i] = x;
+            big = fmaxf(big, fmaxf(fabsf((float)x), fabsf((float)d[i])));
+        }
+        big = warp_maxf(big);
+        if (lane == 0) {
+            sh.gam = gam;
+            sh.inu = inu;
+            sh.eta = (g[n] - mg) * inu;
+            sh.tol = 16.0 * 2.22e-16 * (double)big;
+            if (!ok || !(big < 1e6f)) sh.bad = 1;
+        }
+    }
+    __syncthreads();
+    const double gam = sh.gam, tol = sh.tol, inu = sh.inu, eta = sh.eta;
+    // the poles that take part, in ascending order
+    if (tid == 0) sh.p = 0;
+    __syncthreads();
+    // (as integers in the order of the doubles: an FP64 comparison holds the pipe like an addition)
+    long long *key = reinterpret_cast<long long *>(mu);
+    if (tid < n) {
+        const long long q = __double_as_longlong(d[tid]);
+        key[tid] = fabs(c[tid]) > tol ? (q ^ ((q >> 63) & 0x7fffffffffffffffll)) : 0x7fffffffffffffffll;
+    }
+    __syncthreads();
+    if (tid < n && key[tid] != 0x7fffffffffffffffll) {
+        int rank = 0;
+        const double x = d[tid];
+        const long long kt = key[tid];
+        for (int j = 0; j < n; ++j) rank += key[j] < kt || (key[j] == kt && j < tid);
+        D[rank] = x;
+        Z[rank] = c[tid];
+        map[rank] = tid;
+        atomicAdd(&sh.p, 1);
+    }
+    __syncthreads();
+    const int p = sh.p;
+    if (tid + 1 < p && D[tid + 1] - D[tid] <= 4.0 * tol) sh.bad = 1;
+    if (tid < p) {
+        Z2[tid] = Z[tid] * Z[tid];
+        zf[tid] = (float)Z2[tid];
+    }
+    if (tid <= p) org[tid] = max(tid - 1, 0);
+    if (p == 0 && tid == 0) sh.bad = 1;
+    __syncthreads();
+    if (sh.bad) return false;
+    // roots in FP32, four threads each: first the pole it is nearer to
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int e = tid; e < (p + 1) * p; e += ST) {
+            const int k = e / p, i = e - k * p;
+            df[e] = (float)(D[i] - D[org[k]]);
+        }
+        __syncthreads();
+        if (pass == 0) {
+            const int k = min(max(tid >> 2, 1), p);  // (threads of no interior root repeat another's)
+            const float *de = df + k * p;
+            float x, size;
+            const float gap = k < p ? de[k] : 1.f;
+            const float F = be_step32(de, zf, p, k, k - 1, (float)(D[k - 1] - gam), 0.5f * gap, tid & 3, x, size);
+            __syncthreads();
+            if ((tid & 3) == 0 && (tid >> 2) == k && k < p && !(F >= 0.f)) org[k] = k;
+        }
+        __syncthreads();
+    }
+    {
+        const int k = min(tid >> 2, p), o = org[k];
+        const float *de = df + k * p, e = (float)(D[o] - gam);
+        float A, B;
+        if (k == 0 || k == p) {  // |x - pole| <= |pole - gam| + ||c||
+            float z = 0.f;
+            for (int i = 0; i < p; ++i) z += zf[i];
+            const float w = fabsf(e) + sqrtf(z) * 1.0001f + 1e-30f;
+            A = k == 0 ? -w : 0.f;
+            B = k == 0 ? 0.f : w;
+        } else {
+            A = o == k ? 0.5f * de[k - 1] : 0.f;
+            B = o == k ? 0.f : 0.5f * de[k];
+        }
+        float m = 0.5f * (A + B);
+        bool on = true;
+        for (int it = 0; it < 32 && __any_sync(0xffffffffu, on); ++it) {
+            float x, size;
+            const float F = be_step32(de, zf, p, k, o, e, m, tid & 3, x, size);
+            if (!on) continue;
+            if (fabsf(F) <= 2.4e-7f * size) {
+                on = false;
+                continue;
+            }
+            if (F > 0.f) B = m;
+            else A = m;
+            if (!(x > A && x < B)) x = 0.5f * (A + B);
+            on = fabsf(x - m) > 1e-6f * fabsf(x);
+            m = x;
+        }
+        if ((tid & 3) == 0 && (tid >> 2) <= p) mu[k] = (double)m;
+    }
+    __syncthreads();
+    // FP64: Newton steps on mu F(mu) = mu (origin - gam + mu - S1) - c_o^2, S1 and S2 the sums over
+    // the other poles; the terms of a root spread over the threads of its column of parts
+    const int RS = p + 1 <= 32 ? 32 : 64, parts = ST / RS, root = tid & (RS - 1), pt = tid / RS;
+    for (int it = 0; it < 8; ++it) {
+        double S1 = 0.0, S2 = 0.0;
+        const bool on = root <= p;
+        const int o = on ? org[root] : 0;
+        const double m = on ? mu[root] : 1.0, Do = D[o];
+        if (on)
+            for (int i = pt; i < p; i += parts) {
+                if (i == o) continue;
+                const double q = rcp_newton(m - (D[i] - Do)), t = Z2[i] * q;
+                S1 += t;
+                S2 += t * q;
+            }
+        part[tid] = S1;
+        part[ST + tid] = S2;
+        __syncthreads();
+        int more = 0;
+        if (tid <= p) {  // (the first p + 1 threads are part 0 of every root)
+            for (int q = 1; q < parts; ++q) {
+                S1 += part[q * RS + tid];
+                S2 += part[ST + q * RS + tid];
+            }
+            const double r = (Do - gam) + m - S1, z = Z2[o], h = m * r - z, hp = r + m + m * S2;
+            double x = m - h / hp;
+            // the root stays on its side of the pole and short of the next one
+            const double lim = root == 0 || root == p ? 1e30 : 0.75 * (D[root] - D[root - 1]);
+            if (!(x * m > 0.0 && fabs(x) < lim)) {
+                x = m;
+                if (it > 2) sh.bad = 1;
+            }
+            const double dx = fabs(x - m);
+            mu[tid] = x;
+            more = dx > 1e-9 * fabs(x);  // quadratic: the next step would be at the rounding level
+            if (it == 7 && more) sh.bad = 1;
+        }
+        if (!__syncthreads_or(more)) break;
+    }
+    if (sh.bad) return false;
+    // Loewner borders: products over the roots in parts, each factor a quotient near 1
+    {
+        const int i = root;
+        double pr = 1.0;
+        if (i < p)
+            for (int j = pt; j < p; j += parts) {
+                const double f = (D[org[j]] - D[i]) + mu[j];
+                pr *= j == i ? f : f * rcp_newton(D[j] - D[i]);
+            }
+        part[tid] = pr;
+        __syncthreads();
+        if (tid < p) {
+            for (int q = 1; q < parts; ++q) pr *= part[q * RS + tid];
+            pr *= (D[org[p]] - D[tid]) + mu[p];
+            const double x = sqrt(fabs(pr));
+            ct[tid] = Z[tid] < 0.0 ? -x : x;
+        }
+        __syncthreads();
+    }
+    // eigenvectors c_i / (x_j - d_i) (the last component 1) and their norms
+    for (int e = tid; e < p * (p + 1); e += ST) {
+        const int i = e / (p + 1), j = e - i * (p + 1);
+        Q[i * lds + j] = ct[i] * rcp_newton((D[org[j]] - D[i]) + mu[j]);
+    }
+    __syncthreads();
+    row_sums2(p + 1, p, part,
+              [&](int j, int i, double &x, double &y) {
+                  const double q = Q[i * lds + j];
+                  x += q * q;
+                  y += q * gh[map[i]];
+              },
+              [&](int j, double x, double y) {
+                  const double f = rsqrt(1.0 + x);
+                  nrm[j] = f;
+                  ah[j] = (y + eta) * f;  // component of g
+                  nd[j] = D[org[j]] + mu[j];
+              });
+    // Yo = [Y, w / nu] Q: rows 0..n-1, then the last row (0, ..., 0, 1 / nu)
+    for (int e = tid; e < n * (p + 1); e += ST) {
+        const int r = e / (p + 1), j = e - r * (p + 1);
+        double x = -yw[r] * inu;
+        for (int i = 0; i < p; ++i) x += Ym[r * lds + map[i]] * Q[i * lds + j];
+        Yo[r * lds + j] = x * nrm[j];
+    }
+    for (int j = tid; j <= p; j += ST) Yo[n * lds + j] = inu * nrm[j];
+    // eigenpairs that the border leaves alone, behind the others
+    if (wid == 0) {
+        int at = p + 1;
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane;
+            const bool still = i < n && !(fabs(c[i]) > tol);
+            const unsigned m = __ballot_sync(0xffffffffu, still);
+            if (still) {
+                const int j = at + __popc(m & ((1u << lane) - 1u));
+                nd[j] = d[i];
+                ah[j] = gh[i];
+                for (int r = 0; r < n; ++r) Yo[r * lds + j] = Ym[r * lds + i];
+                Yo[n * lds + j] = 0.0;
+            }
+            at += __popc(m);
+        }
+    }
+    __syncthreads();
+    for (int j = tid; j < K; j += ST) {
+        d[j] = nd[j];
+        gh[j] = ah[j];
+    }
+    __syncthreads();
+    return true;
+}
+
 }  // namespace
 
-__global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
+__global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a, const __grid_constant__ GcvGrid grid) {
     extern __shared__ double sm[];
-    __shared__ double s_rho, s_rho0sq, s_t, s_scale;
-    __shared__ double s_grid[GRID_POINTS];
+    __shared__ double s_rho, s_rho0sq, s_t, s_scale, s_lam;
+    __shared__ GcvShared s_gcv;
+    __shared__ BorderShared s_be;
     __shared__ float s_redf[NW];
     __shared__ int s_fail, s_flag, s_idx[NW], s_end[4];
     __shared__ JacobiShared<float> jf;
@@ -662,6 +1208,8 @@ __global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
     double *vec = Em + lds * lds;
     double *theta = vec, *gh = vec + lds, *c2 = vec + 2 * lds, *invd = vec + 3 * lds, *hv = vec + 4 * lds;
     float *fvec = reinterpret_cast<float *>(vec + 5 * lds);  // 3 x lds floats within 2 x lds doubles
+    double *bv = vec + 7 * lds;                              // bordered solve: BE_NV vectors, partial sums
+    double *bpart = bv + BE_NV * lds;
     float *thf = fvec, *af = fvec + lds, *c2f = fvec + 2 * lds;
     float *Af = reinterpret_cast<float *>(Tm);
     float *Wf = reinterpret_cast<float *>(Em);
@@ -687,6 +1235,105 @@ __global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
     }
     __syncthreads();
     const double rho = s_rho;
+    // lambda by GCV for theta = clamped eigenvalues raw[] in the scaling rho_mu and components gh
+    auto choose_gcv = [&](const double *raw, double rho_mu) {
+        for (int i = tid; i < K; i += ST) {
+            const double x = fmin(fmax(raw[i], 0.0), 1.0);
+            theta[i] = x;
+            c2[i] = x > THETA_TINY ? gh[i] * gh[i] / x : 0.0;
+        }
+        __syncthreads();
+        if (wid == 0) {
+            double kept = 0.0, unused = 0.0;
+            for (int i = lane; i < K; i += 32) kept += c2[i];
+            warp_sum2(kept, unused);
+            if (lane == 0) {
+                s_rho0sq = a.bb[b] - kept;
+                s_scale = kept > 0.0 ? 1.0 / kept : 1.0;
+            }
+        }
+        __syncthreads();
+        for (int i = tid; i < K; i += ST) {
+            thf[i] = (float)theta[i];
+            af[i] = (float)(1.0 - theta[i]);
+            c2f[i] = (float)(c2[i] * s_scale);
+        }
+        __syncthreads();
+        if (a.rule != MOF_RULE_GCV) return;
+        if (tid == 0) s_t = rho / rho_mu;
+        __syncthreads();
+        gcv_lambda(Spec{K, rho, s_rho0sq, theta, c2}, SpecF{K, thf, af, c2f}, grid, s_t, s_gcv);
+        if (tid == 0) s_lam = s_gcv.mu * rho_mu;
+        __syncthreads();
+    };
+    // ---------------------------------------------- 0. from the previous call's eigenvectors
+    bool bordered = false;
+    double lam = a.lam_fixed;
+    if (a.Y) {
+        double *Yg = a.Y + (long long)b * ld * ld, *dg = a.Yd + (long long)b * ld, *hg = a.Yh + (long long)b * ld;
+        const int nY = a.nY[b];
+        const double rho0 = a.Yrho[b];
+        if (nY > 0 && (nY == K || nY == K - 1)) {
+            for (int e = tid; e < nY * nY; e += ST) {
+                const int i = e / nY, j = e - i * nY;
+                AT(Cm, i, j) = Yg[i * ld + j];
+            }
+            for (int i = tid; i < nY; i += ST) {
+                hv[i] = dg[i];
+                gh[i] = hg[i];
+            }
+            __syncthreads();
+            double *Ym = Cm;
+            bordered = nY == K;
+            if (!bordered) {
+                bordered = be_update(GA, GL, g, ld, K, rho0, Cm, Tm, Um, lds, hv, gh, bv, bpart, s_be);
+                Ym = Tm;
+            }
+            if (bordered) {
+                if (nY != K) {
+                    for (int e = tid; e < K * K; e += ST) {
+                        const int i = e / K, j = e - i * K;
+                        Yg[i * ld + j] = AT(Tm, i, j);
+                    }
+                    for (int i = tid; i < K; i += ST) {
+                        dg[i] = hv[i];
+                        hg[i] = gh[i];
+                    }
+                    if (tid == 0) a.nY[b] = K;
+                }
+                choose_gcv(hv, rho0);
+                lam = s_lam;
+                const double mu = lam / rho0;
+                // z = Y diag(1 / (theta + mu (1 - theta))) Y^T g, and one step of refinement with the
+                // residual of (G_A + lam G_L) z = g
+                double *w = bv, *zz = bv + lds, *rr = bv + 2 * lds;
+                for (int i = tid; i < K; i += ST) w[i] = gh[i] / (theta[i] + mu * (1.0 - theta[i]));
+                __syncthreads();
+                row_sums(K, K, bpart, [&](int i, int k) { return AT(Ym, i, k) * w[k]; }, [&](int i, double t) { zz[i] = t; });
+                row_sums2(K, K, bpart,
+                          [&](int i, int k, double &x, double &y) {  // (the Grams are stored symmetric)
+                              x += GA[k * ld + i] * zz[k];
+                              y += GL[k * ld + i] * zz[k];
+                          },
+                          [&](int i, double x, double y) { rr[i] = g[i] - (x + lam * y); });
+                row_sums(K, K, bpart, [&](int j, int r) { return AT(Ym, r, j) * rr[r]; },
+                         [&](int j, double t) { w[j] = t / (theta[j] + mu * (1.0 - theta[j])); });
+                row_sums(K, K, bpart, [&](int i, int k) { return AT(Ym, i, k) * w[k]; }, [&](int i, double t) { zz[i] += t; });
+                int bad = 0;
+                for (int i = tid; i < K; i += ST) {
+                    z[i] = gh[i] = zz[i];
+                    bad |= !isfinite(zz[i]);
+                }
+                if (__syncthreads_or(bad) && tid == 0) atomicOr(a.err, 2);
+                if (tid == 0) {
+                    a.lam[b] = lam;
+                    a.flag[b] = 0;
+                }
+            }
+        }
+    }
+    if (!bordered) {
+    __syncthreads();
     for (int e = tid; e < K * K; e += ST) {
         const int i = e / K, j = e - (e / K) * K;
         const double ga = GA[i * ld + j];
@@ -722,7 +1369,6 @@ __global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
     }
     __syncthreads();
 
-    double lam = a.lam_fixed;
     if (a.rule != MOF_RULE_FIXED) {
         // ------------------------------------------ 2a. FP32 Jacobi on C
         if (K <= 32) {  // registers only
@@ -774,122 +1420,24 @@ __global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
         __syncthreads();
 
         // ------------------------------------------ 2c. FP64 Jacobi polish
-        jacobi<double>(Um, lds, (double *)nullptr, lds, gh, K, Kp, JACOBI64_MAX_SWEEPS, 1e-16f, 1e-12f, jd, s_redf);
+        jacobi<double>(Um, lds, a.Y ? Xm : (double *)nullptr, lds, gh, K, Kp, JACOBI64_MAX_SWEEPS, 1e-16f, 1e-12f, jd, s_redf);
         for (int i = tid; i < K; i += ST) {
-            theta[i] = fmin(fmax(AT(Um, i, i), 0.0), 1.0);
-            c2[i] = theta[i] > THETA_TINY ? gh[i] * gh[i] / theta[i] : 0.0;
+            bv[i] = AT(Um, i, i);
+            if (a.Y) {
+                a.Yd[(long long)b * ld + i] = bv[i];
+                a.Yh[(long long)b * ld + i] = gh[i];
+            }
         }
         __syncthreads();
 
         // ------------------------------------------ 3-4. lambda
-        if (wid == 0) {
-            double kept = 0.0, unused = 0.0;
-            for (int i = lane; i < K; i += 32) kept += c2[i];
-            warp_sum2(kept, unused);
-            if (lane == 0) {
-                s_rho0sq = a.bb[b] - kept;
-                s_scale = kept > 0.0 ? 1.0 / kept : 1.0;
-            }
-        }
-        __syncthreads();
-        for (int i = tid; i < K; i += ST) {
-            thf[i] = (float)theta[i];
-            af[i] = (float)(1.0 - theta[i]);
-            c2f[i] = (float)(c2[i] * s_scale);
-        }
-        __syncthreads();
+        choose_gcv(bv, rho);
         const Spec S{K, rho, s_rho0sq, theta, c2};
         const SpecF SF{K, thf, af, c2f};
         const double lrho = log10(rho);
         const double lo = lrho - BRACKET_DECADES, hi = lrho + BRACKET_DECADES;
         const double step = (hi - lo) / (GRID_POINTS - 1);
-        if (a.rule == MOF_RULE_GCV) {
-            // GCV at every grid point in FP64 and its first minimum (ties to the smaller
-            // lambda), as the grid search defines it; a scan in lower precision can pick another
-            // of two nearly equal minima. One thread per point, its terms summed in order: a
-            // warp's FP64 instruction occupies the pipe as long with one active lane as with 32,
-            // so lanes over points take far fewer FP64 instructions than lanes over the terms
-            // with a reduction (and one exp10 per point instead of one per lane)
-            for (int gi = tid; gi < GRID_POINTS; gi += ST) {
-                const double mu = exp10(lo + gi * step) / rho;
-                double N = 0.0, D = 0.0;
-                for (int i = 0; i < S.K; ++i) {
-                    const double th = S.theta[i], am = 1.0 - th, d = th + mu * am;
-                    const double g = d > 0.0 ? mu * am / d : 1.0;
-                    N += S.c2[i] * g * g;
-                    D += g;
-                }
-                s_grid[gi] = gcv_value(N, D);
-            }
-            __syncthreads();
-            if (wid == 0) {
-                double bv = DBL_MAX;
-                int ig = GRID_POINTS;
-                for (int gi = lane; gi < GRID_POINTS; gi += 32)
-                    if (s_grid[gi] < bv) {
-                        bv = s_grid[gi];
-                        ig = gi;
-                    }
-                for (int o = 16; o > 0; o >>= 1) {
-                    const double bo = __shfl_xor_sync(0xffffffffu, bv, o);
-                    const int io = __shfl_xor_sync(0xffffffffu, ig, o);
-                    if (bo < bv || (bo == bv && io < ig)) {
-                        bv = bo;
-                        ig = io;
-                    }
-                }
-                if (ig >= GRID_POINTS) ig = 0;
-                bv = s_grid[ig];
-                double vmax = bv;  // the flatness test over the NREF points around the minimum
-                for (int w = -(NREF / 2); w <= NREF / 2; ++w) vmax = fmax(vmax, s_grid[min(max(ig + w, 0), GRID_POINTS - 1)]);
-                const bool flat = vmax - bv <= 1e-13 * bv;
-                // safeguarded Newton on dG/dt = 0 inside [t_{i-1}, t_{i+1}]: FP32 steps
-                // (in t - log10 rho) to a starting point, then FP64 steps on the full cell pair
-                const double A0 = lo + max(ig - 1, 0) * step, B0 = lo + min(ig + 1, GRID_POINTS - 1) * step;
-                float tf = (float)(ig * step - BRACKET_DECADES);
-                float Af0 = (float)(A0 - lrho), Bf0 = (float)(B0 - lrho);
-                for (int it = 0; it < (flat ? 0 : NEWTON32_MAX); ++it) {
-                    float s[6], d1, d2;
-                    const float mu = exp10f(tf);
-                    lam_terms6<float>(SF, mu, s);
-                    for (int k = 0; k < 6; ++k) s[k] = warp_sum_t(s[k]);
-                    gcv_dt<float>(s, mu, d1, d2);
-                    if (d1 == 0.0f || !(d1 == d1)) break;
-                    if (fabsf(d1) <= 1e-5f * gcv_dt_scale<float>(s, mu)) break;  // at the rounding level
-                    const float tn = newton_step<float>(tf, d1, d2, Af0, Bf0);
-                    const float dt = fabsf(tn - tf);
-                    tf = tn;
-                    if (dt <= 1e-6f || Bf0 - Af0 <= 1e-6f) break;
-                }
-                double t = lrho + (double)tf, A1 = A0, B1 = B0;
-                if (!(t > A1 && t < B1)) t = lo + ig * step;
-                for (int it = 0; it < (flat ? 0 : NEWTON_MAX); ++it) {
-                    double s6[6], d1, d2;
-                    const double mu = exp10(t) / rho;
-                    lam_terms6<double>(S, mu, s6);
-                    warp_sum6(s6);
-                    gcv_dt<double>(s6, mu, d1, d2);
-                    if (d1 == 0.0) break;
-                    if (fabs(d1) <= 1e-12 * gcv_dt_scale<double>(s6, mu)) break;  // at the rounding level
-                    const bool pure = d2 > 0.0 && t - d1 / d2 > A1 && t - d1 / d2 < B1;
-                    const double tn = newton_step<double>(t, d1, d2, A1, B1);
-                    const double dt = fabs(tn - t);
-                    t = tn;
-                    if (dt <= 1e-10 * fmax(1.0, fabs(t)) || B1 - A1 <= 1e-10 * fmax(1.0, fabs(t))) break;
-                    if (pure && dt <= 1e-6 * fmax(1.0, fabs(t))) break;  // quadratic: the next step is ~1e-12
-                }
-                if (flat) {
-                    t = lo + ig * step;
-                } else {
-                    double N, D;
-                    lam_terms_nd(S, exp10(t) / rho, N, D);
-                    warp_sum2(N, D);
-                    if (gcv_value(N, D) > bv) t = lo + ig * step;
-                }
-                if (lane == 0) s_t = t;
-            }
-            __syncthreads();
-        } else {  // DP on F(t) = N(mu(t)) + rho0^2 - (eta delta)^2, increasing in t
+        if (a.rule != MOF_RULE_GCV) {  // DP on F(t) = N(mu(t)) + rho0^2 - (eta delta)^2, increasing in t
             if (wid < 2) {  // the bracket ends, in FP64
                 double N, N1;
                 lam_terms_n<double>(S, exp10(wid ? hi : lo) / rho, N, N1);
@@ -955,10 +1503,13 @@ __global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
             } else if (tid == 0) {
                 s_t = flag == 1 ? lo : hi;
             }
-            if (tid == 0) s_flag = flag;
+            if (tid == 0) {
+                s_flag = flag;
+                s_lam = exp10(s_t);
+            }
             __syncthreads();
         }
-        lam = exp10(s_t);
+        lam = s_lam;
     }
     const double mu = lam / rho;
 
@@ -987,6 +1538,28 @@ __global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
             a.flag[b] = s_flag;
         }
     }
+    if (a.Y) {  // Y = R^-1 X for the next call: rows from the last on, one barrier each
+        __syncthreads();
+        for (int i = K - 1; i >= 0; --i) {
+            for (int j = tid; j < K; j += ST) AT(Xm, i, j) *= invd[i];
+            __syncthreads();
+            for (int e = tid; e < i * K; e += ST) {
+                const int k = e / K, j = e - k * K;
+                AT(Xm, k, j) -= AT(Rm, k, i) * AT(Xm, i, j);
+            }
+            __syncthreads();
+        }
+        double *Yg = a.Y + (long long)b * ld * ld;
+        for (int e = tid; e < K * K; e += ST) {
+            const int i = e / K, j = e - i * K;
+            Yg[i * ld + j] = AT(Xm, i, j);
+        }
+        if (tid == 0) {
+            a.Yrho[b] = rho;
+            a.nY[b] = K;
+        }
+    }
+    }  // !bordered
     if (!a.proj) return;
 
     // ---------------------------------------------- 6. proj = Mg^-1 ((G_A + lam G_L) z - g)
@@ -1000,42 +1573,27 @@ __global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
         AT(Tm, i, j) = (j <= i && i < n0) ? Li[i * ld + j] : 0.0;
     }
     __syncthreads();
-    // out_i = sum_k M(i, k) v_k, a warp per row, lanes over k
-    auto matvec = [&](double *out, int n, auto &&row) {
-        for (int i = wid; i < n; i += NW) {
-            double t = 0.0;
-            for (int k = lane; k < n; k += 32) t += row(i, k);
-            t = warp_sum(t);
-            if (lane == 0) out[i] = t;
-        }
-        __syncthreads();
-    };
     for (int r = n0; r < K; ++r) {  // Linv of [L 0; l^T d]: the row [-(l^T Linv) / d, 1 / d], l = Linv Mg[:, r]
-        matvec(lv, r, [&](int i, int k) { return k <= i ? AT(Tm, i, k) * Mg[k * ld + r] : 0.0; });
-        matvec(cv, r, [&](int i, int k) { return k >= i ? AT(Tm, k, i) * lv[k] : 0.0; });
+        row_sums(r, r, bpart, [&](int i, int k) { return k <= i ? AT(Tm, i, k) * Mg[k * ld + r] : 0.0; }, [&](int i, double t) { lv[i] = t; });
+        row_sums(r, r, bpart, [&](int i, int k) { return k >= i ? AT(Tm, k, i) * lv[k] : 0.0; }, [&](int i, double t) { cv[i] = t; });
         if (wid == 0) {
             double t = 0.0;
             for (int k = lane; k < r; k += 32) t += lv[k] * lv[k];
             t = warp_sum(t);
-            const double id = 1.0 / sqrt(fmax(Mg[r * ld + r] - t, 1e-300));
+            const double id = rsqrt(fmax(Mg[r * ld + r] - t, 1e-300));
             for (int k = lane; k < r; k += 32) Li[r * ld + k] = AT(Tm, r, k) = -cv[k] * id;
             if (lane == 0) Li[r * ld + r] = AT(Tm, r, r) = id;
         }
         __syncthreads();
     }
-    // the Grams are symmetric: entry (i, k) is read as (k, i)'s mirror, lanes over k
-    for (int i = wid; i < K; i += NW) {
-        double sa = 0.0, sl = 0.0;
-        for (int k = lane; k < K; k += 32) {
-            sa += GA[i * ld + k] * zs[k];
-            sl += GL[i * ld + k] * zs[k];
-        }
-        warp_sum2(sa, sl);
-        if (lane == 0) cv[i] = sa + lam * sl - g[i];
-    }
-    __syncthreads();
-    matvec(lv, K, [&](int i, int k) { return k <= i ? AT(Tm, i, k) * cv[k] : 0.0; });
-    matvec(zs, K, [&](int i, int k) { return k >= i ? AT(Tm, k, i) * lv[k] : 0.0; });
+    row_sums2(K, K, bpart,
+              [&](int i, int k, double &x, double &y) {  // (the Grams are stored symmetric)
+                  x += GA[k * ld + i] * zs[k];
+                  y += GL[k * ld + i] * zs[k];
+              },
+              [&](int i, double x, double y) { cv[i] = x + lam * y - g[i]; });
+    row_sums(K, K, bpart, [&](int i, int k) { return k <= i ? AT(Tm, i, k) * cv[k] : 0.0; }, [&](int i, double t) { lv[i] = t; });
+    row_sums(K, K, bpart, [&](int i, int k) { return k >= i ? AT(Tm, k, i) * lv[k] : 0.0; }, [&](int i, double t) { zs[i] = t; });
     for (int i = tid; i < K; i += ST) a.proj[(long long)b * ld + i] = zs[i];
     if (tid == 0) a.nL[b] = K;
 #undef AT
@@ -1044,7 +1602,7 @@ __global__ void __launch_bounds__(ST, 1) k_small_solve(SmallArgs a) {
 
 static size_t small_smem(int ld) {
     const size_t lds = (size_t)((ld + 1) | 1);
-    return sizeof(double) * (6 * lds * lds + 7 * lds);
+    return sizeof(double) * (6 * lds * lds + (7 + BE_NV) * lds + BE_PART);
 }
 
 mof_status prepare_small_solve(int ld) {
@@ -1062,8 +1620,13 @@ mof_status prepare_small_solve(int ld) {
 }
 
 mof_status launch_small_solve(const SmallArgs &a, cudaStream_t st) {
+    static const GcvGrid grid = [] {
+        GcvGrid g;
+        for (int i = 0; i < GRID_POINTS; ++i) g.v[i] = std::pow(10.0, -BRACKET_DECADES + i * (2.0 * BRACKET_DECADES / (GRID_POINTS - 1)));
+        return g;
+    }();
     const size_t smem = small_smem(a.ld);
-    ::mof::count_launch(), k_small_solve<<<a.B, ST, smem, st>>>(a);
+    ::mof::count_launch(), k_small_solve<<<a.B, ST, smem, st>>>(a, grid);
     MOF_LAUNCH_CHECK();
     return MOF_OK;
 }

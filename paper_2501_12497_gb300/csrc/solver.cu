@@ -136,8 +136,8 @@ struct WS {
     // ---- Solve-OF (P pairs)
     real *ux, *uy, *ut, *bof, *Vof, *Uof, *AtB, *wv, *wu, *y1, *y2, *sof, *vnew_of, *q_of;
     double *GA, *GL, *gof, *zof, *gam, *nrm_of, *coef_of, *coefU_of, *scale_of, *alpha_of, *alpha1_of, *beta_of,
-        *beta1_of, *bb_of, *Mg_of, *Linv_of, *pres_of;
-    int *Kv_of, *Ku_of, *grow_of, *gkb_of, *act_of, *app_of, *flag_of, *nL_of, *done_of;
+        *beta1_of, *bb_of, *Mg_of, *Linv_of, *pres_of, *Y_of, *Yd_of, *Yh_of, *Yrho_of;
+    int *Kv_of, *Ku_of, *grow_of, *gkb_of, *act_of, *app_of, *flag_of, *nL_of, *done_of, *nY_of;
     real *wf_of = nullptr, *wl_of = nullptr;  // IRLS weights of Solve-OF with p = q = 1 (P ns, 4 P ns)
     double *rn_of = nullptr;                  // norm^2 of its residual before orthogonalisation (P)
     int pq1 = 0;                              // workspace holds the p = q = 1 arrays
@@ -417,6 +417,11 @@ static mof_status ensure_ws(mof_problem *p, const mof_solver_params &prm, int n_
         w->app_of = a.take<int>(P);
         w->flag_of = a.take<int>(P);
         w->nL_of = a.take<int>(P);
+        w->nY_of = a.take<int>(P);
+        w->Y_of = a.take<double>((size_t)P * Kof * Kof);
+        w->Yd_of = a.take<double>((size_t)P * Kof);
+        w->Yh_of = a.take<double>((size_t)P * Kof);
+        w->Yrho_of = a.take<double>(P);
         w->done_of = a.take<int>(P);
         w->wf_of = a.take<real>(w->pq1 ? P * ns : 0);
         w->wl_of = a.take<real>(w->pq1 ? 4 * P * ns : 0);
@@ -616,13 +621,17 @@ __global__ void k_of_resid(const real *__restrict__ ux, const real *__restrict__
 // would store, up to rounding. The small solver forms d by the inverse of Mg's Cholesky factor,
 // one row longer with every append (48 us per iteration of 7 pairs in FP64 for a factorisation and
 // two triangular solves in one warp; 6 us of the small solve as matrix-vector products).
-// Also the inverse Cholesky factor of Mg over the first K vectors (I) and no appended vector
-// waiting for its scale (slot = -1).
-__global__ void k_of_mg_init(double *__restrict__ Mg, double *__restrict__ Linv, int *__restrict__ nL, const int *__restrict__ K,
+// Also the inverse Cholesky factor of Mg over the first K vectors (I), no appended vector
+// waiting for its scale (slot = -1) and no eigenvectors of the small problem yet (nY = 0).
+__global__ void k_of_mg_init(double *__restrict__ Mg, double *__restrict__ Linv, int *__restrict__ nL, int *__restrict__ nY,
+                             const int *__restrict__ K,
                              int *__restrict__ slot, int ld, const int *__restrict__ act, int B) {
     const int b = blockIdx.x;
     if (b >= B) return;
-    if (threadIdx.x == 0) slot[b] = -1;
+    if (threadIdx.x == 0) {
+        slot[b] = -1;
+        nY[b] = 0;
+    }
     if (act && !act[b]) return;
     double *M = Mg + (long long)b * ld * ld, *L = Linv + (long long)b * ld * ld;
     for (int e = threadIdx.x; e < ld * ld; e += blockDim.x) M[e] = L[e] = (e / ld == e % ld) ? 1.0 : 0.0;
@@ -1513,7 +1522,7 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
         const int gram_ctas = (int)((ns + ofc<real>() - 1) / ofc<real>());
         const int gram_red = (2 * Kof + 1 + 7) / 8;
         real *wfg = pq1 ? w.wf_of + (long long)b0 * ns : nullptr, *wlg = pq1 ? w.wl_of + (long long)b0 * 4 * ns : nullptr;
-        ::mof::count_launch(), k_of_mg_init<<<nb, 256, 0, gst>>>(w.Mg_of + b0 * KK, w.Linv_of + b0 * KK, w.nL_of + b0, Kvg,
+        ::mof::count_launch(), k_of_mg_init<<<nb, 256, 0, gst>>>(w.Mg_of + b0 * KK, w.Linv_of + b0 * KK, w.nL_of + b0, w.nY_of + b0, Kvg,
                                                                   reinterpret_cast<int *>(kg.aux), Kof, actg, nb);
         // the one-pass projection with the Gram column needs 16-byte aligned component segments
         const bool pass_ok = !pq1 && Kof <= 64 && of_pass_applicable<real>(ns, Vg, wvg);
@@ -1534,6 +1543,13 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
         sa.Mg = w.Mg_of + b0 * KK;
         sa.Linv = w.Linv_of + b0 * KK;
         sa.nL = w.nL_of + b0;
+        if (!pq1) {  // (with p = q = 1 all Grams change every iteration)
+            sa.Y = w.Y_of + b0 * KK;
+            sa.Yd = w.Yd_of + (long long)b0 * Kof;
+            sa.Yh = w.Yh_of + (long long)b0 * Kof;
+            sa.Yrho = w.Yrho_of + b0;
+            sa.nY = w.nY_of + b0;
+        }
         BasisRef<real> BS{Vg, N2, Kof, nb, Kvg, nullptr};
         const int wg_ctas = (int)std::min<long long>(WG_CTAS, (ns + WG_P - 1) / WG_P);
         for (int it = 0; it < prm.of_iters; ++it) {

@@ -158,6 +158,11 @@ struct SmallArgs {
     double *Linv;
     int *nL;
     double *proj;          // [B][ld] out
+    // State between the calls of one basis that grows by at most a vector per call while its Grams
+    // stay as they are (null: none): generalised eigenvectors Y [B][ld][ld], their eigenvalues Yd,
+    // Yh = Y^T g, the scaling Yrho and their number nY (zero before the first call).
+    double *Y, *Yd, *Yh, *Yrho;
+    int *nY;
 };
 mof_status launch_small_solve(const SmallArgs &a, cudaStream_t st);
 // Raise the kernel's dynamic shared-memory limit for leading dimension ld
