@@ -1215,8 +1215,8 @@ __global__ void k_of_fields(const real *__restrict__ u, int dr, real *__restrict
 // down `rows` rows, with the rows y - 1, y, y + 1 of the image and of u_{p+1} - u_p in registers; the
 // neighbours of a lane's V columns come from the adjacent lanes. Each image row is read twice
 // (as frame p and as frame p + 1 of pair p - 1, the second time from L2) plus two halo rows per strip.
-// ux and uy take their terms in the order of k_of_fields; ut sums three differences per row,
-// then three rows. V = 4 needs rows of a multiple of 4 pixels and 16-byte aligned arrays.
+// All sums take their terms in the order of k_of_fields (identical results: Solve-OF amplifies the
+// rounding of its fields a hundredfold). V = 4 needs rows of a multiple of 4 pixels and 16-byte aligned arrays.
 // What bounds it: DRAM (62 % of the copy rate with the first pass over u in the count). 1024x1024x64:
 // 250 us against 461 for shared-memory tiles that walk the frames in order; 256x256x32: 17 against
 // 52 us; 181x149x9: 9 against 17 us.
@@ -1271,25 +1271,20 @@ __global__ void __launch_bounds__(32 * FW) k_of_fields_rows(const real *__restri
 #pragma unroll
         for (int k = 0; k < V + 2; ++k) d[k] = g[k] - f[k];
     };
-    real f0[V + 2], f1[V + 2], f2[V + 2], d[V + 2], s0[V], s1[V], s2[V];
-    auto sum3 = [&](real (&o)[V]) {
-#pragma unroll
-        for (int k = 0; k < V; ++k) o[k] = d[k] + d[k + 1] + d[k + 2];
-    };
-    load(y0 - 1, f0, d);
-    sum3(s0);
-    load(y0, f1, d);
-    sum3(s1);
+    real f0[V + 2], f1[V + 2], f2[V + 2], d0[V + 2], d1[V + 2], d2[V + 2];
+    load(y0 - 1, f0, d0);
+    load(y0, f1, d1);
     const int ye = min(y0 + rows, ny);
     for (int y = y0; y < ye; ++y) {
-        load(y + 1, f2, d);
-        sum3(s2);
+        load(y + 1, f2, d2);
         real gx[V], gy[V], gt[V];
 #pragma unroll
         for (int k = 0; k < V; ++k) {
             gx[k] = ((f0[k + 2] - f0[k]) * half + (f1[k + 2] - f1[k]) * half + (f2[k + 2] - f2[k]) * half) / three;
             gy[k] = ((f2[k] - f0[k]) * half + (f2[k + 1] - f0[k + 1]) * half + (f2[k + 2] - f0[k + 2]) * half) / three;
-            gt[k] = (s0[k] + s1[k] + s2[k]) / (three * three);
+            real t = d0[k] + d0[k + 1] + d0[k + 2];
+            t = t + d1[k] + d1[k + 1] + d1[k + 2];
+            gt[k] = (t + d2[k] + d2[k + 1] + d2[k + 2]) / (three * three);
         }
         if (on) {
             const long long o = p * ns + (long long)y * nx + x;
@@ -1310,11 +1305,8 @@ __global__ void __launch_bounds__(32 * FW) k_of_fields_rows(const real *__restri
         for (int k = 0; k < V + 2; ++k) {
             f0[k] = f1[k];
             f1[k] = f2[k];
-        }
-#pragma unroll
-        for (int k = 0; k < V; ++k) {
-            s0[k] = s1[k];
-            s1[k] = s2[k];
+            d0[k] = d1[k];
+            d1[k] = d2[k];
         }
     }
 }
