@@ -392,195 +392,236 @@ __global__ void __launch_bounds__(SDT) k_sub_dot(const real *__restrict__ V, lon
 //   y  = Ups^T Ups x'                           (pointwise: u_c (u_x x'_x + u_y x'_y))
 //   dots  V^T x', V^T y, V^T q                  (q = L^T L r, the graph Laplacian of r, precomputed)
 //   scalars ||x'||^2, x'^T y, x'^T q, x'^T Ups^T b
-// A CTA owns OPX pixels of both components: TMA bulk copies stage, for each basis vector and for
-// r and q and Ups^T b, the two 1 KB segments of those pixels, and the segments of u_x and u_y,
-// completing on one mbarrier (bounded wait). The chunk partials (3 Kmax + 4 per chunk,
-// FP32 16-element partials accumulated with their rounding errors, FP64 across lanes) are
-// reduced by k_of_pass_finish. With x' = r - V d the new vector is v = x' / ||x'|| and its Gram
+// A CTA is one warp and owns every nparts-th tile of 512 bytes per component (128 FP32 pixels):
+// bulk copies stage, for each basis vector and for r, q and Ups^T b, the two segments of those
+// pixels, and the segments of u_x and u_y, on one mbarrier (bounded wait). A lane holds 16 bytes of
+// each component, so x', y and the dots need no barrier; the lanes' sums of eight vectors are
+// reduced together (9 shuffles each instead of 40), to one vector per lane, and are accumulated in
+// FP64 over the warp's tiles. Those totals (3 Kmax + 4 per warp) are reduced by k_of_pass_finish.
+// Bound by HBM once enough tiles are in flight, which one warp per tile gives: (K + 4) KB of shared
+// memory each, 6 to 16 warps per SM that load, compute and start the next load independently. 63
+// pairs of 1024^2, K = 10 to 28: 3.4 ms per pass (0.55 of the measured copy rate) with 128-thread
+// CTAs of one tile each, which loaded K, waited, and met at five barriers; 2.2 ms (0.87) so.
+// 31 pairs of 256^2: 135 -> 106 us. With x' = r - V d the new vector is v = x' / ||x'|| and its Gram
 // column follows from these without another pass over the basis (k_of_pass_finish):
 //   G_A[i][v] = (V^T y)_i / ||x'||,   G_L[i][v] = ((V^T q)_i - (G_L d)_i) / ||x'||,
 //   g[v] = x'^T Ups^T b / ||x'||,     G_A[v][v] = x'^T y / ||x'||^2,
 //   G_L[v][v] = (x'^T q - d^T V^T q + d^T G_L d) / ||x'||^2,   Mg[i][v] = (V^T x')_i / ||x'||.
-constexpr int OP_T = 128;  // threads per CTA
 template <typename real>
-constexpr int opx() { return 1024 / (int)sizeof(real); }  // pixels per CTA: 256 (FP32), 128 (FP64): 1 KB copies
+constexpr int opx() { return 512 / (int)sizeof(real); }  // pixels per tile: 128 (FP32), 64 (FP64)
 
-long long of_pass_chunks(long long ns, int elem_bytes) { return (ns * elem_bytes + 1023) / 1024; }
+// Warps per frame pair: each takes up to OP_TILES tiles, fewer where the pairs together would not
+// give the GPU's 152 x 32 warp slots one each (64^2 x 7 pairs: one tile per warp, 448 warps; 1024^2 x
+// 63: eight, which spreads the start of a warp and shortens the reduction behind). A function of the
+// problem alone: the sums do not depend on how the pairs are grouped.
+constexpr int OP_TILES = 8;
+static int of_pass_parts_of(long long ns, int pairs, int elem_bytes) {
+    const long long nt = (ns * elem_bytes + 511) / 512;
+    const long long T = std::max(1LL, std::min<long long>(OP_TILES, nt * pairs / (152 * 32)));
+    return (int)((nt + T - 1) / T);
+}
+long long of_pass_parts(long long ns, int pairs) { return std::max(of_pass_parts_of(ns, pairs, 4), of_pass_parts_of(ns, pairs, 8)); }
 int of_pass_stride(int Kmax) { return 3 * Kmax + 4; }
 
+// 8 bytes of values: two FP32 or one FP64
 template <typename real>
-__global__ void __launch_bounds__(OP_T) k_of_proj_gram_pass(const real *V, long long ns, int Kmax,
-                                                           const int *__restrict__ K, const int *__restrict__ act,
-                                                           const double *__restrict__ d, const real *__restrict__ x,
-                                                           const real *__restrict__ q, real *to, const real *__restrict__ AtB, const real *__restrict__ ux,
-                                                           const real *__restrict__ uy, double *__restrict__ partial,
-                                                           int nchunk, int *__restrict__ err, int kcap) {
-    constexpr int PX = opx<real>(), CH = 2 * PX;  // elements of one vector in the tile
-    constexpr int EPT = CH / OP_T;                // 4 (FP32) or 2 (FP64): 16 bytes per thread
-    using vec_t = typename std::conditional<sizeof(real) == 4, float4, double2>::type;
-    extern __shared__ __align__(128) unsigned char op_smem[];
-    real *sx = reinterpret_cast<real *>(op_smem);  // [CH] r, then x'
-    real *sq = sx + CH, *sa = sq + CH;             // [CH] q, Ups^T b
-    real *sfx = sa + CH, *sfy = sfx + PX;           // [PX] u_x, u_y
-    real *sy = sfy + PX;                            // [CH] y
-    real *sV = sy + CH;                             // [kcap][CH]
-    __shared__ real sd[64];
+using half_t = typename std::conditional<sizeof(real) == 4, F2, double>::type;
+__device__ __forceinline__ double fma2(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ double mul2(double a, double b) { return a * b; }
+__device__ __forceinline__ double sub2(double a, double b) { return a - b; }
+__device__ __forceinline__ float hsum(F2 a) {
+    float x, y;
+    unpack2(a, x, y);
+    return x + y;
+}
+__device__ __forceinline__ double hsum(double a) { return a; }
+
+// The sums over the warp of eight values per lane: value lane >> 2 is returned (equal in the four
+// lanes of a group).
+template <typename real>
+__device__ __forceinline__ real warp_sums8(real (&t)[8], int lane) {
+#pragma unroll
+    for (int h = 4; h > 0; h >>= 1) {
+        const bool up = lane & (h << 2);
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const real send = up ? t[i] : t[i + h];
+            t[i] = (up ? t[i + h] : t[i]) + __shfl_xor_sync(0xffffffffu, send, h << 2);
+        }
+    }
+    real v = t[0];
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v;
+}
+
+template <typename real>
+__global__ void __launch_bounds__(32) k_of_proj_gram_pass(const real *V, long long ns, int Kmax, const int *__restrict__ K,
+                                                         const int *__restrict__ act, const double *__restrict__ d,
+                                                         const real *__restrict__ x, const real *__restrict__ q, real *to,
+                                                         const real *__restrict__ AtB, const real *__restrict__ ux,
+                                                         const real *__restrict__ uy, double *__restrict__ partial, int nparts,
+                                                         int *__restrict__ err, int kcap) {
+    constexpr int PX = opx<real>(), EPL = 16 / (int)sizeof(real);
+    using half = half_t<real>;
+    struct __align__(16) Q {  // a lane's 16 bytes of a segment
+        half h[2];
+    };
+    extern __shared__ __align__(128) unsigned char op_smem[];  // segments of 512 bytes: r, q, Ups^T b (2 each), u_x, u_y, V_j (2 each)
+    __shared__ half sd[64];
     __shared__ __align__(8) unsigned long long bar;
-    __shared__ double s_red[OP_T / 32][4];
-    const int b = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x;
+    const int b = blockIdx.y, part = blockIdx.x, lane = threadIdx.x;
     if (act && !act[b]) return;
-    int Kb = min(K[b], Kmax);
+    const int K0 = K[b];
+    int Kb = min(K0, Kmax);
     if (Kb > kcap) {
-        if (tid == 0 && err) atomicOr(err, 8);
+        if (lane == 0 && err) atomicOr(err, 8);
         Kb = kcap;
     }
-    const long long p0 = (long long)chunk * PX;
-    const int len = (int)min((long long)PX, ns - p0);  // pixels of this chunk (a multiple of 16 bytes)
     const unsigned bar_a = smem_u32(&bar);
-    if (tid == 0) {
+    if (lane == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar_a) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        const unsigned bytes = (unsigned)len * (unsigned)sizeof(real);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_a),
-                     "r"(bytes * (unsigned)(2 * Kb + 8))
-                     : "memory");
-        const long long N2 = 2 * ns;
-        const real *xb = x + b * N2, *qb = q + b * N2, *ab = AtB + b * N2;
-        bulk_g2s(sx, xb + p0, bytes, bar_a);
-        bulk_g2s(sx + PX, xb + ns + p0, bytes, bar_a);
-        bulk_g2s(sq, qb + p0, bytes, bar_a);
-        bulk_g2s(sq + PX, qb + ns + p0, bytes, bar_a);
-        bulk_g2s(sa, ab + p0, bytes, bar_a);
-        bulk_g2s(sa + PX, ab + ns + p0, bytes, bar_a);
-        bulk_g2s(sfx, ux + b * ns + p0, bytes, bar_a);
-        bulk_g2s(sfy, uy + b * ns + p0, bytes, bar_a);
-        const real *Vb = V + (long long)b * Kmax * N2;
-        for (int j = 0; j < Kb; ++j) {
-            bulk_g2s(sV + (long long)j * CH, Vb + (long long)j * N2 + p0, bytes, bar_a);
-            bulk_g2s(sV + (long long)j * CH + PX, Vb + (long long)j * N2 + ns + p0, bytes, bar_a);
-        }
     }
-    for (int j = tid; j < Kb; j += OP_T) sd[j] = (real)d[(long long)b * Kmax + j];
-    __syncthreads();
-    if (!mbar_wait(bar_a, 0, g_wait_polls)) {
-        if (tid == 0 && err) atomicOr(err, 4);
-        mbar_wait(bar_a, 0);
-        return;
-    }
-    // x' = r - V d on this thread's EPT consecutive elements (comp = i0 / PX)
-    const int i0 = tid * EPT, pix0 = i0 % PX;
-    {
-        real acc[EPT];
-#pragma unroll
-        for (int e = 0; e < EPT; ++e) acc[e] = 0;
-        for (int j = 0; j < Kb; ++j) {
-            const vec_t v = *reinterpret_cast<const vec_t *>(sV + (long long)j * CH + i0);
-            const real *vv = reinterpret_cast<const real *>(&v);
-            const real dj = sd[j];
-#pragma unroll
-            for (int e = 0; e < EPT; ++e) acc[e] += vv[e] * dj;
+    const long long N2 = 2 * ns;
+    const int ntile = (int)((ns + PX - 1) / PX);
+    const real *Vb = V + (long long)b * Kmax * N2;
+    auto fetch = [&](int tile) {
+        const long long p0 = (long long)tile * PX;
+        const unsigned bytes = (unsigned)min((long long)PX, ns - p0) * (unsigned)sizeof(real);  // (a multiple of 16)
+        if (lane == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_a), "r"(bytes * (unsigned)(2 * Kb + 8))
+                         : "memory");
+        __syncwarp();
+        for (int i = lane; i < 2 * Kb + 8; i += 32) {
+            const long long c = (i & 1) ? ns : 0;
+            const real *src;
+            if (i >= 8) src = Vb + (long long)((i - 8) >> 1) * N2 + c;
+            else if (i >= 6) src = (i == 6 ? ux : uy) + b * ns;
+            else src = (i < 2 ? x : (i < 4 ? q : AtB)) + b * N2 + c;
+            bulk_g2s(op_smem + i * 512, src + p0, bytes, bar_a);
         }
-        vec_t xv = *reinterpret_cast<const vec_t *>(sx + i0);
-        real *xx = reinterpret_cast<real *>(&xv);
+    };
+    fetch(part);
+    for (int j = lane; j < Kb; j += 32) {
+        if constexpr (sizeof(real) == 4) sd[j] = both((float)d[(long long)b * Kmax + j]);
+        else sd[j] = d[(long long)b * Kmax + j];
+    }
+    __syncwarp();
+    const Q *seg = reinterpret_cast<const Q *>(op_smem) + lane;  // segment i: seg[i * 32]
+    double acc[3][2] = {}, acs = 0.0;
+    unsigned phase = 0;
+    for (int tile = part; tile < ntile; tile += nparts) {
+        const long long p = (long long)tile * PX + lane * EPL;
+        const bool in = p < ns;  // all of a lane's pixels or none
+        if (!in) {
+            Q zero;
+            if constexpr (sizeof(real) == 4) zero.h[0] = zero.h[1] = both(0.f);
+            else zero.h[0] = zero.h[1] = 0.0;
+            for (int i = 0; i < 2 * Kb + 8; ++i) const_cast<Q *>(seg)[i * 32] = zero;
+        }
+        if (!mbar_wait(bar_a, phase, g_wait_polls)) {
+            if (lane == 0 && err) atomicOr(err, 4);
+            mbar_wait(bar_a, phase);  // do not leave while copies may still land
+            return;
+        }
+        phase ^= 1;
+        const Q *sv = seg + 8 * 32;
+        Q xa = seg[0], xb = seg[32];
+        {  // x' = r - V d
+            half s[4];
+            if constexpr (sizeof(real) == 4) s[0] = s[1] = s[2] = s[3] = both(0.f);
+            else s[0] = s[1] = s[2] = s[3] = 0.0;
+#pragma unroll 4
+            for (int j = 0; j < Kb; ++j) {
+                const Q va = sv[j * 64], vb = sv[j * 64 + 32];
+                const half dj = sd[j];
+                s[0] = fma2(va.h[0], dj, s[0]);
+                s[1] = fma2(va.h[1], dj, s[1]);
+                s[2] = fma2(vb.h[0], dj, s[2]);
+                s[3] = fma2(vb.h[1], dj, s[3]);
+            }
 #pragma unroll
-        for (int e = 0; e < EPT; ++e) xx[e] = (pix0 + e < len) ? xx[e] - acc[e] : (real)0;
-        *reinterpret_cast<vec_t *>(sx + i0) = xv;
-        // into the slot behind the basis, where an append finds it (a full basis appends nothing)
-        if (K[b] < Kmax) {
-            real *ob = to + ((long long)b * Kmax + Kb) * 2 * ns + (i0 < PX ? 0 : ns) + p0 + pix0;
-            if (pix0 + EPT <= len) {
-                *reinterpret_cast<vec_t *>(ob) = xv;
-            } else {
-#pragma unroll
-                for (int e = 0; e < EPT; ++e)
-                    if (pix0 + e < len) ob[e] = xx[e];
+            for (int e = 0; e < 2; ++e) {
+                xa.h[e] = sub2(xa.h[e], s[e]);
+                xb.h[e] = sub2(xb.h[e], s[2 + e]);
             }
         }
-    }
-    __syncthreads();
-    // y = Ups^T Ups x' and the four scalars
-    double s4[4] = {0.0, 0.0, 0.0, 0.0};
-    {
-        real a4[4] = {0, 0, 0, 0};
+        if (in && K0 < Kmax) {  // into the slot behind the basis, where an append finds it (a full basis appends nothing)
+            real *ob = to + ((long long)b * Kmax + Kb) * N2 + p;
+            *reinterpret_cast<Q *>(ob) = xa;
+            *reinterpret_cast<Q *>(ob + ns) = xb;
+        }
+        // y = Ups^T Ups x' and the four scalars
+        Q ya, yb;
+        const Q qa = seg[64], qb = seg[96];
+        {
+            const Q fx = seg[6 * 32], fy = seg[7 * 32], aa = seg[4 * 32], ab = seg[5 * 32];
+            half s[4];
 #pragma unroll
-        for (int e = 0; e < EPT; ++e) {
-            const int i = i0 + e, p = i % PX;
-            real yv = 0;
-            if (p < len) {
-                const real w = sfx[p] * sx[p] + sfy[p] * sx[PX + p];
-                yv = (i < PX ? sfx[p] : sfy[p]) * w;
+            for (int e = 0; e < 2; ++e) {
+                const half w = fma2(fx.h[e], xa.h[e], mul2(fy.h[e], xb.h[e]));
+                ya.h[e] = mul2(fx.h[e], w);
+                yb.h[e] = mul2(fy.h[e], w);
+                s[0] = e ? fma2(xa.h[e], xa.h[e], s[0]) : mul2(xa.h[e], xa.h[e]);
+                s[1] = e ? fma2(xa.h[e], ya.h[e], s[1]) : mul2(xa.h[e], ya.h[e]);
+                s[2] = e ? fma2(xa.h[e], qa.h[e], s[2]) : mul2(xa.h[e], qa.h[e]);
+                s[3] = e ? fma2(xa.h[e], aa.h[e], s[3]) : mul2(xa.h[e], aa.h[e]);
+                s[0] = fma2(xb.h[e], xb.h[e], s[0]);
+                s[1] = fma2(xb.h[e], yb.h[e], s[1]);
+                s[2] = fma2(xb.h[e], qb.h[e], s[2]);
+                s[3] = fma2(xb.h[e], ab.h[e], s[3]);
             }
-            sy[i] = yv;
-            if (p < len) {  // the tile beyond len holds no copied data
-                const real xi = sx[i];
-                a4[0] += xi * xi;
-                a4[1] += xi * yv;
-                a4[2] += xi * sq[i];
-                a4[3] += xi * sa[i];
+            real t[8] = {hsum(s[0]), hsum(s[1]), hsum(s[2]), hsum(s[3]), 0, 0, 0, 0};
+            acs += (double)warp_sums8(t, lane);
+        }
+        // dots of the basis vectors with x', y and q: eight vectors at a time, four such blocks to a
+        // value per lane (lane l: vector 8 (l & 3) + (l >> 2) of the 32)
+#pragma unroll
+        for (int jb = 0; jb < 2; ++jb) {
+            if (jb * 32 >= Kb) break;
+            real v1 = 0, v2 = 0, v3 = 0;
+#pragma unroll 1
+            for (int g = 0; g < 4; ++g) {
+                const int j0 = jb * 32 + g * 8;
+                if (j0 >= Kb) break;
+                real t1[8], t2[8], t3[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    t1[i] = t2[i] = t3[i] = 0;
+                    if (j0 + i < Kb) {
+                        const Q va = sv[(j0 + i) * 64], vb = sv[(j0 + i) * 64 + 32];
+                        t1[i] = hsum(fma2(vb.h[1], xb.h[1], fma2(vb.h[0], xb.h[0], fma2(va.h[1], xa.h[1], mul2(va.h[0], xa.h[0])))));
+                        t2[i] = hsum(fma2(vb.h[1], yb.h[1], fma2(vb.h[0], yb.h[0], fma2(va.h[1], ya.h[1], mul2(va.h[0], ya.h[0])))));
+                        t3[i] = hsum(fma2(vb.h[1], qb.h[1], fma2(vb.h[0], qb.h[0], fma2(va.h[1], qa.h[1], mul2(va.h[0], qa.h[0])))));
+                    }
+                }
+                const real u1 = warp_sums8(t1, lane), u2 = warp_sums8(t2, lane), u3 = warp_sums8(t3, lane);
+                const bool mine = (lane & 3) == g;
+                v1 = mine ? u1 : v1;
+                v2 = mine ? u2 : v2;
+                v3 = mine ? u3 : v3;
             }
+            acc[0][jb] += (double)v1;
+            acc[1][jb] += (double)v2;
+            acc[2][jb] += (double)v3;
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if constexpr (sizeof(real) == 4) s4[k] = (double)warp_sumf(a4[k]);
-            else s4[k] = warp_sum(a4[k]);
-        }
-    }
-    const int w = tid >> 5, l = tid & 31;
-    if (l == 0)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) s_red[w][k] = s4[k];
-    __syncthreads();
-    // partials stored output-major, [b][output][chunk], so that the reduction reads each
-    // output's chunks contiguously
-    double *out = partial + (long long)b * (3 * Kmax + 4) * nchunk + chunk;
-    if (tid < 4) {
-        double t = 0.0;
-        for (int ww = 0; ww < OP_T / 32; ++ww) t += s_red[ww][tid];
-        out[(long long)(3 * Kmax + tid) * nchunk] = t;
-    }
-    // dots of every basis vector with x', y and q: warp w takes j = w, w + 2, ...; lane l holds
-    // the elements l + 32 e of x', y, q in registers (consecutive lanes read consecutive words:
-    // no bank conflicts); elements beyond the chunk's pixels count as zero
-    constexpr int LE = CH / 32;
-    real rx[LE], ry[LE], rq[LE];
-#pragma unroll
-    for (int e = 0; e < LE; ++e) {
-        const int i = l + 32 * e;
-        const bool in = (i % PX) < len;
-        rx[e] = in ? sx[i] : (real)0;
-        ry[e] = in ? sy[i] : (real)0;
-        rq[e] = in ? sq[i] : (real)0;
-    }
-    for (int j = w; j < Kb; j += OP_T / 32) {
-        const real *vj = sV + (long long)j * CH + l;
-        real t1 = 0, t2 = 0, t3 = 0;
-#pragma unroll
-        for (int e = 0; e < LE; ++e) {
-            if (((l + 32 * e) % PX) < len) {
-                const real v = vj[32 * e];
-                t1 += v * rx[e];
-                t2 += v * ry[e];
-                t3 += v * rq[e];
-            }
-        }
-        // the warp's partial sums in the storage precision (FP64 work is slow on this GPU), then
-        // FP64 across the chunks
-        double o1, o2, o3;
-        if constexpr (sizeof(real) == 4) {
-            o1 = (double)warp_sumf(t1);
-            o2 = (double)warp_sumf(t2);
-            o3 = (double)warp_sumf(t3);
-        } else {
-            o1 = warp_sum(t1);
-            o2 = warp_sum(t2);
-            o3 = warp_sum(t3);
-        }
-        if (l == 0) {
-            out[(long long)j * nchunk] = o1;
-            out[(long long)(Kmax + j) * nchunk] = o2;
-            out[(long long)(2 * Kmax + j) * nchunk] = o3;
+        if (tile + nparts < ntile) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();  // every lane has read the tile
+            fetch(tile + nparts);
         }
     }
+    // stored output-major, [b][output][warp], so that the reduction reads each output contiguously
+    double *out = partial + (long long)b * (3 * Kmax + 4) * nparts + part;
+#pragma unroll
+    for (int jb = 0; jb < 2; ++jb) {
+        const int j = jb * 32 + 8 * (lane & 3) + (lane >> 2);
+        if (j < Kb)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) out[(long long)(c * Kmax + j) * nparts] = acc[c][jb];
+    }
+    if (lane < 16 && !(lane & 3)) out[(long long)(3 * Kmax + (lane >> 2)) * nparts] = acs;
 }
 
 // ||x[b]||^2 per chunk
@@ -1131,7 +1172,7 @@ bool of_pass_applicable(long long ns, const void *V, const void *x) {
 }
 
 template <typename real>
-mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long long ns, const double *d, const real *x, const real *q,
+mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long long ns, int pairs, const double *d, const real *x, const real *q,
                                     const real *AtB, const real *ux, const real *uy, double *partial, double *res, int *err,
                                     int kcap, const double *scale, double tol, int *grow, double *GA, double *GL, double *g,
                                     double *Mg, double *nrm2_out, int *appended, double *aux, int *done, cudaStream_t st) {
@@ -1142,10 +1183,10 @@ mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long lon
             return fail(MOF_ECUDA, "shared-memory attribute of the Solve-OF pass");
         configured.store(true);
     }
-    const int nc = (int)of_pass_chunks(ns, (int)sizeof(real));
+    const int nc = of_pass_parts_of(ns, pairs, (int)sizeof(real));
     const int kc = kcap > 0 ? std::min(kcap, B.Kmax) : B.Kmax;
-    const size_t smem = (size_t)(kc + 5) * 2048;
-    ::mof::count_launch(), k_of_proj_gram_pass<real><<<dim3(nc, B.B), OP_T, smem, st>>>(B.V, ns, B.Kmax, B.K, B.act, d, x, q, B.V, AtB,
+    const size_t smem = (size_t)(kc + 4) * 1024;
+    ::mof::count_launch(), k_of_proj_gram_pass<real><<<dim3(nc, B.B), 32, smem, st>>>(B.V, ns, B.Kmax, B.K, B.act, d, x, q, B.V, AtB,
                                                                                      ux, uy, partial, nc, err, kc);
     const int stride = of_pass_stride(B.Kmax);
     int *slot = reinterpret_cast<int *>(aux);
@@ -1159,7 +1200,7 @@ mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long lon
 template bool of_pass_applicable<float>(long long, const void *, const void *);
 template bool of_pass_applicable<double>(long long, const void *, const void *);
 #define MOF_INST_OF(real)                                                                                                      \
-    template mof_status launch_of_proj_gram_pass<real>(const BasisRef<real> &, int *, long long, const double *, const real *, \
+    template mof_status launch_of_proj_gram_pass<real>(const BasisRef<real> &, int *, long long, int, const double *, const real *, \
                                                        const real *, const real *, const real *, const real *, double *,      \
                                                        double *, int *, int, const double *, double, int *, double *,         \
                                                        double *, double *, double *, double *, int *, double *, int *,        \

@@ -304,7 +304,7 @@ static long long of_partial_per_pair(const mof_problem *p, int Kof, int of_ell) 
     const long long gram_chunks = (ns + 511) / 512;  // chunks of the FP64 Gram kernel (the smaller)
     const long long gram = (long long)std::min(of_ell, Kof) * gram_chunks * (2LL * Kof + 1);
     const long long wgram = (long long)WG_CTAS * wg_pstride(Kof);
-    const long long pass = of_pass_chunks(ns, 8) * of_pass_stride(Kof);  // k_of_proj_gram_pass (FP64 chunks)
+    const long long pass = of_pass_parts(ns, p->nt - 1) * of_pass_stride(Kof);  // k_of_proj_gram_pass
     return std::max(std::max(std::max(krylov_partial_doubles(2 * ns, Kof), gram), wgram), pass);
 }
 
@@ -1605,7 +1605,7 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
                     // p = q = 2: the projection, the new vector's Gram columns and the append in
                     // one pass over the basis (no separate Gram-column pass after it)
                     Scope sc(tm, "of_subdot", gst);
-                    MOF_TRY(launch_of_proj_gram_pass<real>(BAg, Kvg, ns, cg, wvg, w.q_of + (long long)b0 * N2, AtBg, uxg, uyg,
+                    MOF_TRY(launch_of_proj_gram_pass<real>(BAg, Kvg, ns, P, cg, wvg, w.q_of + (long long)b0 * N2, AtBg, uxg, uyg,
                                                            kg.partial, w.pres_of + (long long)b0 * of_pass_stride(Kof), w.err, kcap,
                                                            w.scale_of + b0, tol, w.grow_of + b0, w.GA + b0 * KK, w.GL + b0 * KK,
                                                            w.gof + (long long)b0 * Kof, Mgg, w.nrm_of + b0, appg, kg.aux,

@@ -112,14 +112,14 @@ struct Krylov {
 // launch_of_combine: s = V z, scaling a vector appended since the last call to x' / ||x'||.
 // partial: [B][chunks][3 Kmax + 4] doubles; res: [B][3 Kmax + 4]; aux: 2 B doubles (the slot and
 // scale between an append and the next combine); done: [B] ints, zero between calls.
-long long of_pass_chunks(long long ns, int elem_bytes);
+long long of_pass_parts(long long ns, int pairs);
 int of_pass_stride(int Kmax);
 template <typename real> bool of_pass_applicable(long long ns, const void *V, const void *x);
 template <typename real>
 mof_status launch_of_resid_lap(int nb, int nx, int ny, const real *ux, const real *uy, const real *AtB, const real *s,
                                const double *gam, real *r, real *q, const int *act, cudaStream_t st);
 template <typename real>
-mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long long ns, const double *d, const real *x, const real *q,
+mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long long ns, int pairs, const double *d, const real *x, const real *q,
                                     const real *AtB, const real *ux, const real *uy, double *partial, double *res, int *err,
                                     int kcap, const double *scale, double tol, int *grow, double *GA, double *GL, double *g,
                                     double *Mg, double *nrm2_out, int *appended, double *aux, int *done, cudaStream_t st);

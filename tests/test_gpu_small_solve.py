@@ -39,3 +39,22 @@ def test_bordered_solves(prec, ell, iters):
     got = s.cpu().double().numpy().reshape(want.shape)
     err = np.linalg.norm(got - want) / np.linalg.norm(want)
     assert err <= (1e-6 if f64 else 1e-3), err
+
+
+# frames whose last tile of the projection pass is ragged, and enough of them that a warp takes
+# several tiles (2 in FP32, 4 in FP64)
+@pytest.mark.parametrize("prec", [api.MOF_FP64, api.MOF_FP32])
+def test_projection_pass_tiles(prec):
+    n, nt = 362, 11
+    g = np.random.default_rng(5)
+    f64 = prec == api.MOF_FP64
+    y, x = np.mgrid[0:n, 0:n] / n
+    u = np.stack([np.sin(7 * x + 0.05 * t) * np.cos(5 * y - 0.04 * t) for t in range(nt)]) + 0.01 * g.standard_normal((nt, n, n))
+    u = u.astype(np.float64 if f64 else np.float32)
+    p = api.mof_problem_create(n, n, nt, 8, [1] * nt, np.zeros(nt), 1.0, 1.0, prec)
+    s = torch.empty(p.nv, dtype=torch.float64 if f64 else torch.float32, device="cuda")
+    api.mof_solve_of(p, api.mof_default_params(of_ell=3, of_iters=6), torch.tensor(u, device="cuda").reshape(-1), s)
+    want = OS.solve_of(u.astype(np.float64), OS.Params(of_ell=3, of_iters=6))
+    got = s.cpu().double().numpy().reshape(want.shape)
+    err = np.linalg.norm(got - want) / np.linalg.norm(want)
+    assert err <= (1e-6 if f64 else 1e-3), err
