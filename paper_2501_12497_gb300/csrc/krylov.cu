@@ -1100,8 +1100,9 @@ mof_status launch_of_combine(const BasisRef<real> &B, const double *z, double *a
 }
 
 // r = Ups^T Ups s - Ups^T b + gamma (L(+)L)^T (L(+)L) s (the normal-equation residual of Alg. 2)
-// and q = L^T L r on both components (graph Laplacians with free boundary) in one pass: a CTA
-// forms r on its 32 x 8 tile and a border of one pixel from s with a border of two.
+// and q = L^T L r on both components (graph Laplacians with free boundary) in one pass, on 32 x 8
+// tiles with the borders of s and r in shared memory, one thread per pixel. FP64: bound by the FP64
+// pipe (1024^2 x 7 pairs 640 us; the marching form below 633, 256^2 x 31 184 against 254 us).
 template <typename real>
 __device__ __forceinline__ real lap5(real c, bool l, real fl, bool r, real fr, bool u, real fu, bool d, real fd) {
     real v = 0;
@@ -1112,10 +1113,10 @@ __device__ __forceinline__ real lap5(real c, bool l, real fl, bool r, real fr, b
     return v;
 }
 template <typename real>
-__global__ void __launch_bounds__(256) k_of_resid_lap(const real *__restrict__ ux, const real *__restrict__ uy,
-                                                      const real *__restrict__ AtB, const real *__restrict__ s,
-                                                      const double *__restrict__ gam, real *__restrict__ r, real *__restrict__ q,
-                                                      int nx, int ny, const int *__restrict__ act) {
+__global__ void __launch_bounds__(256) k_of_resid_lap_tile(const real *__restrict__ ux, const real *__restrict__ uy,
+                                                           const real *__restrict__ AtB, const real *__restrict__ s,
+                                                           const double *__restrict__ gam, real *__restrict__ r, real *__restrict__ q,
+                                                           int nx, int ny, const int *__restrict__ act) {
     constexpr int W = 32, H = 8;
     __shared__ real S[2][H + 4][W + 4], R[2][H + 2][W + 2];
     __shared__ real s_g;
@@ -1156,11 +1157,118 @@ __global__ void __launch_bounds__(256) k_of_resid_lap(const real *__restrict__ u
     }
 }
 
+// The same for FP32 rows of a multiple of 4 pixels. A lane takes V = 4 columns and marches down
+// `rows` rows with three rows of s and of r in registers; the neighbours come from the adjacent lanes,
+// so the first and last lane of a warp only serve the others (except at the image's edge). The next
+// row is loaded before the present one is used. Bound by HBM: six values read and four written per
+// pixel. 63 pairs of 1024^2: 0.45 ms (0.86 of the copy rate) against 1.15 for the tiles; 31 pairs of
+// 256^2: 22 against 37 us.
+constexpr int RL_W = 4;  // warps per CTA
 template <typename real>
-mof_status launch_of_resid_lap(int nb, int nx, int ny, const real *ux, const real *uy, const real *AtB, const real *s,
+__global__ void __launch_bounds__(32 * RL_W) k_of_resid_lap(const real *__restrict__ ux, const real *__restrict__ uy,
+                                                            const real *__restrict__ AtB, const real *__restrict__ s,
+                                                            const double *__restrict__ gam, real *__restrict__ r,
+                                                            real *__restrict__ q, int nx, int ny, int rows,
+                                                            const int *__restrict__ act) {
+    constexpr int V = 16 / (int)sizeof(real), HL = 1, OUT = 32 - 2 * HL;  // HL: serving lanes on each side
+    const int b = blockIdx.z, lane = threadIdx.x, y0 = (blockIdx.y * RL_W + threadIdx.y) * rows;
+    if (y0 >= ny || !act[b]) return;  // whole warps
+    const int C = nx / V, c = blockIdx.x * OUT + lane;
+    const bool out = c < C && (lane >= HL || blockIdx.x == 0) && (lane < 32 - HL || blockIdx.x == gridDim.x - 1);
+    const int x = min(c, C - 1) * V, ye = min(y0 + rows, ny);
+    const long long ns = (long long)nx * ny;
+    ux += b * ns + x;
+    uy += b * ns + x;
+    AtB += b * 2 * ns + x;
+    s += b * 2 * ns + x;
+    r += b * 2 * ns + x;
+    q += b * 2 * ns + x;
+    const real g = (real)gam[b];
+    struct __align__(V * sizeof(real)) Vec {
+        real v[V];
+    };
+    auto row = [&](const real *f, int y) { return *reinterpret_cast<const Vec *>(f + (long long)min(max(y, 0), ny - 1) * nx); };
+    Vec sm[2], sc[2], sp[2], rm[2], rc[2], f[4];
+    auto fetch = [&](int y, Vec (&sn)[2], Vec (&fn)[4]) {  // s of row y + 1, the fields of row y
+        sn[0] = row(s, y + 1);
+        sn[1] = row(s + ns, y + 1);
+        fn[0] = row(ux, y);
+        fn[1] = row(uy, y);
+        fn[2] = row(AtB, y);
+        fn[3] = row(AtB + ns, y);
+    };
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        sm[k] = row(s + k * ns, y0 - 2);
+        sc[k] = row(s + k * ns, y0 - 1);
+#pragma unroll
+        for (int e = 0; e < V; ++e) rm[k].v[e] = rc[k].v[e] = 0;
+    }
+    fetch(y0 - 1, sp, f);
+    // a row's five-point sums; m, n: the rows above and below
+    auto lap = [&](const Vec &m, const Vec &w, const Vec &n, int y, Vec &o) {
+        const real lf = __shfl_up_sync(0xffffffffu, w.v[V - 1], 1), rt = __shfl_down_sync(0xffffffffu, w.v[0], 1);
+#pragma unroll
+        for (int e = 0; e < V; ++e)
+            o.v[e] = lap5(w.v[e], x + e > 0, e ? w.v[e ? e - 1 : 0] : lf, x + e < nx - 1, e < V - 1 ? w.v[e < V - 1 ? e + 1 : e] : rt, y > 0,
+                          m.v[e], y < ny - 1, n.v[e]);
+    };
+    for (int y = y0 - 1; y <= ye; ++y) {
+        Vec sn[2], fn[4], rp[2];
+        if (y < ye) fetch(y + 1, sn, fn);
+        Vec l0, l1;
+        lap(sm[0], sc[0], sp[0], y, l0);
+        lap(sm[1], sc[1], sp[1], y, l1);
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            const real ax = f[0].v[e], ay = f[1].v[e], a = ax * sc[0].v[e] + ay * sc[1].v[e];
+            rp[0].v[e] = ax * a - f[2].v[e] + g * l0.v[e];
+            rp[1].v[e] = ay * a - f[3].v[e] + g * l1.v[e];
+        }
+        if (out && y >= y0 && y < ye) {
+            *reinterpret_cast<Vec *>(r + (long long)y * nx) = rp[0];
+            *reinterpret_cast<Vec *>(r + ns + (long long)y * nx) = rp[1];
+        }
+        if (y > y0) {
+            lap(rm[0], rc[0], rp[0], y - 1, l0);
+            lap(rm[1], rc[1], rp[1], y - 1, l1);
+            if (out) {
+                *reinterpret_cast<Vec *>(q + (long long)(y - 1) * nx) = l0;
+                *reinterpret_cast<Vec *>(q + ns + (long long)(y - 1) * nx) = l1;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            rm[k] = rc[k];
+            rc[k] = rp[k];
+            sm[k] = sc[k];
+            sc[k] = sp[k];
+            sp[k] = sn[k];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) f[k] = fn[k];
+    }
+}
+
+template <typename real>
+mof_status launch_of_resid_lap(int nb, int pairs, int nx, int ny, const real *ux, const real *uy, const real *AtB, const real *s,
                                const double *gam, real *r, real *q, const int *act, cudaStream_t st) {
-    ::mof::count_launch(), k_of_resid_lap<real><<<dim3((nx + 31) / 32, (ny + 7) / 8, nb), dim3(32, 8), 0, st>>>(ux, uy, AtB, s, gam, r, q,
-                                                                                                            nx, ny, act);
+    auto al = [](const void *p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
+    const int gx = std::max(1, (nx / 4 - 2 + 29) / 30);
+    ::mof::count_launch();
+    // marching where strips of 4 rows give every SM four warps (256^2 x 7 pairs, 1344 strips: 10 against
+    // 13 us; 128^2 x 7, 224 strips: 8.8 both)
+    if (sizeof(real) == 4 && nx % 4 == 0 && al(ux) && al(uy) && al(AtB) && al(s) && al(r) && al(q) &&
+        (long long)gx * pairs * ((ny + 3) / 4) >= 152LL * 4) {
+        // strips of 16 rows (four rows of s and two of the rest are read twice) where they give every SM
+        // 16 warps, else of 8 or 4
+        int rows = 16;
+        while (rows > 4 && (long long)gx * pairs * ((ny + rows - 1) / rows) < 152LL * 16) rows /= 2;
+        k_of_resid_lap<float><<<dim3(gx, (ny + RL_W * rows - 1) / (RL_W * rows), nb), dim3(32, RL_W), 0, st>>>(
+            (const float *)ux, (const float *)uy, (const float *)AtB, (const float *)s, gam, (float *)r, (float *)q, nx, ny, rows, act);
+    } else {
+        k_of_resid_lap_tile<real><<<dim3((nx + 31) / 32, (ny + 7) / 8, nb), dim3(32, 8), 0, st>>>(ux, uy, AtB, s, gam, r, q, nx, ny, act);
+    }
     MOF_LAUNCH_CHECK();
     return MOF_OK;
 }
@@ -1206,7 +1314,7 @@ template bool of_pass_applicable<double>(long long, const void *, const void *);
                                                        double *, double *, double *, double *, int *, double *, int *,        \
                                                        cudaStream_t);                                                          \
     template mof_status launch_of_combine<real>(const BasisRef<real> &, const double *, double *, real *, cudaStream_t);       \
-    template mof_status launch_of_resid_lap<real>(int, int, int, const real *, const real *, const real *, const real *,       \
+    template mof_status launch_of_resid_lap<real>(int, int, int, int, const real *, const real *, const real *, const real *,       \
                                                   const double *, real *, real *, const int *, cudaStream_t);
 MOF_INST_OF(float)
 MOF_INST_OF(double)

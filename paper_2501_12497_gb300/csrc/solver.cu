@@ -1587,7 +1587,7 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
                 ::mof::count_launch(), k_sqrt_into<<<pb, 64, 0, gst>>>(w.rn_of + b0, w.scale_of + b0, nb);
             } else if (pass_ok) {
                 Scope sc(tm, "of_resid", gst);
-                MOF_TRY(launch_of_resid_lap<real>(nb, p->nx, p->ny, uxg, uyg, AtBg, sg, sa.lam, wvg, w.q_of + (long long)b0 * N2, actg,
+                MOF_TRY(launch_of_resid_lap<real>(nb, P, p->nx, p->ny, uxg, uyg, AtBg, sg, sa.lam, wvg, w.q_of + (long long)b0 * N2, actg,
                                                   gst));
             } else {
                 Scope sc(tm, "of_resid", gst);

@@ -116,7 +116,7 @@ long long of_pass_parts(long long ns, int pairs);
 int of_pass_stride(int Kmax);
 template <typename real> bool of_pass_applicable(long long ns, const void *V, const void *x);
 template <typename real>
-mof_status launch_of_resid_lap(int nb, int nx, int ny, const real *ux, const real *uy, const real *AtB, const real *s,
+mof_status launch_of_resid_lap(int nb, int pairs, int nx, int ny, const real *ux, const real *uy, const real *AtB, const real *s,
                                const double *gam, real *r, real *q, const int *act, cudaStream_t st);
 template <typename real>
 mof_status launch_of_proj_gram_pass(const BasisRef<real> &B, int *Kmut, long long ns, int pairs, const double *d, const real *x, const real *q,

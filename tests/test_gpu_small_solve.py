@@ -58,3 +58,23 @@ def test_projection_pass_tiles(prec):
     got = s.cpu().double().numpy().reshape(want.shape)
     err = np.linalg.norm(got - want) / np.linalg.norm(want)
     assert err <= (1e-6 if f64 else 1e-3), err
+
+
+# widths whose rows are taken by the marching residual kernel in strips of 4 rows (364 x 61: a last
+# strip of one row, the last warp with one lane of its own) and of 16 (364 x 1000), frames that are no
+# multiple of 4 values (45 x 47: scalar half-steps, no one-pass projection) and of many chunks
+@pytest.mark.parametrize("nx,ny,nt,ell,iters", [(364, 61, 22, 3, 4), (364, 1000, 14, 2, 2), (45, 47, 5, 12, 3), (128, 65, 4, 9, 2)])
+@pytest.mark.parametrize("prec", [api.MOF_FP64, api.MOF_FP32])
+def test_residual_and_golub_kahan_sizes(prec, nx, ny, nt, ell, iters):
+    g = np.random.default_rng(6)
+    f64 = prec == api.MOF_FP64
+    y, x = np.mgrid[0:ny, 0:nx] / max(nx, ny)
+    u = np.stack([np.sin(9 * x + 0.05 * t) * np.cos(6 * y - 0.04 * t) for t in range(nt)]) + 0.01 * g.standard_normal((nt, ny, nx))
+    u = u.astype(np.float64 if f64 else np.float32)
+    p = api.mof_problem_create(nx, ny, nt, 8, [1] * nt, np.zeros(nt), 1.0, 1.0, prec)
+    s = torch.empty(p.nv, dtype=torch.float64 if f64 else torch.float32, device="cuda")
+    api.mof_solve_of(p, api.mof_default_params(of_ell=ell, of_iters=iters), torch.tensor(u, device="cuda").reshape(-1), s)
+    want = OS.solve_of(u.astype(np.float64), OS.Params(of_ell=ell, of_iters=iters))
+    got = s.cpu().double().numpy().reshape(want.shape)
+    err = np.linalg.norm(got - want) / np.linalg.norm(want)
+    assert err <= (1e-6 if f64 else 1e-3), err
