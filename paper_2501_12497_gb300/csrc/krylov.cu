@@ -746,6 +746,272 @@ __global__ void __launch_bounds__(KT) k_append(real *__restrict__ V, long long N
     }
 }
 
+// ------------------------------------------------------------ Golub-Kahan half-steps
+// A half-step forms x = (operator applied to the other side's vector) - c v_prev, takes it out of
+// the basis once more (x' = x - V V^T x; V^T x = 0 by the recurrence) and appends x' / ||x'||.
+// k_gk_dots forms x (by FRONT, below) and V^T x, k_gk_sub forms x' in the slot behind the basis and
+// ||x'||; the last CTA of a problem to finish (counter done[b], left at zero) adds the partials and,
+// in k_gk_sub, takes the append decision (as k_append_prep_sum). The vector's scale 1 / ||x'|| is
+// applied by the next half-step's front, which reads the vector anyway, or by k_gk_scale. Two
+// launches and 11 + 4 K passes over ns values per half-step on the V side of Solve-OF instead of six
+// and 17 + 4 K: bound by HBM on large frames (63 pairs of 1024^2, 10 steps: 31.4 -> 23.3 ms), by the
+// launches and the last CTA on small ones (31 pairs of 256^2: 1.74 -> 0.99 ms; image step of 64^2 x 8
+// in FP64 with its projections: 1.90 -> 1.52 ms).
+//   FRONT 0: x = a - coef prev (prev may be null: x = a, which is then not written)
+//   FRONT 1: x = Ups^T u - coef prev, u of N / 2 values (prev may be null)
+//   FRONT 2: x = Ups v - coef prev, v of 2 N values
+// FRONT 1, 2: u / v is multiplied by inv[b] and written back first when inv is given.
+template <typename real, int FRONT, bool VEC>
+__global__ void __launch_bounds__(KT) k_gk_dots(const real *V, long long N, int Kmax, const int *__restrict__ K,
+                                                const int *__restrict__ act, GkFront<real> f, double *__restrict__ partial,
+                                                int nchunk, double *__restrict__ out, int *done) {
+    // a chunk: FRONT 1: the same DCH / 2 pixels of both components
+    constexpr int DCH = dch<real>(), SEG = FRONT == 1 ? 2 : 1, PER = DCH / SEG, W = VEC ? 4 : 1;
+    __shared__ __align__(16) real sx[DCH];
+    __shared__ int s_last;
+    const int b = blockIdx.y, chunk = blockIdx.x, tid = threadIdx.x, w = tid >> 5, l = tid & 31;
+    if (act && !act[b]) return;
+    const int Kb = min(K[b], Kmax);
+    const long long L = N / SEG, c0 = (long long)chunk * PER;
+    const int len = (int)min((long long)PER, L - c0);
+    struct __align__(W * sizeof(real)) Vec {
+        real v[W];
+    };
+    auto ld = [](const real *q) { return *reinterpret_cast<const Vec *>(q); };
+    auto st = [](real *q, const Vec &v) { *reinterpret_cast<Vec *>(q) = v; };
+    const real cf = f.prev ? (real)f.coef[b] : (real)0, iv = f.inv ? f.inv[b] : (real)1;
+    const real *pb = f.prev ? f.prev + b * f.pstride + c0 : nullptr;
+    real *xb = f.x + b * f.xstride + c0;
+    for (int i = tid * W; i < PER; i += KT * W) {
+        Vec x[SEG];
+#pragma unroll
+        for (int g = 0; g < SEG; ++g)
+#pragma unroll
+            for (int e = 0; e < W; ++e) x[g].v[e] = 0;
+        if (i < len) {
+            if constexpr (FRONT == 0) {
+                x[0] = ld(f.a + b * f.astride + c0 + i);
+            } else {
+                const Vec ax = ld(f.ux + b * f.fstride + c0 + i), ay = ld(f.uy + b * f.fstride + c0 + i);
+                real *ab = f.s + b * f.astride + c0 + i;
+                Vec u = ld(ab);
+                if constexpr (FRONT == 1) {
+                    if (f.inv) {
+#pragma unroll
+                        for (int e = 0; e < W; ++e) u.v[e] *= iv;
+                        st(ab, u);
+                    }
+#pragma unroll
+                    for (int e = 0; e < W; ++e) {
+                        x[0].v[e] = ax.v[e] * u.v[e];
+                        x[SEG - 1].v[e] = ay.v[e] * u.v[e];
+                    }
+                } else {
+                    Vec u1 = ld(ab + N);
+                    if (f.inv) {
+#pragma unroll
+                        for (int e = 0; e < W; ++e) {
+                            u.v[e] *= iv;
+                            u1.v[e] *= iv;
+                        }
+                        st(ab, u);
+                        st(ab + N, u1);
+                    }
+#pragma unroll
+                    for (int e = 0; e < W; ++e) x[0].v[e] = ax.v[e] * u.v[e] + ay.v[e] * u1.v[e];
+                }
+            }
+            if (pb) {
+#pragma unroll
+                for (int g = 0; g < SEG; ++g) {
+                    const Vec q = ld(pb + g * L + i);
+#pragma unroll
+                    for (int e = 0; e < W; ++e) x[g].v[e] -= cf * q.v[e];
+                }
+            }
+            if (FRONT != 0 || pb)
+#pragma unroll
+                for (int g = 0; g < SEG; ++g) st(xb + g * L + i, x[g]);
+        }
+#pragma unroll
+        for (int g = 0; g < SEG; ++g) st(sx + g * PER + i, x[g]);
+    }
+    __syncthreads();
+    double *pt = partial + (long long)b * Kmax * nchunk;  // [vector][chunk]
+    const real *Vb = V + (long long)b * Kmax * N + c0;
+    for (int j = w; j < Kb; j += KT / 32) {
+        const real *vj = Vb + (long long)j * N;
+        double t;
+        if constexpr (VEC) {  // (sums as in k_mdot)
+            DFAcc a;
+#pragma unroll
+            for (int g = 0; g < SEG; ++g) {
+                const float4 *v4 = reinterpret_cast<const float4 *>(vj + g * L), *x4 = reinterpret_cast<const float4 *>(sx + g * PER);
+                const int n4 = len >> 2;
+                int i = l;
+#pragma unroll 1
+                for (; i + 96 < n4; i += 128) {
+                    const float4 q0 = v4[i], q1 = v4[i + 32], q2 = v4[i + 64], q3 = v4[i + 96];
+                    const float4 y0 = x4[i], y1 = x4[i + 32], y2 = x4[i + 64], y3 = x4[i + 96];
+                    float t4 = q0.x * y0.x + q0.y * y0.y + q0.z * y0.z + q0.w * y0.w;
+                    t4 += q1.x * y1.x + q1.y * y1.y + q1.z * y1.z + q1.w * y1.w;
+                    t4 += q2.x * y2.x + q2.y * y2.y + q2.z * y2.z + q2.w * y2.w;
+                    t4 += q3.x * y3.x + q3.y * y3.y + q3.z * y3.z + q3.w * y3.w;
+                    a.add(t4);
+                }
+                for (; i < n4; i += 32) {
+                    const float4 q = v4[i], y = x4[i];
+                    a.add(q.x * y.x + q.y * y.y + q.z * y.z + q.w * y.w);
+                }
+            }
+            t = warp_sum(a.value());
+        } else {
+            real a = 0;
+#pragma unroll
+            for (int g = 0; g < SEG; ++g)
+                for (int i = l; i < len; i += 32) a += vj[g * L + i] * sx[g * PER + i];
+            if constexpr (sizeof(real) == 4) t = (double)warp_sumf(a);
+            else t = warp_sum(a);
+        }
+        if (l == 0) pt[(long long)j * nchunk + chunk] = t;
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        s_last = atomicAdd(done + b, 1) == (int)gridDim.x - 1;
+        if (s_last) done[b] = 0;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int j = w; j < Kb; j += KT / 32) {
+        const double *src = pt + (long long)j * nchunk;
+        double t = 0.0;
+#pragma unroll 8
+        for (int c = l; c < nchunk; c += 32) t += __ldcg(src + c);
+        t = warp_sum(t);
+        if (l == 0) out[(long long)b * Kmax + j] = t;
+    }
+}
+
+template <typename real, bool VEC>
+__global__ void __launch_bounds__(CT) k_gk_sub(real *V, long long N, int Kmax, int *K, const int *act, const double *__restrict__ c,
+                                               const real *__restrict__ x, long long xstride, double *__restrict__ partial,
+                                               int nblk, double *__restrict__ nrm2_out, const double *__restrict__ scale, double tol,
+                                               int *grow, int *__restrict__ slot, real *__restrict__ inv, double *__restrict__ sq1,
+                                               double *__restrict__ sq2, int *done) {
+    __shared__ real sc[64];
+    __shared__ double sh[CT / 32];
+    __shared__ int s_last;
+    const int b = blockIdx.y, tid = threadIdx.x;
+    if (act && !act[b]) return;
+    const int Kb = min(K[b], Kmax);
+    for (int j = tid; j < Kb; j += CT) sc[j] = (real)c[(long long)b * Kmax + j];
+    __syncthreads();
+    const long long i4 = ((long long)blockIdx.x * CT + tid) * 4;
+    const real *Vb = V + (long long)b * Kmax * N;
+    real *ob = V + ((long long)b * Kmax + Kb) * N;
+    const real *xb = x + b * xstride;
+    const bool put = Kb < Kmax;  // a full basis appends nothing
+    real n2 = 0;
+    if (i4 < N) {
+        real acc[4] = {0, 0, 0, 0}, v[4];
+        if (VEC) {
+            int j = 0;
+            for (; j + 3 < Kb; j += 4) {
+                const float4 q0 = *reinterpret_cast<const float4 *>(Vb + (long long)j * N + i4);
+                const float4 q1 = *reinterpret_cast<const float4 *>(Vb + (long long)(j + 1) * N + i4);
+                const float4 q2 = *reinterpret_cast<const float4 *>(Vb + (long long)(j + 2) * N + i4);
+                const float4 q3 = *reinterpret_cast<const float4 *>(Vb + (long long)(j + 3) * N + i4);
+                const real c0 = sc[j], c1 = sc[j + 1], c2 = sc[j + 2], c3 = sc[j + 3];
+                acc[0] += q0.x * c0 + q1.x * c1 + q2.x * c2 + q3.x * c3;
+                acc[1] += q0.y * c0 + q1.y * c1 + q2.y * c2 + q3.y * c3;
+                acc[2] += q0.z * c0 + q1.z * c1 + q2.z * c2 + q3.z * c3;
+                acc[3] += q0.w * c0 + q1.w * c1 + q2.w * c2 + q3.w * c3;
+            }
+            for (; j < Kb; ++j) {
+                const float4 q = *reinterpret_cast<const float4 *>(Vb + (long long)j * N + i4);
+                const real cj = sc[j];
+                acc[0] += q.x * cj;
+                acc[1] += q.y * cj;
+                acc[2] += q.z * cj;
+                acc[3] += q.w * cj;
+            }
+            const float4 y = *reinterpret_cast<const float4 *>(xb + i4);
+            v[0] = y.x - acc[0];
+            v[1] = y.y - acc[1];
+            v[2] = y.z - acc[2];
+            v[3] = y.w - acc[3];
+            if (put) *reinterpret_cast<float4 *>(ob + i4) = make_float4(v[0], v[1], v[2], v[3]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) n2 += v[e] * v[e];
+        } else {
+            for (int j = 0; j < Kb; ++j) {
+                const real cj = sc[j];
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (i4 + e < N) acc[e] += Vb[(long long)j * N + i4 + e] * cj;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (i4 + e < N) {
+                    v[e] = xb[i4 + e] - acc[e];
+                    if (put) ob[i4 + e] = v[e];
+                    n2 += v[e] * v[e];
+                }
+        }
+    }
+    const double t = block_sum_to_double(n2, sh);
+    if (tid == 0) {
+        partial[(long long)b * nblk + blockIdx.x] = t;
+        __threadfence();
+        s_last = atomicAdd(done + b, 1) == (int)gridDim.x - 1;
+        if (s_last) done[b] = 0;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const double *src = partial + (long long)b * nblk;
+    double s = 0.0;
+#pragma unroll 8
+    for (int q = tid; q < nblk; q += CT) s += __ldcg(src + q);
+    s = block_sum_to_double(s, sh);
+    if (tid != 0) return;
+    nrm2_out[b] = s;
+    const int g = grow[b];
+    if (g) {
+        const double r = sqrt(s);
+        if (sq1) sq1[b] = r;
+        if (sq2) sq2[b] = r;
+    }
+    const bool ok = append_ok(g, Kb, Kmax, s, scale, b, tol);
+    slot[b] = ok ? Kb : -1;
+    inv[b] = ok ? (real)(1.0 / sqrt(s)) : (real)0;
+    if (ok) K[b] = Kb + 1;
+    else grow[b] = 0;
+}
+
+// the vector in slot[b] (-1: none) times inv[b]
+template <typename real>
+__global__ void __launch_bounds__(KT) k_gk_scale(real *__restrict__ V, long long N, int Kmax, const int *__restrict__ slot,
+                                                 const real *__restrict__ inv) {
+    const int b = blockIdx.y, sl = slot[b];
+    if (sl < 0) return;
+    const real iv = inv[b];
+    real *vd = V + ((long long)b * Kmax + sl) * N;
+    const long long i0 = ((long long)blockIdx.x * KT + threadIdx.x) * 4;
+    if (sizeof(real) == 4 && i0 + 3 < N && (reinterpret_cast<uintptr_t>(vd + i0) & 15) == 0) {
+        float4 q = *reinterpret_cast<float4 *>(vd + i0);
+        q.x *= (float)iv;
+        q.y *= (float)iv;
+        q.z *= (float)iv;
+        q.w *= (float)iv;
+        *reinterpret_cast<float4 *>(vd + i0) = q;
+    } else {
+        for (long long i = i0; i < min(i0 + 4, N); ++i) vd[i] *= iv;
+    }
+}
+
 mof_status set_wait_polls(long long polls) {
     const long long v = polls < 0 ? MBAR_MAX_POLLS : (polls > MBAR_MAX_POLLS ? MBAR_MAX_POLLS : polls);
     MOF_CUDA(cudaMemcpyToSymbol(g_wait_polls, &v, sizeof(v)));
@@ -835,20 +1101,6 @@ void Krylov<real>::subtract(const BasisRef<real> &B, const double *c, long long 
 }
 
 template <typename real>
-int Krylov<real>::subtract_parts(const BasisRef<real> &B, const double *c, long long cstride, const real *x, long long xstride,
-                                 real *out, long long ostride, cudaStream_t st) const {
-    const int nb = (int)((B.N + 4LL * CT - 1) / (4LL * CT));
-    const bool vec = vec_ok<real>(B.V, B.N, (long long)B.Kmax * B.N) && (ostride % 4 == 0);
-    if (vec)
-        ::mof::count_launch(), k_combine<real, 1, true><<<dim3(nb, B.B), CT, 0, st>>>(B.V, B.N, B.Kmax, B.K, B.act, c, cstride, x,
-                                                                                   xstride, out, ostride, partial, nb);
-    else
-        ::mof::count_launch(), k_combine<real, 1, false><<<dim3(nb, B.B), CT, 0, st>>>(B.V, B.N, B.Kmax, B.K, B.act, c, cstride, x,
-                                                                                    xstride, out, ostride, partial, nb);
-    return nb;
-}
-
-template <typename real>
 void Krylov<real>::norm2(const real *x, long long N, long long xstride, int nb, double *out, cudaStream_t st,
                          bool exact) const {
     const int nc = (int)krylov_chunks(N);
@@ -885,6 +1137,43 @@ bool Krylov<real>::sub_dot(const BasisRef<real> &B, const double *c, long long c
 }
 
 template <typename real>
+void Krylov<real>::gk_half_step(const BasisRef<real> &B, int *Kmut, int front, const GkFront<real> &f, double *coef, double *nrm2_out,
+                                const double *scale, double tol, int *grow, double *sq1, double *sq2, int *done, bool scaled,
+                                cudaStream_t st) const {
+    const long long L = front == 1 ? B.N / 2 : B.N;
+    const int per = front == 1 ? dch<real>() / 2 : dch<real>(), nc = (int)((L + per - 1) / per);
+    auto al = [](const void *q) { return reinterpret_cast<uintptr_t>(q) % 16 == 0; };
+    const bool vec = vec_ok<real>(B.V, L, (long long)B.Kmax * B.N) && al(f.a) && al(f.s) && al(f.ux) && al(f.uy) && al(f.prev) &&
+                     al(f.x) && f.astride % 4 == 0 && f.pstride % 4 == 0 && f.xstride % 4 == 0 && f.fstride % 4 == 0;
+    // x: where the front leaves it (FRONT 0 without prev leaves it where it is)
+    const real *x = front == 0 && !f.prev ? f.a : f.x;
+    const long long xs = front == 0 && !f.prev ? f.astride : f.xstride;
+#define GK(F)                                                                                                                     \
+    if (vec) k_gk_dots<real, F, sizeof(real) == 4><<<dim3(nc, B.B), KT, 0, st>>>(B.V, B.N, B.Kmax, B.K, B.act, f, partial, nc, coef, done); \
+    else k_gk_dots<real, F, false><<<dim3(nc, B.B), KT, 0, st>>>(B.V, B.N, B.Kmax, B.K, B.act, f, partial, nc, coef, done);
+    ::mof::count_launch();
+    if (front == 0) {
+        GK(0)
+    } else if (front == 1) {
+        GK(1)
+    } else {
+        GK(2)
+    }
+#undef GK
+    const int nb = (int)((B.N + 4LL * CT - 1) / (4LL * CT));
+    int *slot = reinterpret_cast<int *>(aux);
+    real *inv = reinterpret_cast<real *>(aux + B.B);
+    ::mof::count_launch();
+    if (vec)
+        k_gk_sub<real, sizeof(real) == 4><<<dim3(nb, B.B), CT, 0, st>>>(B.V, B.N, B.Kmax, Kmut, B.act, coef, x, xs, partial, nb, nrm2_out,
+                                                                        scale, tol, grow, slot, inv, sq1, sq2, done);
+    else
+        k_gk_sub<real, false><<<dim3(nb, B.B), CT, 0, st>>>(B.V, B.N, B.Kmax, Kmut, B.act, coef, x, xs, partial, nb, nrm2_out, scale, tol,
+                                                            grow, slot, inv, sq1, sq2, done);
+    if (scaled) ::mof::count_launch(), k_gk_scale<real><<<dim3(nb, B.B), KT, 0, st>>>(B.V, B.N, B.Kmax, slot, inv);
+}
+
+template <typename real>
 void Krylov<real>::reorth(const BasisRef<real> &B, real *x, long long xstride, double *coef, double *nrm2_out,
                           cudaStream_t st) const {
     // classical Gram-Schmidt against V, twice (CGS2); coef is [B][Kmax] scratch
@@ -906,20 +1195,6 @@ void Krylov<real>::reorth_second(const BasisRef<real> &B, real *x, long long xst
         dots(B, x, xstride, coef, B.Kmax, 1.0, st);
     }
     subtract(B, coef, B.Kmax, x, xstride, x, xstride, nrm2_out, st);
-}
-
-template <typename real>
-int Krylov<real>::reorth_second_parts(const BasisRef<real> &B, real *x, long long xstride, const double *c1, double *coef,
-                                      cudaStream_t st, int kcap) const {
-    if (c1) {
-        if (!sub_dot(B, c1, B.Kmax, x, xstride, coef, st, kcap)) {
-            subtract(B, c1, B.Kmax, x, xstride, x, xstride, nullptr, st);
-            dots(B, x, xstride, coef, B.Kmax, 1.0, st);
-        }
-    } else {
-        dots(B, x, xstride, coef, B.Kmax, 1.0, st);
-    }
-    return subtract_parts(B, coef, B.Kmax, x, xstride, x, xstride, st);
 }
 
 template <typename real>

@@ -137,7 +137,7 @@ struct WS {
     real *ux, *uy, *ut, *bof, *Vof, *Uof, *AtB, *wv, *wu, *y1, *y2, *sof, *vnew_of, *q_of;
     double *GA, *GL, *gof, *zof, *gam, *nrm_of, *coef_of, *coefU_of, *scale_of, *alpha_of, *alpha1_of, *beta_of,
         *beta1_of, *bb_of, *Mg_of, *Linv_of, *pres_of, *Y_of, *Yd_of, *Yh_of, *Yrho_of;
-    int *Kv_of, *Ku_of, *grow_of, *gkb_of, *act_of, *app_of, *flag_of, *nL_of, *done_of, *nY_of;
+    int *Kv_of, *Ku_of, *grow_of, *gkb_of, *act_of, *app_of, *flag_of, *nL_of, *done_of, *done_im, *nY_of;
     real *wf_of = nullptr, *wl_of = nullptr;  // IRLS weights of Solve-OF with p = q = 1 (P ns, 4 P ns)
     double *rn_of = nullptr;                  // norm^2 of its residual before orthogonalisation (P)
     int pq1 = 0;                              // workspace holds the p = q = 1 arrays
@@ -423,6 +423,7 @@ static mof_status ensure_ws(mof_problem *p, const mof_solver_params &prm, int n_
         w->Yh_of = a.take<double>((size_t)P * Kof);
         w->Yrho_of = a.take<double>(P);
         w->done_of = a.take<int>(P);
+        w->done_im = a.take<int>(1);
         w->wf_of = a.take<real>(w->pq1 ? P * ns : 0);
         w->wl_of = a.take<real>(w->pq1 ? 4 * P * ns : 0);
         w->rn_of = a.take<double>(w->pq1 ? P : 0);
@@ -486,15 +487,6 @@ __global__ void k_neg(const real *__restrict__ a, real *__restrict__ b, long lon
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) b[i] = -a[i];
 }
 // x[b] -= coef[b] * y[b]  (coef device, per problem)
-template <typename real>
-__global__ void k_axpy_dev(real *__restrict__ x, long long xstride, const real *__restrict__ y, long long ystride,
-                           const double *__restrict__ coef, long long N, const int *__restrict__ act) {
-    const int b = blockIdx.y;
-    if (act && !act[b]) return;
-    const real c = block_scalar<real>(coef + b);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
-        x[b * xstride + i] -= c * y[b * ystride + i];
-}
 // err |= 16 when the data's squared norm is not finite (a NaN or an infinity in b)
 __global__ void k_flag_nonfinite(const double *__restrict__ v, int *__restrict__ err) {
     if (threadIdx.x == 0 && !isfinite(v[0])) atomicOr(err, 16);
@@ -502,10 +494,6 @@ __global__ void k_flag_nonfinite(const double *__restrict__ v, int *__restrict__
 __global__ void k_sqrt_into(const double *__restrict__ a, double *__restrict__ b, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) b[i] = sqrt(a[i]);
-}
-__global__ void k_sqrt_into_if(const double *__restrict__ a, double *__restrict__ b, int n, const int *__restrict__ act) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && (!act || act[i])) b[i] = sqrt(a[i]);
 }
 __global__ void k_mul_into(const double *__restrict__ a, const double *__restrict__ c, double *__restrict__ out, int n) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -540,43 +528,6 @@ __global__ void k_store_slot(real *__restrict__ base, long long N, const int *__
     if (!app[0]) return;
     real *d = base + (long long)(K[0] - 1) * N;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) d[i] = v[i];
-}
-
-// ------------------------------------------------------------ Upsilon kernels
-// GKB steps of Solve-OF, one problem per frame pair (blockIdx.y):
-//   out = Upsilon^T u_j - beta_j v_{j-1}     (V side, length 2 ns)
-template <typename real>
-__global__ void k_of_upsT(const real *__restrict__ ux, const real *__restrict__ uy, const real *__restrict__ U, int ldU,
-                          int j, const real *__restrict__ V, int ldV, const double *__restrict__ beta,
-                          real *__restrict__ out, long long ns, const int *__restrict__ act) {
-    const int b = blockIdx.y;
-    if (!act[b]) return;
-    const real *uj = U + ((long long)b * ldU + j) * ns;
-    const real *vp = j > 0 ? V + ((long long)b * ldV + j - 1) * 2 * ns : nullptr;
-    const real bj = j > 0 ? block_scalar<real>(beta + b) : (real)0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ns; i += (long long)gridDim.x * blockDim.x) {
-        const real r = uj[i];
-        real o0 = ux[b * ns + i] * r, o1 = uy[b * ns + i] * r;
-        if (vp) {
-            o0 -= bj * vp[i];
-            o1 -= bj * vp[ns + i];
-        }
-        out[b * 2 * ns + i] = o0;
-        out[b * 2 * ns + ns + i] = o1;
-    }
-}
-//   out = Upsilon v_j - alpha_j u_j           (U side, length ns)
-template <typename real>
-__global__ void k_of_ups(const real *__restrict__ ux, const real *__restrict__ uy, const real *__restrict__ V, int ldV, int j,
-                         const real *__restrict__ U, int ldU, const double *__restrict__ alpha, real *__restrict__ out,
-                         long long ns, const int *__restrict__ act) {
-    const int b = blockIdx.y;
-    if (!act[b]) return;
-    const real *vj = V + ((long long)b * ldV + j) * 2 * ns;
-    const real *uj = U + ((long long)b * ldU + j) * ns;
-    const real aj = block_scalar<real>(alpha + b);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ns; i += (long long)gridDim.x * blockDim.x)
-        out[b * ns + i] = ux[b * ns + i] * vj[i] + uy[b * ns + i] * vj[ns + i] - aj * uj[i];
 }
 
 // Graph Laplacian of one component with free boundary: (Psi^T Psi f)(x,y).
@@ -1486,16 +1437,19 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
             ::mof::count_launch(), k_sqrt_into<<<pb, 64, 0, gst>>>(nrmg, w.scale_of + b0, nb);
             // u_1 = b / ||b||
             kg.append(BU, Kug, bofg, ns, bbg, nullptr, 0.0, gkbg, nullptr, nullptr, gst);
-            for (int j = 0; j < w.of_ell && j < prm.of_ell; ++j) {
-                ::mof::count_launch(), k_of_upsT<real><<<dim3(fb(ns), nb), 256, 0, gst>>>(uxg, uyg, Ug, ldU, j, Vg, Kof, w.beta_of + b0, wvg, ns, gkbg);
+            const real *inv = reinterpret_cast<const real *>(kg.aux + nb);  // scale of the vector appended last
+            int *doneg = w.done_of + b0;
+            const int steps = std::min(w.of_ell, prm.of_ell);
+            for (int j = 0; j < steps; ++j) {
                 // V^T x = 0 by the recurrence; alpha (and alpha_1) = ||x|| with the append
-                const int nv = kg.reorth_second_parts(BV, wvg, N2, nullptr, w.coef_of + (long long)b0 * Kof, gst);
-                kg.append_parts(BV, Kvg, wvg, N2, nv, nrmg, j == 0 ? nullptr : w.alpha1_of + b0, tol, gkbg, nullptr, nullptr,
-                                w.alpha_of + b0, j == 0 ? w.alpha1_of + b0 : nullptr, gst);
-                ::mof::count_launch(), k_of_ups<real><<<dim3(fb(ns), nb), 256, 0, gst>>>(uxg, uyg, Vg, Kof, j, Ug, ldU, w.alpha_of + b0, wug, ns, gkbg);
-                const int nu = kg.reorth_second_parts(BU, wug, ns, nullptr, w.coefU_of + (long long)b0 * ldU, gst);
-                kg.append_parts(BU, Kug, wug, ns, nu, nrmg, w.beta1_of + b0, tol, gkbg, nullptr, nullptr, w.beta_of + b0, nullptr,
-                                gst);
+                GkFront<real> f{nullptr, Ug + j * ns, ldU * ns, uxg, uyg, ns, j ? inv : nullptr, w.beta_of + b0,
+                                j ? Vg + (j - 1) * N2 : nullptr, Kof * N2, wvg, N2};
+                kg.gk_half_step(BV, Kvg, 1, f, w.coef_of + (long long)b0 * Kof, nrmg, j == 0 ? nullptr : w.alpha1_of + b0, tol, gkbg,
+                                w.alpha_of + b0, j == 0 ? w.alpha1_of + b0 : nullptr, doneg, j == steps - 1, gst);
+                if (j == steps - 1) break;  // u_{l+1} is not needed
+                GkFront<real> h{nullptr, Vg + j * N2, Kof * N2, uxg, uyg, ns, inv, w.alpha_of + b0, Ug + j * ns, ldU * ns, wug, ns};
+                kg.gk_half_step(BU, Kug, 2, h, w.coefU_of + (long long)b0 * ldU, nrmg, w.beta1_of + b0, tol, gkbg, w.beta_of + b0, nullptr,
+                                doneg, false, gst);
             }
         }
         if (!pq1) {
@@ -1778,7 +1732,7 @@ mof_status SolveRun<real>::begin(cudaStream_t ust) {
     tg_smem = theta_gram_smem<real>(Kmax);
     MOF_CUDA(cudaFuncSetAttribute(k_theta_gram<real>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tg_smem));
 
-    BasisRef<real> BV{w.V, n, Kmax, 1, w.K, nullptr};
+    BasisRef<real> BV{w.V, n, Kmax, 1, w.K, nullptr}, BG{w.V, n, Kmax, 1, w.K, w.gkb};
     BasisRef<real> BH{w.HV, m, Kmax, 1, w.K, nullptr};
     BasisRef<real> BU{w.U, m, w.ell + 1, 1, w.KU, w.gkb};
     {
@@ -1805,17 +1759,13 @@ mof_status SolveRun<real>::begin(cudaStream_t ust) {
         kr.append(BU, w.KU, w.b, m, w.bb, nullptr, 0.0, w.gkb, nullptr, nullptr, st);
         for (int j = 0; j < prm.ell; ++j) {
             MOF_TRY(launch_backproject<real>(p, w.U + (long long)j * m, w.r, st, prm.plain));
-            if (j > 0) ::mof::count_launch(), k_axpy_dev<real><<<dim3(fb(n), 1), 256, 0, st>>>(w.r, n, w.V + (long long)(j - 1) * n, n, w.beta, n, w.gkb);
-            kr.reorth_second(BV, w.r, n, nullptr, w.coef, w.nrm2, st);  // V^T x = 0 by the recurrence
-            if (j == 0) ::mof::count_launch(), k_sqrt_into_if<<<1, 1, 0, st>>>(w.nrm2, w.alpha1, 1, w.gkb);
-            ::mof::count_launch(), k_sqrt_into_if<<<1, 1, 0, st>>>(w.nrm2, w.alpha, 1, w.gkb);
-            kr.append(BV, w.K, w.r, n, w.nrm2, j == 0 ? nullptr : w.alpha1, tol, w.gkb, nullptr, nullptr, st);
+            GkFront<real> f{w.r, nullptr, n, nullptr, nullptr, 0, nullptr, w.beta, j ? w.V + (long long)(j - 1) * n : nullptr, n, w.r, n};
+            kr.gk_half_step(BG, w.K, 0, f, w.coef, w.nrm2, j == 0 ? nullptr : w.alpha1, tol, w.gkb, w.alpha, j == 0 ? w.alpha1 : nullptr,
+                            w.done_im, true, st);
             MOF_TRY(launch_project<real>(p, w.V + (long long)j * n, w.uT, w.HV + (long long)j * m, st, prm.plain));
-            ::mof::count_launch(), k_copy<real><<<fb(m), 256, 0, st>>>(w.HV + (long long)j * m, w.tm, m);
-            ::mof::count_launch(), k_axpy_dev<real><<<dim3(fb(m), 1), 256, 0, st>>>(w.tm, m, w.U + (long long)j * m, m, w.alpha, m, w.gkb);
-            kr.reorth_second(BU, w.tm, m, nullptr, w.coef, w.nrm2, st);
-            ::mof::count_launch(), k_sqrt_into_if<<<1, 1, 0, st>>>(w.nrm2, w.beta, 1, w.gkb);
-            kr.append(BU, w.KU, w.tm, m, w.nrm2, w.beta1, tol, w.gkb, nullptr, nullptr, st);
+            if (j == prm.ell - 1) break;  // u_{l+1} is not needed
+            GkFront<real> h{w.HV + (long long)j * m, nullptr, m, nullptr, nullptr, 0, nullptr, w.alpha, w.U + (long long)j * m, m, w.tm, m};
+            kr.gk_half_step(BU, w.KU, 0, h, w.coef, w.nrm2, w.beta1, tol, w.gkb, w.beta, nullptr, w.done_im, true, st);
         }
         // breakdown scale of the expansions: ||H^T b|| = alpha_1 beta_1
         ::mof::count_launch(), k_mul_into<<<1, 1, 0, st>>>(w.alpha1, w.beta1, w.scaleR, 1);

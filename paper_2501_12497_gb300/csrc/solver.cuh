@@ -44,6 +44,24 @@ struct DotOuts {
     DotOut o[3];
 };
 
+// What a Golub-Kahan half-step starts from (k_gk_dots): a (front 0), or s and the velocity gradients
+// ux, uy (fronts 1 and 2, s scaled in place by inv when given); coef, prev: the recurrence term
+// (prev null: none); x receives the vector.
+template <typename real>
+struct GkFront {
+    const real *a;
+    real *s;
+    long long astride;  // of a or s
+    const real *ux, *uy;
+    long long fstride;
+    const real *inv;
+    const double *coef;
+    const real *prev;
+    long long pstride;
+    real *x;
+    long long xstride;
+};
+
 long long krylov_chunks(long long N);
 // doubles of Krylov::partial needed per problem of length N and basis capacity Kmax
 long long krylov_partial_doubles(long long N, int Kmax);
@@ -71,6 +89,13 @@ struct Krylov {
                   long long ostride, double *nrm2_out, cudaStream_t st) const;
     void norm2(const real *x, long long N, long long xstride, int nb, double *out, cudaStream_t st,
                bool exact = false) const;
+    // One Golub-Kahan half-step: x from the front, x - V V^T x, its norm (||x||^2 in nrm2_out,
+    // ||x|| in sq1 / sq2, which may be null, for problems still growing) and the append (as
+    // append_parts). scaled: the new vector is normalised here; else it stays x' until the next
+    // half-step's front scales it by inv = aux[B..2B) (as real). done: [B] ints, zero between calls.
+    void gk_half_step(const BasisRef<real> &B, int *Kmut, int front, const GkFront<real> &f, double *coef, double *nrm2_out,
+                      const double *scale, double tol, int *grow, double *sq1, double *sq2, int *done, bool scaled,
+                      cudaStream_t st) const;
     // x[b] <- (I - V V^T)^2 x[b] (classical Gram-Schmidt twice); ||x||^2 -> nrm2_out
     void reorth(const BasisRef<real> &B, real *x, long long xstride, double *coef, double *nrm2_out, cudaStream_t st) const;
     // the same with the first projection's coefficients V^T x supplied by the caller from an
@@ -86,13 +111,6 @@ struct Krylov {
     // partial (at partial + B.B * nparts * Kmax), their number per problem in *nparts
     bool sub_dot(const BasisRef<real> &B, const double *c, long long cstride, real *x, long long xstride, double *out,
                  cudaStream_t st, int kcap = 0, int *nparts = nullptr) const;
-    // x[b] <- x[b] - V[b] c[b], the per-block partials of ||x[b]||^2 left in partial;
-    // returns their number per problem (for append_parts)
-    int subtract_parts(const BasisRef<real> &B, const double *c, long long cstride, const real *x, long long xstride,
-                       real *out, long long ostride, cudaStream_t st) const;
-    // reorth_second with the final norm left as partials (returns their number per problem)
-    int reorth_second_parts(const BasisRef<real> &B, real *x, long long xstride, const double *c1, double *coef,
-                            cudaStream_t st, int kcap = 0) const;
     // append with ||x||^2 summed from the nparts partials of the preceding update (written to
     // nrm2_out), and sqrt(||x||^2) written to sq1 / sq2 (may be null) for problems still growing
     // (parts: where the partials are, default the start of partial)
