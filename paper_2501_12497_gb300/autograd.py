@@ -1,7 +1,8 @@
 """Differentiable forms of the MMGKS-OF operators for torch.autograd.
 
-Each forward and each backward pass is one call into the C ABI (hand-written
-sm_103a kernels); this module only allocates outputs and routes gradients:
+Each forward and each backward pass is one or two calls into the C ABI (hand-written
+sm_103a kernels); the nodes that allocate outputs and route gradients are native
+(csrc/autograd.cpp):
 
   project(p, u)               b = H u                      (Sec. 2.1)
       backward: du = H^T db                                 (mof_apply_AT)
@@ -15,65 +16,39 @@ clipped (derivative from the right at integer sample positions). Tensors are
 CUDA tensors of the problem's precision, flat or of any shape with the
 problem's element counts; gradients come back flat.
 """
+import importlib.util
+import os
+
 import torch
 
 from . import api
+from .build import AUTOGRAD_PATH
+
+_native = None
+
+
+def _nodes():
+    global _native
+    if _native is None:
+        api.load()
+        if not os.path.exists(AUTOGRAD_PATH):
+            raise RuntimeError("_autograd.so is not built (%s); run __graft_entry__.build()" % AUTOGRAD_PATH)
+        spec = importlib.util.spec_from_file_location("_autograd", AUTOGRAD_PATH)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        _native = mod
+    return _native
 
 
 def _dtype(p):
     return torch.float64 if p.precision == api.MOF_FP64 else torch.float32
 
 
-def _flat(x):
-    return x.contiguous().reshape(-1)
-
-
-class _Project(torch.autograd.Function):
-    @staticmethod
-    def forward(ctx, u, p):
-        ctx.p = p
-        b = torch.empty(p.m, dtype=u.dtype, device=u.device)
-        api.mof_apply_A(p, _flat(u), b)
-        return b
-
-    @staticmethod
-    def backward(ctx, db):
-        p = ctx.p
-        du = torch.empty(p.n, dtype=db.dtype, device=db.device)
-        api.mof_apply_AT(p, _flat(db), du)
-        return du, None
-
-
-class _FlowResidual(torch.autograd.Function):
-    @staticmethod
-    def forward(ctx, u, s, sr, p):
-        u, s, sr = _flat(u), _flat(s), _flat(sr)
-        ctx.p = p
-        ctx.save_for_backward(u, s, sr)
-        r = torch.empty(2 * (p.nt - 1) * p.nx * p.ny, dtype=u.dtype, device=u.device)
-        api.mof_apply_flow(p, u, s, sr, r)
-        return r
-
-    @staticmethod
-    def backward(ctx, dr):
-        p = ctx.p
-        u, s, sr = ctx.saved_tensors
-        dr = _flat(dr)
-        du = gs = gsr = None
-        if ctx.needs_input_grad[0]:
-            du = torch.empty_like(u)
-            api.mof_apply_flowT(p, dr, s, sr, du)
-        if ctx.needs_input_grad[1] or ctx.needs_input_grad[2]:
-            gs, gsr = torch.empty_like(s), torch.empty_like(sr)
-            api.mof_apply_flow_ds(p, u, s, sr, dr, gs, gsr)
-        return du, gs, gsr, None
-
-
 def project(p, u):
     """H u for a problem p, differentiable in u."""
     if u.dtype != _dtype(p):
         raise TypeError("u must be %s for this problem" % _dtype(p))
-    return _Project.apply(u, p)
+    return _nodes().project(p, u)
 
 
 def flow_residual(p, u, s, sr):
@@ -81,4 +56,4 @@ def flow_residual(p, u, s, sr):
     for name, t in (("u", u), ("s", s), ("sr", sr)):
         if t.dtype != _dtype(p):
             raise TypeError("%s must be %s for this problem" % (name, _dtype(p)))
-    return _FlowResidual.apply(u, s, sr, p)
+    return _nodes().flow_residual(p, u, s, sr)
