@@ -83,12 +83,16 @@ static AngleParams angle_params(double theta, int frame, int nx, int ny, int nb,
     P.wfoot_d = h / mu;
     P.rfoot = (float)P.rfoot_d;
     P.wfoot = (float)P.wfoot_d;
-    P.inv_rfoot = (float)(1.0 / P.rfoot_d);
+    P.inv_rfoot_d = 1.0 / P.rfoot_d;
+    P.inv_rfoot = (float)P.inv_rfoot_d;
     P.wide = !(std::fabs(P.f0_c) < F0_LIMIT && std::fabs(P.f0_c + (nb - 1) * P.f0_k) < F0_LIMIT);
     P.f0kQ = P.wide ? 0 : std::llround(std::ldexp(P.f0_k, 40));
     P.f0cQ = P.wide ? 0 : std::llround(std::ldexp(P.f0_c, 40));
     P.dfQ = std::llround(std::ldexp(P.df, 40));
     P.wstep_lo = (float)(P.wstep_d - (double)P.wstep);
+    const double d51 = std::ldexp(P.df, 51), d51f = std::floor(d51);
+    P.df51 = (long long)d51f;
+    P.df51_lo = (unsigned)std::ldexp(d51 - d51f, 32);
     return P;
 }
 
@@ -243,7 +247,16 @@ mof_status mof_problem_create(const mof_geometry *g, int precision, mof_problem 
             P.t0Q = std::llround(std::ldexp(P.t0, 40));
             P.tAQ = std::llround(std::ldexp(P.tA, 40));
             P.tBQ = std::llround(std::ldexp(P.tB, 40));
+            P.tA55 = std::llround(std::ldexp(P.tA, 55));
+            P.tB55 = std::llround(std::ldexp(P.tB, 55));
         }
+    // FP64 in fixed point: the frame's extent, and the bin coordinates at its corners
+    p->fix64 = std::max(g->nx, g->ny) <= FIX64_LIMIT && g->nb <= FIX64_LIMIT;
+    for (const AngleParams &P : tab) {
+        const double ax = (g->nx + 31) * P.tA, by = (g->ny + 31) * P.tB;
+        for (double v : {P.t0, P.t0 + ax, P.t0 + by, P.t0 + ax + by})
+            if (!(std::fabs(v) <= FIX64_LIMIT)) p->fix64 = false;
+    }
     cudaError_t e = cudaGetDevice(&p->device);
     if (e == cudaSuccess) e = cudaMalloc(&p->d_ang, sizeof(AngleParams) * A);
     if (e == cudaSuccess) e = cudaMalloc(&p->d_aoff, sizeof(int) * (g->nt + 1));

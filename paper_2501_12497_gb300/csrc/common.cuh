@@ -65,7 +65,7 @@ struct AngleParams {
     float wfoot;        // footprint height h / mu
     int frame;          // frame this angle belongs to
     int pad_;
-    double wstep_d, rfoot_d, wfoot_d;  // the same three in FP64 (FP64 kernels)
+    double wstep_d, rfoot_d, wfoot_d, inv_rfoot_d;  // the same three in FP64 and 1 / rfoot (FP64 kernels)
     // FP32 march in fixed point, units of 2^-40 pixels: f(j) = f0cQ + k f0kQ + j dfQ; wide: some
     // ray's f0 lies beyond F0_LIMIT pixels (f0_c and f0_k then give it in FP64)
     long long f0kQ, f0cQ, dfQ;
@@ -73,7 +73,15 @@ struct AngleParams {
     float wstep_lo;     // wstep_d - wstep
     long long t0Q, tAQ, tBQ;  // t0, tA, tB in units of 2^-40 bins (set where mof_problem::bp_reach > 0)
     float inv_rfoot;    // 1 / rfoot
+    // FP64 kernels in fixed point: df in units of 2^-51 with 32 bits more; tA, tB in units of 2^-55
+    // (set where mof_problem::bp_reach > 0)
+    unsigned df51_lo;
+    long long df51, tA55, tB55;
 };
+
+// Largest frame extent and bin coordinate of the FP64 kernels in fixed point (12 bits and the sign, a
+// margin for the steps beside the frame)
+constexpr double FIX64_LIMIT = 4000.0;
 
 // Fan beam (flat detector): one Joseph march per ray (view a, bin k), stored per
 // ray because the rays of one view are not parallel. The crossing of step j is
@@ -120,6 +128,7 @@ struct mof_problem {
     int timing = 0;
     void *timer = nullptr;              // kernel-class timer (solver.cu)
     int warp_mode = 0;                  // M(s): 0 bilinear, 1 rounding and clipping (Sec. 3)
+    bool fix64 = false;                 // parallel FP64 pair: every coordinate it meets lies within FIX64_LIMIT
     int bp_reach = 0;                   // parallel FP32 transpose: footprints within this many bins each side (1, 2), 0: any
     int fan = 0;                        // 1: fan beam with a flat detector
     int fan_tile = 0;                   // 1: the tiled FP32 transpose applies
