@@ -1145,7 +1145,9 @@ constexpr int TG_S = TG_ROWS + 4;  // column stride of the shared row tile
 // four columns puts the 128-bit reads of the eight column groups a warp's 4x4
 // blocks touch on eight different bank quads
 __host__ __device__ constexpr int tg_col(int j) { return j * TG_S + 4 * (j / 4); }
-constexpr int TG_MAXG = 8;         // row groups per 4x4 block at most
+// Row groups per 4x4 block at most: 16 busy 96 threads at K = 10 (1024x1024x64: 24.9 ms for the four Grams
+// of two iterations; 8: 27.7, 32: 25.2, 64: 25.6, where the compensated sums of more groups cost more)
+constexpr int TG_MAXG = 16;
 constexpr int TG_VEC = 8;          // basis vectors per step of the difference rows (16 loads in flight)
 
 template <typename real>
