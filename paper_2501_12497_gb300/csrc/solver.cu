@@ -636,13 +636,16 @@ __global__ void k_of_proj_gram(const double *__restrict__ GA, const double *__re
 //   G_L[i][j] = (L v_i)^T (L v_j) = v_i^T (L^T L v_j),   g[j] = (Ups v_j)^T b,
 // with Ups v = u_x v_x + u_y v_y pointwise and L the forward differences in x
 // and y of both velocity components (no boundary row), so L^T L is the graph
-// Laplacian of each component with free boundary. Column j is blockIdx.z (mode
-// 0: the first columns, j < K) or K - 1 (mode 1: the vector appended last,
+// Laplacian of each component with free boundary. Column j is one of the first
+// ncol (mode 0, j < K) or K - 1 (mode 1, ncol = 1: the vector appended last,
 // where appended). A CTA owns a chunk of OFC pixels of one pair: it stages
 // Ups^T Ups v_j and L^T L v_j (both components) in shared memory, and its warps
 // stream the basis vectors i = w, w + 8, ... over the chunk with plain
 // coalesced loads, taking two dot products per vector, with sums per chunk in
-// the storage precision; k_of_gram_reduce adds the chunks in FP64.
+// the storage precision; k_of_gram_reduce adds the chunks in FP64. The columns of
+// a chunk run side by side, so that all but the first find its vectors in L2 (63
+// pairs of 1024^2, ten columns: 6.9 ms, now staging and dots; column after column, 55 vector reads from
+// HBM, 7.9).
 constexpr int OFG_T = 256;
 template <typename real>
 constexpr int ofc() { return 4096 / (int)sizeof(real); }  // pixels per chunk: 1024 (FP32), 512 (FP64)
@@ -655,23 +658,24 @@ __device__ __forceinline__ real warp_sum_r(real v) {
 
 template <typename real>
 __global__ void __launch_bounds__(OFG_T) k_of_gram_cols(const real *__restrict__ V, int Kmax, const int *__restrict__ K,
-                                                        const int *__restrict__ act, int mode, const real *__restrict__ ux,
-                                                        const real *__restrict__ uy, const real *__restrict__ bof, int nx,
-                                                        int ny, double *__restrict__ partial) {
+                                                        const int *__restrict__ act, int mode, int ncol,
+                                                        const real *__restrict__ ux, const real *__restrict__ uy,
+                                                        const real *__restrict__ bof, int nx, int ny,
+                                                        double *__restrict__ partial) {
     constexpr int OFC = ofc<real>();
     __shared__ __align__(16) real s_y[4][OFC];  // (Ups^T Ups v_j)_x, _y, (L^T L v_j)_x, _y
     __shared__ real s_red[OFG_T / 32];
-    const int b = blockIdx.y, chunk = blockIdx.x, nchunk = gridDim.x;
+    const int b = blockIdx.y, chunk = blockIdx.x / ncol, col = blockIdx.x - chunk * ncol, nchunk = gridDim.x / ncol;
     if (!act[b]) return;
     const int Kb = min(K[b], Kmax);
-    const int j = mode == 0 ? (int)blockIdx.z : Kb - 1;
+    const int j = mode == 0 ? col : Kb - 1;
     if (j < 0 || j >= Kb) return;
     const long long ns = (long long)nx * ny, N2 = 2 * ns;
     const int c0 = chunk * OFC;
     const int len = (int)min((long long)OFC, ns - c0);
     const real *Vb = V + (long long)b * Kmax * N2;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    double *out = partial + (((long long)b * gridDim.z + blockIdx.z) * nchunk + chunk) * (2 * Kmax + 1);
+    double *out = partial + (((long long)b * ncol + col) * nchunk + chunk) * (2 * Kmax + 1);
     // stage the normal-equation parts of column j; g_j on the way
     const real *vj = Vb + (long long)j * N2;
     real gs = 0;
@@ -718,7 +722,7 @@ __global__ void __launch_bounds__(OFG_T) k_of_gram_cols(const real *__restrict__
             // two quads of both components per step (16 products per partial); OFC / 4 is a
             // multiple of 64, so every lane takes the same number of steps
             for (int q = lane; q < OFC / 4; q += 64) {
-                const float4 X = __ldcs(X4 + q), Y = __ldcs(Y4 + q), X2 = __ldcs(X4 + q + 32), Y2 = __ldcs(Y4 + q + 32);
+                const float4 X = X4[q], Y = Y4[q], X2 = X4[q + 32], Y2 = Y4[q + 32];
                 const float4 a0 = A0[q], a1 = A1[q], l0 = L0[q], l1 = L1[q];
                 const float4 b0 = A0[q + 32], b1 = A1[q + 32], m0 = L0[q + 32], m1 = L1[q + 32];
                 float pa = X.x * a0.x + X.y * a0.y + X.z * a0.z + X.w * a0.w + Y.x * a1.x + Y.y * a1.y + Y.z * a1.z + Y.w * a1.w;
@@ -1458,7 +1462,7 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
             Scope sc(tm, "of_gram", gst);
             const int gram_ctas = (int)((ns + ofc<real>() - 1) / ofc<real>()), gram_red = (2 * Kof + 1 + 7) / 8;
             const int ncol = std::min(prm.of_ell, Kof);
-            ::mof::count_launch(), k_of_gram_cols<real><<<dim3(gram_ctas, nb, ncol), OFG_T, 0, gst>>>(Vg, Kof, Kvg, actg, 0, uxg, uyg, bofg,
+            ::mof::count_launch(), k_of_gram_cols<real><<<dim3(gram_ctas * ncol, nb), OFG_T, 0, gst>>>(Vg, Kof, Kvg, actg, 0, ncol, uxg, uyg, bofg,
                                                                                                    p->nx, p->ny, kg.partial);
             ::mof::count_launch(), k_of_gram_reduce<<<dim3(gram_red, nb, ncol), 256, 0, gst>>>(kg.partial, gram_ctas, Kof, Kvg, actg, 0,
                                                                                              w.GA + b0 * KK, w.GL + b0 * KK,
@@ -1588,7 +1592,7 @@ static mof_status solve_of_impl(mof_problem *p, const mof_solver_params &prm, WS
             }
             if (!pq1) {
                 Scope sc(tm, "of_gram", gst);
-                ::mof::count_launch(), k_of_gram_cols<real><<<dim3(gram_ctas, nb, 1), OFG_T, 0, gst>>>(Vg, Kof, Kvg, appg, 1, uxg, uyg, bofg,
+                ::mof::count_launch(), k_of_gram_cols<real><<<dim3(gram_ctas, nb), OFG_T, 0, gst>>>(Vg, Kof, Kvg, appg, 1, 1, uxg, uyg, bofg,
                                                                                                     p->nx, p->ny, kg.partial);
                 ::mof::count_launch(), k_of_gram_reduce<<<dim3(gram_red, nb, 1), 256, 0, gst>>>(kg.partial, gram_ctas, Kof, Kvg, appg, 1,
                                                                                               w.GA + b0 * KK, w.GL + b0 * KK,
