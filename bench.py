@@ -359,6 +359,28 @@ def class_bytes(name, w, of_scale=1, tau=1):
     return None
 
 
+def fused_bytes(name, w, of_scale=1, tau=1):
+    """class_bytes as the kernels divide the work: the residual's Laplacian is taken with the
+    residual (class of_resid) and a new vector is scaled by s = V z on its way through, so the
+    projection pass moves K + 5 vectors and s = V z one more per vector appended; a Golub-Kahan
+    half-step takes its dot products while it forms its vector, subtracts straight into the
+    basis and leaves the scale to the next."""
+    m = class_bytes(name, w, of_scale, tau)
+    if m is None or name not in ("of_subdot", "of_combine", "of_gkb"):
+        return m
+    calls = sum(1 for k in range(1, N_OUTER) if k % tau == 0)
+    ns, P = (w.nx // of_scale) * (w.ny // of_scale), w.nt - 1
+    if name == "of_subdot":
+        return m[0] - calls * P * 8 * ns * 4 * (OF_ITERS - 1), m[1]
+    if name == "of_combine":
+        return m[0] + calls * P * 8 * ns * (OF_ITERS - 1), m[1]
+    # per step j < OF_ELL: u_j and the fields read, u_j scaled (j > 0), x written (5 ns), dot products
+    # with the j stored v, the update into the basis (4 ns and the j again); but for the last: v_j
+    # read and scaled, the fields, x (7 ns), dot products with j + 1 u, the update (2 ns, the u again)
+    return calls * P * 4 * ns * (5 + sum(9 + 4 * j + (j > 0) for j in range(OF_ELL)) +
+                                 sum(11 + 2 * j for j in range(OF_ELL - 1))), m[1]
+
+
 # DRAM bytes over algorithmic bytes per launch of the kernel that dominates a class, from an
 # ncu capture of that kernel (k_of_proj_gram_pass: 31 pairs of 256x256 frames at K = 20 and
 # 21, 408.9 MB for 406.3 MB and 425.1 MB for 422.6 MB); the class's traffic per launch is
@@ -367,11 +389,11 @@ TRAFFIC_RATIO = {"of_subdot": 1.006}
 
 # the main kernel of each timing class
 CLASS_KERNEL = {
-    "of_gkb": "Golub-Kahan start of Solve-OF (k_of_upsT, k_of_ups, k_mdot, k_combine, k_append)",
+    "of_gkb": "Golub-Kahan start of Solve-OF (k_gk_dots, k_gk_sub)",
     "of_gram": "k_of_gram_cols (Gram columns of the Solve-OF Golub-Kahan start, with their reduction)",
-    "of_subdot": "k_of_proj_gram_pass (Solve-OF projection pass with the new Gram column; with the residual's "
-                 "Laplacian, the chunk reduction and the append)",
-    "of_combine": "k_combine (s = V z of Solve-OF)",
+    "of_subdot": "k_of_proj_gram_pass (Solve-OF projection pass with the new Gram column; with the reduction of "
+                 "its partials and the append decision)",
+    "of_combine": "k_of_combine (s = V z of Solve-OF)",
     "theta_gram": "k_theta_gram (weighted Gram of Theta V)",
 }
 
@@ -540,7 +562,7 @@ def run_ours(args):
     step1_ms = sum(v[0] for v in class_ms.values())
     modeled = {}
     for name, (ms, cnt) in class_ms.items():
-        m = class_bytes(name, w, args.of_scale, args.tau) if args.of_pq == 2 and not fp64 else None
+        m = fused_bytes(name, w, args.of_scale, args.tau) if args.of_pq == 2 and not fp64 else None
         if m is None or ms <= 0:
             continue
         nbytes, nlaunch = m
