@@ -1221,7 +1221,7 @@ void Krylov<real>::append(const BasisRef<real> &B, int *Kmut, const real *x, lon
     ::mof::count_launch(), k_append<real><<<dim3(blocks, B.B), KT, 0, st>>>(B.V, B.N, B.Kmax, slot, inv, x, xstride, stage);
 }
 
-// The chunk partials of k_of_proj_gram_pass summed in FP64 (one warp per output, lanes over its
+// The totals of k_of_proj_gram_pass (one per warp and output) summed in FP64 (one warp per output, lanes over its
 // contiguous chunks, fixed order): res[b][0..3 Kmax + 4). The last CTA of a pair to finish
 // (counter done[b], left at zero) takes the append decision on ||x'|| (as k_append_prep) and
 // writes, for an appended vector v = x' / ||x'||, its Gram columns G_A, G_L, g, its Euclidean

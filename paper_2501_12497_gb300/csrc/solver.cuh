@@ -128,7 +128,7 @@ struct Krylov {
 // basis forming x' = r - V d (into the slot behind the basis) with the dot products that give the
 // new vector's Gram columns, then the append decision and the new columns of G_A, G_L, g and Mg.
 // launch_of_combine: s = V z, scaling a vector appended since the last call to x' / ||x'||.
-// partial: [B][chunks][3 Kmax + 4] doubles; res: [B][3 Kmax + 4]; aux: 2 B doubles (the slot and
+// partial: [B][3 Kmax + 4][of_pass_parts] doubles; res: [B][3 Kmax + 4]; aux: 2 B doubles (the slot and
 // scale between an append and the next combine); done: [B] ints, zero between calls.
 long long of_pass_parts(long long ns, int pairs);
 int of_pass_stride(int Kmax);
