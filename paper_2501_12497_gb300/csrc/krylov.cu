@@ -1316,8 +1316,10 @@ __global__ void __launch_bounds__(PF_T) k_of_pass_finish(const double *__restric
 
 // s[b] = sum_j V[b][j] z[b][j] for Solve-OF, with the scale of a vector appended by
 // k_of_pass_finish: slot[b] (-1: none) holds x' still, which becomes x' inv[b] here on its way
-// through (one pass over the vector less than a separate append). 16 bytes per thread.
-template <typename real>
+// through (one pass over the vector less than a separate append). 16 bytes per thread; VEC: s on a
+// 16-byte boundary, else (a caller's own array in the plain form and in timed calls) it is stored value
+// by value.
+template <typename real, bool VEC>
 __global__ void __launch_bounds__(CT) k_of_combine(real *__restrict__ V, long long N, int Kmax, const int *__restrict__ K,
                                                    const double *__restrict__ z, const int *__restrict__ slot,
                                                    const real *__restrict__ inv, real *__restrict__ out) {
@@ -1330,7 +1332,7 @@ __global__ void __launch_bounds__(CT) k_of_combine(real *__restrict__ V, long lo
     const long long i = ((long long)blockIdx.x * CT + threadIdx.x) * EPT;
     if (i >= N) return;
     real *Vb = V + (long long)b * Kmax * N + i;
-    real acc[EPT];
+    __align__(16) real acc[EPT];
 #pragma unroll
     for (int e = 0; e < EPT; ++e) acc[e] = 0;
     const int Kd = sl >= 0 ? Kb - 1 : Kb;  // a new vector is the last one
@@ -1360,7 +1362,13 @@ __global__ void __launch_bounds__(CT) k_of_combine(real *__restrict__ V, long lo
         }
         *reinterpret_cast<vec_t *>(Vb + (long long)Kd * N) = q;
     }
-    *reinterpret_cast<vec_t *>(out + (long long)b * N + i) = *reinterpret_cast<vec_t *>(acc);
+    real *o = out + (long long)b * N + i;
+    if (VEC) {
+        *reinterpret_cast<vec_t *>(o) = *reinterpret_cast<vec_t *>(acc);
+    } else {
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) o[e] = acc[e];
+    }
 }
 
 template <typename real>
@@ -1368,8 +1376,10 @@ mof_status launch_of_combine(const BasisRef<real> &B, const double *z, double *a
     const int *slot = reinterpret_cast<const int *>(aux);
     const real *inv = reinterpret_cast<const real *>(aux + B.B);
     const long long per = CT * (16 / (int)sizeof(real));
-    ::mof::count_launch(), k_of_combine<real><<<dim3((unsigned)((B.N + per - 1) / per), B.B), CT, 0, st>>>(B.V, B.N, B.Kmax, B.K, z, slot,
-                                                                                                      inv, out);
+    const dim3 grid((unsigned)((B.N + per - 1) / per), B.B);
+    ::mof::count_launch();
+    if (reinterpret_cast<uintptr_t>(out) % 16 == 0) k_of_combine<real, true><<<grid, CT, 0, st>>>(B.V, B.N, B.Kmax, B.K, z, slot, inv, out);
+    else k_of_combine<real, false><<<grid, CT, 0, st>>>(B.V, B.N, B.Kmax, B.K, z, slot, inv, out);
     MOF_LAUNCH_CHECK();
     return MOF_OK;
 }
