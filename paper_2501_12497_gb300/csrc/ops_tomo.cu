@@ -441,7 +441,7 @@ constexpr int BP_TX = 32, BP_TY = 8, BP_CHUNK = 64;
 // For footprints of at most RT (1, 2) bins each side and coordinates within FIX64_LIMIT: those of the
 // tile's pixels in fixed point about its origin, the tent weights 1 - (fr + m) / r and
 // 1 - (1 + m - fr) / r by the reciprocal of r, taken as zero (with their bins, whatever they hold)
-// where negative. Six (RT = 1) or ten FP64 instructions a pixel and view, which bound it, against 35
+// where not positive. Six (RT = 1) or ten FP64 instructions a pixel and view, which bound it, against 35
 // with divisions. 64 x 64 x 8, 16 views: 19 us against 50; 256 x 256 x 8, 30 views: 183 against 1045 us.
 struct Bt64 {
     long long t, a, b;  // coordinate of the tile's first pixel, its steps in x and y in units of 2^-55
@@ -483,7 +483,8 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject64_fix(const double
 #pragma unroll
             for (int m = 0; m < RT; ++m) {
                 const int k0 = ib - m, k1 = ib + 1 + m;
-                const bool p0 = __double2hiint(w0) >= 0, p1 = __double2hiint(w1) >= 0;
+                // (integer comparisons; a weight of zero is common: a whole coordinate where r is whole)
+                const bool p0 = __double_as_longlong(w0) > 0, p1 = __double_as_longlong(w1) > 0;
                 const double v0 = p0 && (unsigned)k0 < (unsigned)nb ? ldg(row + k0) : 0.0;
                 const double v1 = p1 && (unsigned)k1 < (unsigned)nb ? ldg(row + k1) : 0.0;
                 s = m ? fma(p0 ? w0 : 0.0, v0, s) : (p0 ? w0 : 0.0) * v0;
