@@ -1083,13 +1083,11 @@ __device__ bool be_update(const double *GA, const double *GL, const double *g, i
                 S2 += part[ST + q * RS + tid];
             }
             const double r = (Do - gam) + m - S1, z = Z2[o], h = m * r - z, hp = r + m + m * S2;
-            double x = m - h / hp;
-            // the root stays on its side of the pole and short of the next one
+            const double x = m - h / hp;
+            // the root stays on its side of the pole and short of the next one: a step that leads away from
+            // there started on the wrong side of the root (an FP32 search among terms that cancel)
             const double lim = root == 0 || root == p ? 1e30 : 0.75 * (D[root] - D[root - 1]);
-            if (!(x * m > 0.0 && fabs(x) < lim)) {
-                x = m;
-                if (it > 2) sh.bad = 1;
-            }
+            if (!(x * m > 0.0 && fabs(x) < lim)) sh.bad = 1;  // (the step from m is the same in every round)
             const double dx = fabs(x - m);
             mu[tid] = x;
             more = dx > 1e-9 * fabs(x);  // quadratic: the next step would be at the rounding level
