@@ -598,19 +598,21 @@ __device__ __forceinline__ unsigned mag_bits(float v) { return __float_as_uint(v
 __device__ __forceinline__ unsigned long long mag_bits(double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
 }
-// sums of a pixel's own terms: FP32 with the additions' rounding errors, FP64 in fixed point later
+// sums of a pixel's own terms: FP32 with the additions' rounding errors, FP64 in fixed point later.
+// FP32: of eighths, as up to eight terms may sum to more than FLT_MAX where the scattered ones bring
+// the result back (exact; an eighth of a subnormal number keeps more than the fixed point's 2^-126).
 template <typename real> struct OwnSum;
 template <> struct OwnSum<float> {
     DFAcc a;
-    __device__ __forceinline__ void add(float v) { a.add(v); }
+    __device__ __forceinline__ void add(float v) { a.add(v * 0.125f); }
     __device__ __forceinline__ void fixed(float sc, int &h, int &l) const {
         int h1, l1;
-        fx_split(a.hi * sc, h, l);
-        fx_split(a.lo * sc, h1, l1);
+        fx_split(a.hi * sc * 8.0f, h, l);
+        fx_split(a.lo * sc * 8.0f, h1, l1);
         h += h1;
         l += l1;
     }
-    __device__ __forceinline__ long long fixed(float sc) const { return fx_term(a.hi * sc) + fx_term(a.lo * sc); }
+    __device__ __forceinline__ long long fixed(float sc) const { return fx_term(a.hi * sc * 8.0f) + fx_term(a.lo * sc * 8.0f); }
 };
 template <> struct OwnSum<double> {
     double v[8];

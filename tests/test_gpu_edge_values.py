@@ -42,3 +42,26 @@ def test_fp64_transpose_takes_no_bin_of_weight_zero(nb, db, bad):
     assert torch.equal(~torch.isfinite(out), foot > 0)
     if bad == float("inf"):
         assert not torch.isnan(out).any()
+
+
+# A pixel's own terms may sum to more than FLT_MAX and be brought back by the scattered ones. The sums are
+# taken in fixed point relative to the tile's largest term, so data scaled by a power of two give the
+# same result scaled, bit for bit. Displacements within a few pixels (32-bit sums) and of up to 20 (64-bit).
+@pytest.mark.parametrize("reach", [0.0, 2.0, 20.0])
+def test_fp32_warp_transposes_near_the_largest_numbers(reach):
+    p = api.mof_problem_create(70, 45, 4, 8, [1] * 4, np.zeros(4), 1.0, 1.0, api.MOF_FP32)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    rand = lambda n, a: (torch.rand(n, device="cuda", generator=g) * 2 - 1) * a
+    s, sr = rand(p.nv, reach), rand(p.nv, reach)
+    down, up = 2.0 ** -8, 2.0 ** 8
+    f32 = torch.float32
+
+    r = rand(p.nv, 3.4e38)
+    got, want = (_out(lambda q, v, o: api.mof_apply_flowT(q, v, s, sr, o), p, p.n, f32, v) for v in (r, r * down))
+    assert torch.isfinite(got).float().mean() > 0.5
+    assert torch.equal(got, want * up)
+
+    x, uk = rand(p.n, 8e37), torch.zeros(p.n, device="cuda")
+    got, want = (_out(lambda q, v, o: api.mof_apply_reg_normal(q, v, uk, s, sr, 1.0, o), p, p.n, f32, v) for v in (x, x * down))
+    assert torch.isfinite(got).float().mean() > 0.5
+    assert torch.equal(got, want * up)
