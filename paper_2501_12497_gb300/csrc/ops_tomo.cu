@@ -84,7 +84,10 @@ struct ProjSplit {
 // The sum of one ray's taps, as the compensated pair (sum, correction to subtract). img: the
 // frame in the march's orientation; F, D: f0 and df in 2^-40 pixels, |f0| < 2^22 pixels,
 // |df| <= 1; off lanes (on = false) take part in the warp's votes only; segment seg of nseg of
-// the warp's steps. All lanes call.
+// the warp's steps. All lanes call. INF: a sum that is not finite is that of plain additions, so that
+// an infinity stays one (its correction would be NaN).
+constexpr float FLT_LARGEST = 3.402823466e+38f;
+template <bool INF>
 __device__ __forceinline__ float2 ray_march(const float *__restrict__ img, int nfast, int nstep, long long F, long long D,
                                             bool on, int seg, int nseg) {
     const unsigned lanes = __ballot_sync(0xffffffffu, on);
@@ -118,7 +121,7 @@ __device__ __forceinline__ float2 ray_march(const float *__restrict__ img, int n
         jhi = min(jhi, jlo + b1 * MARCH - 1);
         jlo += b0 * MARCH;
     }
-    float acc = 0.f, cmp = 0.f;
+    float acc = 0.f, cmp = 0.f, raw = 0.f;
     const unsigned last = (unsigned)(nfast - 1);
     const float df = (float)D * 9.094947017729282e-13f;
     F += (jlo + MARCH / 2) * D;  // the crossing at the middle of the block
@@ -160,11 +163,13 @@ __device__ __forceinline__ float2 ray_march(const float *__restrict__ img, int n
         float s, so;
         unpack2(s2, s, so);
         s += so;
+        if (INF) raw += s;
         F += MARCH * D;
         const float y = __fsub_rn(s, cmp), t = __fadd_rn(acc, y);
         cmp = __fsub_rn(__fsub_rn(t, acc), y);
         acc = t;
     }
+    if (INF && !(fabsf(acc) <= FLT_LARGEST)) return make_float2(raw, 0.f);
     return make_float2(acc, cmp);
 }
 
@@ -180,7 +185,7 @@ __device__ __forceinline__ bool join_segments(float2 &r, const ProjSplit &sp) {
     for (int g = 1; g < sp.segs; ++g) {
         const float2 o = part[threadIdx.x + g * per * 32];
         const float y = __fsub_rn(o.x, __fadd_rn(r.y, o.y)), t = __fadd_rn(r.x, y);
-        r.y = __fsub_rn(__fsub_rn(t, r.x), y);
+        r.y = fabsf(t) <= FLT_LARGEST ? __fsub_rn(__fsub_rn(t, r.x), y) : 0.f;
         r.x = t;
     }
     return true;
@@ -211,7 +216,7 @@ __global__ void __launch_bounds__(32 * PW) k_project32(const float *__restrict__
     const long long ns = (long long)nx * ny;
     const int rows = P.rows;
     const bool on = a < nang && k < nb;
-    float2 r = ray_march((rows ? u : uT) + P.frame * ns, rows ? nx : ny, rows ? ny : nx, F, P.dfQ, on, seg, sp.segs);
+    float2 r = ray_march<false>((rows ? u : uT) + P.frame * ns, rows ? nx : ny, rows ? ny : nx, F, P.dfQ, on, seg, sp.segs);
     if (join_segments(r, sp) && on) b[(long long)a * nb + k] = scale_sum(r, P.wstep, P.wstep_lo);
 }
 
@@ -336,8 +341,8 @@ __global__ void __launch_bounds__(32 * PW) k_project_fan32(const float *__restri
     const FanRay<float> R = rays[(long long)ac * nb + min(k, nb - 1)];
     const int rows = (int)(R.f0q & 1);
     const long long F = R.f0q >> 1, D = R.dq, fr = ang[ac].frame * ns;
-    float2 r = ray_march(u + fr, nx, ny, F, D, on && rows, seg, sp.segs);
-    const float2 rc = ray_march(uT + fr, ny, nx, F, D, on && !rows, seg, sp.segs);
+    float2 r = ray_march<true>(u + fr, nx, ny, F, D, on && rows, seg, sp.segs);
+    const float2 rc = ray_march<true>(uT + fr, ny, nx, F, D, on && !rows, seg, sp.segs);
     if (!rows) r = rc;
     if (!join_segments(r, sp) || !on) return;
     // length per step h sqrt(1 + df^2), its rounding kept: r = sqrt(x) + e, e = (x - s^2) / (2 s)
@@ -657,7 +662,7 @@ __global__ void __launch_bounds__(BT_X *BT_Y) k_backproject_tile(const float *__
             for (int i = 0; i < W; i += 32) {
                 const int k = kk.x + i + lane;
                 const float v = (k >= 0 && k <= kk.y) ? ldg(row + k) * wf : 0.f;
-                finite = finite && fabsf(v) <= 3.402823466e+38f;
+                finite = finite && fabsf(v) <= FLT_LARGEST;
                 s_seg[q][i + lane] = v;
             }
         }
@@ -783,7 +788,9 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject4(const float *__re
 // 32-bit integers modulo 64 pixels (the host admits only geometries where a visited ray is
 // closer than 32). Every pixel of a tile and view visits the same number of rays, the most that
 // its bound allows. The sum over the views is compensated (Kahan).
-// A segment with a non-finite datum takes the weights that are zero out of the sum (careful).
+// From a stage with a datum that is not finite (or so large that a sum of 1e8 may not be) on, the weights
+// that are zero are taken out of the sum, and an infinite sum has no correction, so that it stays one
+// (careful).
 // What bounds it: instruction issue (80 %), about nine instructions per pixel, view and visited
 // ray (2 to 3 rays; 2.8 on average hold the pixel). fan 256x256x32, 30 views:
 // 133 us (error 3.2e-8) against 386 (1.1e-7) for one thread per pixel with four divisions per view
@@ -839,12 +846,12 @@ __device__ __forceinline__ void ft_view(const FtView &V, float h, float scale, f
 #pragma unroll
     for (int e = 0; e < FT_E; ++e) {
         const float yv = __fsub_rn(tap[e], cmp[e]), tt = __fadd_rn(acc[e], yv);
-        cmp[e] = __fsub_rn(__fsub_rn(tt, acc[e]), yv);
+        cmp[e] = !CAREFUL || fabsf(tt) <= FLT_LARGEST ? __fsub_rn(__fsub_rn(tt, acc[e]), yv) : 0.f;
         acc[e] = tt;
     }
 }
 
-__global__ void __launch_bounds__(FT_X *FT_Y) k_backproject_fan_tile(const float *__restrict__ b, float *__restrict__ u,
+__global__ void __launch_bounds__(FT_X *FT_Y, 8) k_backproject_fan_tile(const float *__restrict__ b, float *__restrict__ u,
                                                                      const FanRay<float> *__restrict__ rays,
                                                                      const FanView *__restrict__ views,
                                                                      const int *__restrict__ aoff, int nx, int ny, int nb,
@@ -861,6 +868,7 @@ __global__ void __launch_bounds__(FT_X *FT_Y) k_backproject_fan_tile(const float
 #pragma unroll
     for (int e = 0; e < FT_E; ++e) acc[e] = cmp[e] = 0.f;
     const int a_end = aoff[t + 1];
+    bool careful = false;
     for (int ac = aoff[t]; ac < a_end; ac += FT_CH) {
         const int cn = min(FT_CH, a_end - ac);
         __syncthreads();
@@ -904,7 +912,7 @@ __global__ void __launch_bounds__(FT_X *FT_Y) k_backproject_fan_tile(const float
                     any_r |= rows;
                     any_c |= !rows;
                 }
-                finite = finite && fabsf(v) <= 3.402823466e+38f;
+                finite = finite && fabsf(v) <= 1e30f;
                 s_seg[q][0][i] = __int_as_float(cr);
                 s_seg[q][1][i] = __int_as_float(st);
                 s_seg[q][2][i] = v;
@@ -913,7 +921,7 @@ __global__ void __launch_bounds__(FT_X *FT_Y) k_backproject_fan_tile(const float
             any_c = __any_sync(0xffffffffu, any_c);
             if (lane == 0) s_v[q].steps = any_r && any_c ? 2 : (any_c ? 0 : 1);
         }
-        const bool careful = !__syncthreads_and(finite);
+        careful |= !__syncthreads_and(finite);
         const int x = min(x0 + lane, x1), y = y0 + w * FT_E, dx = lane - FT_X / 2, dy = w * FT_E - FT_Y * FT_E / 2;
         for (int q = 0; q < cn; ++q) {
             const int steps = s_v[q].steps;

@@ -65,3 +65,21 @@ def test_fp32_warp_transposes_near_the_largest_numbers(reach):
     got, want = (_out(lambda q, v, o: api.mof_apply_reg_normal(q, v, uk, s, sr, 1.0, o), p, p.n, f32, v) for v in (x, x * down))
     assert torch.isfinite(got).float().mean() > 0.5
     assert torch.equal(got, want * up)
+
+
+# Infinities and overflow in the FP32 fan pair come out as infinities, as a plain sum has them. The views
+# fill one stage of the transpose and several; the rays are marched in segments and whole.
+@pytest.mark.parametrize("na,nb", [(9, 90), (40, 90), (800, 400)])
+def test_fp32_fan_pair_keeps_infinities(na, nb):
+    f32 = torch.float32
+    p = api.mof_problem_create(64, 48, 2, nb, [na] * 2, 0.1234 + np.linspace(0, 3, 2 * na), 1.0, 1.6 * 90 / nb, api.MOF_FP32,
+                               fan=(140.0, 70.0))
+    g = torch.Generator(device="cuda").manual_seed(4)
+    for fn, nin, nout, at in ((api.mof_apply_A, p.n, p.m, 64 * 20 + 30), (api.mof_apply_AT, p.m, p.n, 2 * nb + nb // 2)):
+        x, e = torch.randn(nin, device="cuda", generator=g), torch.zeros(nin, device="cuda")
+        x[at], e[at] = float("inf"), 1.0
+        out, foot = (_out(fn, p, nout, f32, v) for v in (x, e))
+        assert (foot > 0).any()
+        assert torch.equal(torch.isinf(out), foot > 0) and not torch.isnan(out).any()
+        out = _out(fn, p, nout, f32, torch.full((nin,), 3e38, device="cuda"))
+        assert torch.isinf(out).any() and not torch.isnan(out).any()
