@@ -1373,12 +1373,17 @@ mof_status launch_of_fields(const mof_problem *p, const real *u, int dr, real *u
         // (256x256x32: 17 us with 4 rows, 33 with 16; 181x149x9: 9 and 19)
         int rows = 16;
         while (rows > 2 && (long long)gx * np * ((p->ny + rows - 1) / rows) < 152LL * 16) rows = rows == 16 ? 4 : 2;
-        const dim3 grid(gx, (p->ny + FW * rows - 1) / (FW * rows), np), tb(32, FW);
-        ::mof::count_launch();
-        if (vec)
-            k_of_fields_rows<float, 4><<<grid, tb, 0, st>>>((const float *)u, (float *)ux, (float *)uy, (float *)ut, p->nx, p->ny, rows);
-        else
-            k_of_fields_rows<real, 1><<<grid, tb, 0, st>>>(u, ux, uy, ut, p->nx, p->ny, rows);
+        const dim3 tb(32, FW);
+        for (int p0 = 0; p0 < np; p0 += 65535) {  // the pairs are the grid's z, which holds that many
+            const dim3 grid(gx, (p->ny + FW * rows - 1) / (FW * rows), std::min(np - p0, 65535));
+            const long long o = p0 * p->ns;
+            ::mof::count_launch();
+            if (vec)
+                k_of_fields_rows<float, 4><<<grid, tb, 0, st>>>((const float *)u + o, (float *)ux + o, (float *)uy + o, (float *)ut + o,
+                                                                p->nx, p->ny, rows);
+            else
+                k_of_fields_rows<real, 1><<<grid, tb, 0, st>>>(u + o, ux + o, uy + o, ut + o, p->nx, p->ny, rows);
+        }
     }
     else if (dr == 2)
         ::mof::count_launch(), k_of_fields_tiled<real, 2><<<dim3((p->nx + TX - 1) / TX, (p->ny + TY - 1) / TY), dim3(TX, TY), 0, st>>>(

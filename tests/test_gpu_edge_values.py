@@ -83,3 +83,24 @@ def test_fp32_fan_pair_keeps_infinities(na, nb):
         assert torch.equal(torch.isinf(out), foot > 0) and not torch.isnan(out).any()
         out = _out(fn, p, nout, f32, torch.full((nin,), 3e38, device="cuda"))
         assert torch.isinf(out).any() and not torch.isnan(out).any()
+
+
+# More frame pairs than one launch dimension holds: each pair's fields are those of the same frames in
+# a short sequence. 4 columns: vectors of a row; 3: single pixels.
+@pytest.mark.parametrize("nx", [4, 3])
+@pytest.mark.parametrize("prec", [api.MOF_FP32, api.MOF_FP64])
+def test_velocity_fields_of_very_many_frames(prec, nx):
+    dt = torch.float64 if prec == api.MOF_FP64 else torch.float32
+    ny, nt, few = 3, 65536 + 40, 9
+    create = lambda t: api.mof_problem_create(nx, ny, t, 1, [1] * t, np.zeros(t), 1.0, 1.0, prec)
+    p, q = create(nt), create(few)
+    ns = nx * ny
+    u = torch.randn(nt * ns, device="cuda", dtype=dt, generator=torch.Generator(device="cuda").manual_seed(5))
+    fields = [torch.full(((nt - 1) * ns,), float("nan"), device="cuda", dtype=dt) for _ in range(3)]
+    api.mof_of_fields(p, u, 1, *fields)
+    assert all(torch.isfinite(f).all() for f in fields)
+    for t0 in (0, 65530, 65535, nt - few):
+        part = [torch.empty((few - 1) * ns, device="cuda", dtype=dt) for _ in range(3)]
+        api.mof_of_fields(q, u[t0 * ns:(t0 + few) * ns].clone(), 1, *part)
+        for f, want in zip(fields, part):
+            assert torch.equal(f[t0 * ns:(t0 + few - 1) * ns], want)
