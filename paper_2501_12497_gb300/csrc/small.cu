@@ -1618,6 +1618,8 @@ mof_status prepare_small_solve(int ld) {
 }
 
 mof_status launch_small_solve(const SmallArgs &a, cudaStream_t st) {
+    // (DP and fixed lambda leave the eigenvectors unformed)
+    if (a.Y && a.rule != MOF_RULE_GCV) return fail(MOF_EINVAL, "the small solve keeps eigenvectors between calls for GCV only");
     static const GcvGrid grid = [] {
         GcvGrid g;
         for (int i = 0; i < GRID_POINTS; ++i) g.v[i] = std::pow(10.0, -BRACKET_DECADES + i * (2.0 * BRACKET_DECADES / (GRID_POINTS - 1)));

@@ -178,7 +178,7 @@ struct SmallArgs {
     double *proj;          // [B][ld] out
     // State between the calls of one basis that grows by at most a vector per call while its Grams
     // stay as they are (null: none): generalised eigenvectors Y [B][ld][ld], their eigenvalues Yd,
-    // Yh = Y^T g, the scaling Yrho and their number nY (zero before the first call).
+    // Yh = Y^T g, the scaling Yrho and their number nY (zero before the first call). GCV only.
     double *Y, *Yd, *Yh, *Yrho;
     int *nY;
 };

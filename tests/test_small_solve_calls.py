@@ -72,3 +72,12 @@ def test_every_root_of_the_bordered_problem_is_found(lib):
     Yt = Y.transpose(0, 2, 1)
     assert np.abs(Yt @ M @ Y - np.eye(n)).max() <= 1e-10
     assert np.abs(Yt @ GA @ Y - Yd[:, :, None] * np.eye(n)).max() <= 1e-10
+
+
+# The state of a growing basis (Y) goes with the GCV rule only: the other rules leave parts of it unset.
+@pytest.mark.parametrize("rule", [api.MOF_RULE_DP, api.MOF_RULE_FIXED])
+def test_the_state_of_a_growing_basis_is_refused_with_other_rules(lib, rule):
+    buf = (ctypes.c_double * 64)()
+    at = ctypes.addressof(buf)
+    args = SmallArgs(ld=4, B=0, rule=rule, Y=at)  # no problem: nothing could run
+    assert _launch(lib, args) == api.MOF_EINVAL
