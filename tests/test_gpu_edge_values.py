@@ -104,3 +104,21 @@ def test_velocity_fields_of_very_many_frames(prec, nx):
         api.mof_of_fields(q, u[t0 * ns:(t0 + few) * ns].clone(), 1, *part)
         for f, want in zip(fields, part):
             assert torch.equal(f[t0 * ns:(t0 + few - 1) * ns], want)
+
+
+# The last of 65 bins (by itself in its warp) looks along the frame's last column (row) from 2e-5 pixels
+# inside, parallel to it and turned by up to 1e-6 rad, over a frame that is one in its outer columns (rows)
+# only. A step's coordinate is exact to 2^-22 pixels and a ray takes 1024 of them; 1.5 times that is allowed.
+def test_fp32_rays_along_the_edge_of_the_frame():
+    n, nb, db, turns = 1024, 65, 512.49998 / 32, [0.0, 1e-6, -1e-6, 3e-7, -3e-7, 1e-7]
+    ang = np.array(turns + [np.pi / 2 + a for a in turns])
+    na = [len(turns)] * 2
+    p = api.mof_problem_create(n, n, 2, nb, na, ang, 1.0, db, api.MOF_FP32)
+    u = np.zeros((2, n, n))
+    u[0, :, [0, -1]] = 1.0
+    u[1, [0, -1], :] = 1.0
+    want = O.project(O.Geometry(n, n, 2, nb, na, ang, 1.0, db), u).ravel()
+    got = _out(api.mof_apply_A, p, p.m, torch.float32, torch.tensor(u.ravel(), device="cuda", dtype=torch.float32))
+    assert (want.reshape(-1, nb)[:, -1] > 0.02).all()
+    err = np.abs(got.cpu().numpy() - want).max()
+    assert err <= 1.5 * n * 2.0 ** -22, err
