@@ -520,7 +520,8 @@ __global__ void __launch_bounds__(32) k_of_proj_gram_pass(const real *V, long lo
             else zero.h[0] = zero.h[1] = 0.0;
             for (int i = 0; i < 2 * Kb + 8; ++i) const_cast<Q *>(seg)[i * 32] = zero;
         }
-        if (!mbar_wait(bar_a, phase, g_wait_polls)) {
+        // (the warp leaves as one: a lane that went on would wait for a tile that not all lanes fetch)
+        if (!__all_sync(0xffffffffu, mbar_wait(bar_a, phase, g_wait_polls))) {
             if (lane == 0 && err) atomicOr(err, 4);
             mbar_wait(bar_a, phase);  // do not leave while copies may still land
             return;
