@@ -13,9 +13,10 @@
 // neighbouring source tiles whose footprints can fall into it (the only global
 // atomics: one integer maximum per source tile for the field's reach). Mhat^T and
 // Theta^T W Theta scatter the sources' weighted values into
-// the tile in exact 64-bit fixed point (order independent, so repeated runs are
-// bit-identical); the reverse flow averages the arrivals of each pixel in row-major
-// source order.
+// the tile in exact fixed point (order independent, so repeated runs are bit-identical;
+// FP32: two 32-bit integers per sum, 64-bit ones where the displacements vary widely, and
+// in FP64); the reverse flow enters them into per-pixel lists and averages the arrivals of
+// each pixel in row-major source order.
 #include "common.cuh"
 
 #include <algorithm>

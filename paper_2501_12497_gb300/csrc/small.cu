@@ -135,7 +135,7 @@ __device__ __forceinline__ void warp_sum6(double s[6]) {
 }
 
 // 1 / x from the FP32 reciprocal by two Newton steps, |x| within the normal FP32 range
-__device__ __forceinline__ double rcp_newton(double x) {  // 1 / x, |x| within the normal FP32 range
+__device__ __forceinline__ double rcp_newton(double x) {
     double r = (double)__frcp_rn((float)x);
     r = fma(r, fma(-x, r, 1.0), r);
     return fma(r, fma(-x, r, 1.0), r);

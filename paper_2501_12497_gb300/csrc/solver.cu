@@ -482,11 +482,6 @@ template <typename real>
 __global__ void k_copy(const real *__restrict__ a, real *__restrict__ b, long long n) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) b[i] = a[i];
 }
-template <typename real>
-__global__ void k_neg(const real *__restrict__ a, real *__restrict__ b, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) b[i] = -a[i];
-}
-// x[b] -= coef[b] * y[b]  (coef device, per problem)
 // err |= 16 when the data's squared norm is not finite (a NaN or an infinity in b)
 __global__ void k_flag_nonfinite(const double *__restrict__ v, int *__restrict__ err) {
     if (threadIdx.x == 0 && !isfinite(v[0])) atomicOr(err, 16);
@@ -1149,8 +1144,10 @@ constexpr int TG_S = TG_ROWS + 4;  // column stride of the shared row tile
 // four columns puts the 128-bit reads of the eight column groups a warp's 4x4
 // blocks touch on eight different bank quads
 __host__ __device__ constexpr int tg_col(int j) { return j * TG_S + 4 * (j / 4); }
-// Row groups per 4x4 block at most: 16 busy 96 threads at K = 10 (1024x1024x64: 24.9 ms for the four Grams
-// of two iterations; 8: 27.7, 32: 25.2, 64: 25.6, where the compensated sums of more groups cost more)
+// Row groups per 4x4 block at most: 16 busy 96 threads at K = 10 (1024x1024x64, K = 10 and 11: 24.9 ms for the
+// four Grams of two iterations; 8: 27.7, 32: 25.2, 64: 25.6, where the compensated sums of more groups cost
+// more). It bounds small bases only: from K = 25 on the threads allow at most 9 groups, at K = 39 four, and
+// the Grams of a 30-iteration solve take 25 ms an iteration with it as without.
 constexpr int TG_MAXG = 16;
 constexpr int TG_VEC = 8;          // basis vectors per step of the difference rows (16 loads in flight)
 

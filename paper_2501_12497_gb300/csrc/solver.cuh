@@ -96,17 +96,15 @@ struct Krylov {
     void gk_half_step(const BasisRef<real> &B, int *Kmut, int front, const GkFront<real> &f, double *coef, double *nrm2_out,
                       const double *scale, double tol, int *grow, double *sq1, double *sq2, int *done, bool scaled,
                       cudaStream_t st) const;
-    // x[b] <- (I - V V^T)^2 x[b] (classical Gram-Schmidt twice); ||x||^2 -> nrm2_out
-    void reorth(const BasisRef<real> &B, real *x, long long xstride, double *coef, double *nrm2_out, cudaStream_t st) const;
-    // the same with the first projection's coefficients V^T x supplied by the caller from an
-    // exact identity (c1 [B][Kmax]; null when they are zero, as for a Golub-Kahan residual),
-    // so that only the second projection streams V for its dot products
-    // kcap (> 0): a bound on every K[b] known to the caller, which sizes the fused pass's
-    // shared-memory tile (a larger K[b] sets bit 8 of err)
+    // x[b] <- (I - V V^T)^2 x[b] (classical Gram-Schmidt twice; coef [B][Kmax] scratch), ||x||^2 -> nrm2_out,
+    // with the first projection's coefficients V^T x supplied by the caller from an exact identity
+    // (c1 [B][Kmax]), so that only the second projection streams V for its dot products
     void reorth_second(const BasisRef<real> &B, real *x, long long xstride, const double *c1, double *coef,
-                       double *nrm2_out, cudaStream_t st, int kcap = 0) const;
+                       double *nrm2_out, cudaStream_t st) const;
     // x[b] <- x[b] - V[b] c[b] and out[b] = V[b]^T x[b] in one pass over V (false: not
     // applicable to this layout, nothing enqueued)
+    // kcap (> 0): a bound on every K[b] known to the caller, which sizes the pass's shared-memory
+    // tile (a larger K[b] sets bit 8 of err)
     // nparts (may be null): also the chunk partials of ||x'[b]||^2, after the dot partials in
     // partial (at partial + B.B * nparts * Kmax), their number per problem in *nparts
     bool sub_dot(const BasisRef<real> &B, const double *c, long long cstride, real *x, long long xstride, double *out,
