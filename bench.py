@@ -383,9 +383,9 @@ def fused_bytes(name, w, of_scale=1, tau=1):
 
 # DRAM bytes over algorithmic bytes per launch of the kernel that dominates a class, from an
 # ncu capture of that kernel (k_of_proj_gram_pass: 31 pairs of 256x256 frames at K = 20 and
-# 21, 408.9 MB for 406.3 MB and 425.1 MB for 422.6 MB); the class's traffic per launch is
+# 21, 407.6 MB for 406.3 MB and 424.0 MB for 422.6 MB); the class's traffic per launch is
 # estimated as this ratio times the class's algorithmic bytes per launch
-TRAFFIC_RATIO = {"of_subdot": 1.006}
+TRAFFIC_RATIO = {"of_subdot": 1.003}
 
 # the main kernel of each timing class
 CLASS_KERNEL = {
