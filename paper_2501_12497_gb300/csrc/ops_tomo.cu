@@ -496,8 +496,9 @@ __global__ void __launch_bounds__(BP_TX *BP_TY) k_backproject64_fix(const double
 #pragma unroll
             for (int m = 0; m < RT; ++m) {
                 const int k0 = ib - m, k1 = ib + 1 + m;
-                // (integer comparisons; a weight of zero is common: a whole coordinate where r is whole)
-                const bool p0 = __double_as_longlong(w0) > 0, p1 = __double_as_longlong(w1) > 0;
+                // (a weight of zero is common: a whole coordinate where r is whole. Positive by the upper half's bits:
+                // one comparison, and no weight but zero has them all clear, as fr and 1 / r are multiples of 2^-53)
+                const bool p0 = __double2hiint(w0) > 0, p1 = __double2hiint(w1) > 0;
                 const double v0 = p0 && (unsigned)k0 < (unsigned)nb ? ldg(row + k0) : 0.0;
                 const double v1 = p1 && (unsigned)k1 < (unsigned)nb ? ldg(row + k1) : 0.0;
                 s = m ? fma(p0 ? w0 : 0.0, v0, s) : (p0 ? w0 : 0.0) * v0;
