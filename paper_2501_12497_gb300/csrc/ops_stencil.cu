@@ -1220,9 +1220,10 @@ __global__ void k_of_fields(const real *__restrict__ u, int dr, real *__restrict
 // (as frame p and as frame p + 1 of pair p - 1, the second time from L2) plus two halo rows per strip.
 // All sums take their terms in the order of k_of_fields (identical results: Solve-OF amplifies the
 // rounding of its fields a hundredfold). V = 4 needs rows of a multiple of 4 pixels and 16-byte aligned arrays.
-// What bounds it: DRAM (62 % of the copy rate with the first pass over u in the count). 1024x1024x64:
-// 250 us against 461 for shared-memory tiles that walk the frames in order; 256x256x32: 17 against
-// 52 us; 181x149x9: 9 against 17 us.
+// What bounds it: DRAM on data without equal neighbours (1024x1024x64: 221 us, 0.70 of the copy rate); a
+// difference of exactly zero takes the division's slow path, so frames with flat parts are bound by
+// instructions (phantoms 357 us, constant frames 416). 461 us on phantoms for shared-memory tiles that walk the
+// frames in order; 256x256x32: 12 to 21 us against 52; 181x149x9: 9 against 17 us.
 constexpr int FW = 4;  // warps per CTA
 template <typename real, int V>
 __global__ void __launch_bounds__(32 * FW) k_of_fields_rows(const real *__restrict__ u, real *__restrict__ ux,

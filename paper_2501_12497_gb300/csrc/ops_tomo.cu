@@ -74,7 +74,7 @@ __global__ void k_transpose(const real *__restrict__ u, real *__restrict__ uT, i
 // FP32 however long it is.
 // What bounds it: the two 4-byte loads a step, each of which touches two to three 128-byte
 // lines of L1 (32 adjacent rays cross 32 to 46 pixels of a row; 65 % of the L1 data pipe), and
-// instruction issue (63 %, 13 instructions a step). 1024x1024x64, 90 views: 2.99 ms against 7.21
+// instruction issue (63 %, 13 instructions a step). 1024x1024x64, 90 views: 3.02 ms against 7.21
 // for the march with a conversion pair per coordinate and per-ray step ranges, whose lanes read
 // different rows; 256x256x32, 30 views: 62 against 130 us. Fan beam 256x256x32: 68 against 119 us.
 // Few rays leave the chip idle and the march's load latency exposed, so the warps of a CTA
